@@ -181,12 +181,13 @@ bh_status bh_sync_status(bh_ctx *ctx);
 
 /* Times the binary32 per-cell walk of the current tree at this theta for
  * every launch shape it offers -- CTAs of 2, 4, 8 and 16 warps; warps that
- * walk for 64 targets (a 4x4x4 octant of a block, one pair of x-neighbours
- * per lane) or 128 targets (a 8x4x4 slab, two pairs per lane); either a
+ * walk for 64 targets (a 4x4x4 octant of a block; "one pair per lane") or 128
+ * targets (two x-neighbouring octants, one after the other; "two pairs");
+ * either a
  * plain grid of one warp per group or a persistent grid (as many CTAs as the
  * GPU holds at once) whose warps take 1, 2 or 4 groups at a time from a work
  * counter; and the groups in their own (Morton) order or longest walk first
- * (the periodic walk: CTA width and order, one pair per lane, plain grid) --
+ * (the periodic walk: CTA width and order, one octant, plain grid) --
  * each twice, then the four fastest five times more -- and keeps the fastest
  * for later walks.  For the longest-first order it first walks the tree once
  * at this theta (the persistent grid; the periodic walk on its plain grid),
@@ -202,8 +203,8 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape);
 
 /* Sets the launch shape of the binary32 per-cell walk (the four values
  * bh_autotune chooses among), e.g. one found by an earlier bh_autotune on
- * the same kind of mesh: warps per CTA (1..16), target pairs per lane (1 or
- * 2), groups per take of the persistent grid (0 = plain grid, 1..64) and
+ * the same kind of mesh: warps per CTA (1..16), octants per group (1 or 2,
+ * named target pairs per lane), groups per take of the persistent grid (0 = plain grid, 1..64) and
  * longest_first (1: the walk order made by the last bh_autotune, 0: the
  * groups' own order); 0 for the first two means the default.  Potentials do
  * not depend on the shape (bit for bit).  Drops a captured bh_solve_graph
@@ -277,7 +278,7 @@ bh_status bh_solve_host(bh_ctx *ctx, int nblocks, const int32_t *level, const in
  * Kahan sum) + bh_build + bh_potential compute, on the CURRENT device and on
  * `cuda_stream` (a cudaStream_t, NULL = legacy default stream), without any
  * context and without allocating: the tree lives in one fixed array in device
- * global memory (about 2.7 MB, held by every GPU that loads this library until
+ * global memory (about 3.0 MB, held by every GPU that loads this library until
  * the process exits).
  *   nblocks        1 .. 64 blocks (at most 32,768 cells); more -> BH_ERR_ARG
  *   level, ijk, box_lo, box_len, density, density_is_fp64: as bh_build

@@ -95,6 +95,10 @@ void free_nodes(bhg::Tree &t) {
   release(t.d_aux);
   release(t.d_lvl);
   t.node_cap = 0;
+  release(t.d_sib);
+  release(t.d_squad);
+  release(t.d_cmass);
+  t.sib_cap = 0;
   release(t.d_q64);
   release(t.d_qrec);
   t.quad_cap = 0;
@@ -121,11 +125,13 @@ bh_status ensure_blocks(bh_ctx *ctx, int nb) {
   return BH_OK;
 }
 
-bh_status ensure_nodes(bh_ctx *ctx, int64_t n_nodes) {
+bh_status ensure_nodes(bh_ctx *ctx, int64_t n_nodes, int64_t nb) {
   bhg::Tree &t = ctx->tree;
   const bool quad = ctx->opt.quadrupole != 0 || ctx->opt.learned != 0;
   const bool quad64 = ctx->opt.quadrupole && ctx->opt.precision == BH_PREC_F64;
-  if (t.node_cap >= n_nodes && (!quad || t.quad_cap >= n_nodes)) return BH_OK;
+  const int64_t entries = bhg::sib_entries(nb);
+  if (t.node_cap >= n_nodes && t.sib_cap >= entries && (!quad || t.quad_cap >= n_nodes))
+    return BH_OK;
   free_nodes(t);
   if (quad) {
     if (quad64) BH_CUDA(bhg::dev_malloc(&t.d_q64, (size_t)n_nodes * 6 * sizeof(double)));
@@ -138,6 +144,11 @@ bh_status ensure_nodes(bh_ctx *ctx, int64_t n_nodes) {
   BH_CUDA(bhg::dev_malloc(&t.d_aux, n * sizeof(float2)));
   BH_CUDA(bhg::dev_malloc(&t.d_lvl, n * sizeof(uint8_t)));
   t.node_cap = n_nodes;
+  BH_CUDA(bhg::dev_malloc(&t.d_sib, (size_t)entries * sizeof(bhg::WalkSib)));
+  if (ctx->opt.quadrupole)
+    BH_CUDA(bhg::dev_malloc(&t.d_squad, (size_t)entries * sizeof(bhg::WalkQuad)));
+  BH_CUDA(bhg::dev_malloc(&t.d_cmass, (size_t)nb * bhg::kCellsPerBlock * sizeof(float)));
+  t.sib_cap = entries;
   return BH_OK;
 }
 
@@ -149,16 +160,17 @@ bh_status use_device(bh_ctx *ctx) {
 // The geometry a build takes from the host lives in one device region with a
 // pinned host mirror, so that a build uploads it in one copy:
 // [mmax (nf u64, zeroed) | L, 1/L (nf f64 each) | fstart (nf + 1 int) |
-//  level (nb int) | ijk (3 nb int)], nf = nf_cap, nb = geo_nb_cap.
+//  flev (nf int) | level (nb int) | ijk (3 nb int)], nf = nf_cap, nb = geo_nb_cap.
 struct GeoLayout {
-  size_t L, invL, fstart, level, ijk, end;
+  size_t L, invL, fstart, flev, level, ijk, end;
 };
 GeoLayout geo_layout(int64_t nf, int64_t nb) {
   GeoLayout g;
   g.L = 8 * nf;
   g.invL = 16 * nf;
   g.fstart = 24 * nf;
-  g.level = (g.fstart + 4 * (nf + 1) + 15) & ~(size_t)15;
+  g.flev = g.fstart + 4 * (nf + 1);
+  g.level = (g.flev + 4 * nf + 15) & ~(size_t)15;
   g.ijk = g.level + 4 * nb;
   g.end = g.ijk + 12 * nb;
   return g;
@@ -170,7 +182,7 @@ void free_fields(bhg::Tree &t) {
   t.h_geo = nullptr;
   t.d_mmax = nullptr;
   t.d_L = t.d_invL = nullptr;
-  t.d_fstart = t.d_level = t.d_ijk = nullptr;
+  t.d_fstart = t.d_flev = t.d_level = t.d_ijk = nullptr;
   t.nf_cap = 0;
   t.geo_nb_cap = 0;
 }
@@ -197,6 +209,7 @@ bh_status ensure_fields(bh_ctx *ctx, int nfields, int nb) {
   t.d_L = reinterpret_cast<double *>(t.d_geo + g.L);
   t.d_invL = reinterpret_cast<double *>(t.d_geo + g.invL);
   t.d_fstart = reinterpret_cast<int *>(t.d_geo + g.fstart);
+  t.d_flev = reinterpret_cast<int *>(t.d_geo + g.flev);
   t.d_level = reinterpret_cast<int *>(t.d_geo + g.level);
   t.d_ijk = reinterpret_cast<int *>(t.d_geo + g.ijk);
   t.nf_cap = (int)nf;
@@ -212,9 +225,20 @@ bhg::FieldArgs field_args(bhg::Tree &t) {
   fa.fld = t.d_fld;
   fa.invL = t.d_invL;
   fa.L = t.d_L;
+  fa.flev = t.d_flev;
   fa.mmax = t.d_mmax;
   fa.inv_theta = t.last_inv_theta;
   return fa;
+}
+
+bhg::SibArgs sib_args(const bhg::Tree &t) {
+  bhg::SibArgs a;
+  a.sib = t.d_sib;
+  a.quad = t.d_squad;
+  a.cmass = t.d_cmass;
+  a.tops = (int64_t)bhg::kSibsPerBlock * t.nb;
+  a.slots = t.nb / 7 + 1;
+  return a;
 }
 
 // Moments of the current geometry from a density (k_blocks, then
@@ -235,7 +259,7 @@ bh_status enqueue_moments(bh_ctx *ctx, const void *density, int density_is_fp64,
   }
   BH_CUDA(bhg::launch_moments(s, t.nb, t.d_blk, t.d_orig, t.d_count, t.d_prestart, density, density_is_fp64, fa, t.n_nodes, t.d_mom, t.d_rec, t.d_aux,
                               t.d_lvl, q64, qrec, t.d_flags, bhg::top_args(t.d_top, t.nb_cap),
-                              before_upper));
+                              sib_args(t), before_upper));
   return BH_OK;
 }
 
@@ -328,17 +352,21 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   fstart[nfields] = nb;
   fnode[nfields] = n_nodes;
   int max_level = 0;
-  for (int b = 0; b < nb; ++b) {
-    if (level[b] < 0 || level[b] > bhg::kMaxBlockLevel)
-      return fail(ctx, BH_ERR_GEOMETRY, "%s: block %d has level %d outside [0, 18]", who, b,
-                  level[b]);
-    max_level = level[b] > max_level ? level[b] : max_level;
+  std::vector<int> flev(nfields, 0);
+  for (int f = 0; f < nfields; ++f) {
+    for (int b = fstart[f]; b < fstart[f + 1]; ++b) {
+      if (level[b] < 0 || level[b] > bhg::kMaxBlockLevel)
+        return fail(ctx, BH_ERR_GEOMETRY, "%s: block %d has level %d outside [0, 18]", who, b,
+                    level[b]);
+      flev[f] = level[b] > flev[f] ? level[b] : flev[f];
+    }
+    max_level = flev[f] > max_level ? flev[f] : max_level;
   }
   bh_status st = use_device(ctx);
   if (st != BH_OK) return st;
   if ((st = ensure_blocks(ctx, nb)) != BH_OK) return st;
   if ((st = ensure_fields(ctx, nfields, nb)) != BH_OK) return st;
-  if ((st = ensure_nodes(ctx, n_nodes)) != BH_OK) return st;
+  if ((st = ensure_nodes(ctx, n_nodes, nb)) != BH_OK) return st;
   t.nfields = nfields;
   t.nb = nb;
   t.n_nodes = n_nodes;
@@ -358,6 +386,7 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   memcpy(t.h_geo + g.L, L.data(), (size_t)nfields * sizeof(double));
   memcpy(t.h_geo + g.invL, invL.data(), (size_t)nfields * sizeof(double));
   memcpy(t.h_geo + g.fstart, fstart.data(), (size_t)(nfields + 1) * sizeof(int));
+  memcpy(t.h_geo + g.flev, flev.data(), (size_t)nfields * sizeof(int));
   memcpy(t.h_geo + g.level, level, (size_t)nb * sizeof(int));
   memcpy(t.h_geo + g.ijk, ijk, 3 * (size_t)nb * sizeof(int));
   ctx->build_timed = false;
@@ -500,7 +529,7 @@ static cudaError_t enqueue_walk(bh_ctx *ctx, cudaStream_t s, double G, void *out
     shape.order = (shape.longest && np <= 2 && t.order_n[np - 1] == groups) ? t.d_order[np - 1]
                                                                              : nullptr;
   }
-  return bhg::launch_walk(s, ctx->opt, t.nb, t.d_rec, t.d_mom, t.d_qrec, t.d_q64, t.d_blk,
+  return bhg::launch_walk(s, ctx->opt, t.nb, t.d_rec, t.d_mom, sib_args(t), t.d_q64, t.d_blk,
                           t.d_orig, field_args(t), G, out, n_int, n_test, n_leaf, shape);
 }
 
@@ -535,7 +564,8 @@ bh_status bh_create(bh_ctx **out, const bh_options *opt, int device, void *cuda_
   ctx->opt = o;
   ctx->device = device;
   ctx->stream = (cudaStream_t)cuda_stream;
-  if (cudaSetDevice(device) != cudaSuccess || bhg::prepare_learned_kernels() != cudaSuccess ||
+  if (cudaSetDevice(device) != cudaSuccess || bhg::prepare_walk_kernels() != cudaSuccess ||
+      bhg::prepare_learned_kernels() != cudaSuccess ||
       bhg::prepare_mlp_tc_kernel() != cudaSuccess ||
       bhg::prepare_learned_tc_kernel() != cudaSuccess ||
       bhg::dev_malloc(&ctx->tree.d_flags, 8 * sizeof(unsigned)) != cudaSuccess ||
@@ -640,6 +670,14 @@ bh_status ctx_prepare(bh_ctx *ctx, double theta) { return prepare(ctx, theta); }
 
 extern "C" {
 
+// The squared opening radii for 1/theta on the context's stream.
+static cudaError_t enqueue_s2(bh_ctx *ctx, float inv_theta) {
+  bhg::Tree &t = ctx->tree;
+  const int64_t tops = t.n_nodes - (int64_t)bhg::kNodesPerBlock * t.nb;
+  return bhg::launch_prepare_s2(ctx->stream, t.n_nodes, t.d_aux, t.d_rec,
+                                (int64_t)bhg::kSibsPerBlock * t.nb + 8 * tops, t.d_sib, inv_theta);
+}
+
 static bh_status prepare(bh_ctx *ctx, double theta) {
   bhg::Tree &t = ctx->tree;
   if (!t.built) return fail(ctx, BH_ERR_STATE, "no tree: call bh_build first");
@@ -650,7 +688,7 @@ static bh_status prepare(bh_ctx *ctx, double theta) {
   const float inv_theta = (float)(1.0 / theta);
   t.last_inv_theta = inv_theta;
   if (inv_theta != t.s2_inv_theta) {
-    BH_CUDA(bhg::launch_prepare_s2(ctx->stream, t.n_nodes, t.d_aux, t.d_rec, inv_theta));
+    BH_CUDA(enqueue_s2(ctx, inv_theta));
     t.s2_inv_theta = inv_theta;
   }
   return BH_OK;
@@ -980,7 +1018,7 @@ bh_status bh_solve_graph(bh_ctx *ctx, const void *density, int density_is_fp64, 
     if (e == cudaSuccess) {
       cap = enqueue_moments(ctx, density, density_is_fp64);
       if (cap == BH_OK)
-        e = bhg::launch_prepare_s2(s, t.n_nodes, t.d_aux, t.d_rec, (float)(1.0 / theta));
+        e = enqueue_s2(ctx, (float)(1.0 / theta));
       if (cap == BH_OK && e == cudaSuccess && ctx->opt.learned && !ctx->d_mlp)
         cap = fail(ctx, BH_ERR_STATE, "learned walk: call bh_set_mlp first");
       if (cap == BH_OK && e == cudaSuccess)
@@ -1103,8 +1141,10 @@ bh_status bh_stats(const bh_ctx *ctx, bh_stats_t *out) {
   // pos, fld, and 8 bytes of top-node child lists
   int64_t b = t.nb_cap * (int64_t)(4 + 12 + 8 + 8 + 4 + 4 + 4 + 4 + 16 + 4 + 4 + 4 + 16 + 8);
   b += t.node_cap * (int64_t)(sizeof(double4_32a) + sizeof(bhg::WalkRec) + sizeof(float2) + 1);
+  b += t.sib_cap * (int64_t)(sizeof(bhg::WalkSib) + (t.d_squad ? sizeof(bhg::WalkQuad) : 0));
+  if (t.d_cmass) b += t.sib_cap / bhg::kSibsPerBlock * bhg::kCellsPerBlock * (int64_t)sizeof(float);
   b += t.quad_cap * (int64_t)sizeof(bhg::WalkQuad) + (t.d_q64 ? t.quad_cap * 48 : 0);
-  b += t.nf_cap * (int64_t)(sizeof(int) + 2 * sizeof(double)) + (t.nf_cap ? 4 : 0);
+  b += t.nf_cap * (int64_t)(2 * sizeof(int) + 2 * sizeof(double)) + (t.nf_cap ? 4 : 0);
   b += t.stage_in_bytes + t.stage_out_bytes + 4 * sizeof(unsigned);
   if (ctx->d_mlp) b += sizeof(bhg::MlpDev) + sizeof(bhg::MlpTc) + sizeof(unsigned);
   if (ctx->d_counts) b += 3 * sizeof(unsigned long long);

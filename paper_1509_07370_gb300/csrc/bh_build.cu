@@ -457,13 +457,17 @@ __device__ __forceinline__ WalkRec make_rec(double x, double y, double z, double
 // keep_off: also keep the binary32 offset R - c of the centre of mass from
 // the geometric centre, x and y in the record's two spare words (z goes
 // into the quadrupole record's, store_quad_f), for the parent's quadrupole
-// shift.
+// shift.  spare: the record's first spare word otherwise (a top node's slot).
+// sib: the node's place in sibling order (null: a field's root), kids its
+// children's.
 __device__ __forceinline__ float store_internal(int64_t id, int64_t skip, int level,
                                                 const Moment &r, double4_32a *mom, WalkRec *rec,
                                                 float2 *aux, uint8_t *lvl, int ku,
-                                                float inv_theta, bool keep_off = false) {
+                                                float inv_theta, WalkSib *sib, unsigned kids,
+                                                bool keep_off = false, float spare = 0.0f) {
   mom[id] = make_double4_32a(r.x, r.y, r.z, r.m);
   WalkRec w = make_rec(r.x, r.y, r.z, r.m, ku, skip);
+  w.pad[0] = spare;
   if (keep_off) {
     w.pad[0] = narrow(r.ox);
     w.pad[1] = narrow(r.oy);
@@ -474,6 +478,18 @@ __device__ __forceinline__ float store_internal(int64_t id, int64_t skip, int le
     w.s2 = __fmul_rn(s, s);
   }
   rec[id] = w;
+  if (sib) {
+    WalkSib b;
+    b.px = w.px;
+    b.py = w.py;
+    b.pz = w.pz;
+    b.m = w.m;
+    b.s2 = w.s2;
+    b.kids = kids;
+    b.l = l;
+    b.delta = delta;
+    *sib = b;
+  }
   aux[id] = make_float2(l, delta);
   if (lvl) lvl[id] = (uint8_t)level;
   return w.m;
@@ -535,8 +551,9 @@ __device__ __forceinline__ void add_shifted_ff(float Q[6], const float *Qc, floa
 }
 
 // oz: the node's binary32 offset R_z - c_z (see store_internal), or 0.
+// squad: the node's place in sibling order, or null.
 __device__ __forceinline__ void store_quad_f(int64_t id, const float Q[6], WalkQuad *qrec,
-                                             float oz = 0.0f) {
+                                             WalkQuad *squad, float oz = 0.0f) {
   WalkQuad w;
   w.hxx = 0.5f * Q[0];
   w.hyy = 0.5f * Q[1];
@@ -547,6 +564,7 @@ __device__ __forceinline__ void store_quad_f(int64_t id, const float Q[6], WalkQ
   w.pad[0] = oz;
   w.pad[1] = 0.0f;
   qrec[id] = w;
+  if (squad) *squad = w;
 }
 
 // The quadrupole of a node back from its binary32 walk record.
@@ -588,7 +606,7 @@ __global__ void __launch_bounds__(kBlockThreads)
              float inv_theta, int64_t n_nodes,
              double4_32a *__restrict__ mom, WalkRec *__restrict__ rec, float2 *__restrict__ aux,
              uint8_t *__restrict__ lvl, double *__restrict__ q64, WalkQuad *__restrict__ qrec,
-             unsigned *flags) {
+             const SibArgs sib, unsigned *flags) {
   __shared__ double cm[512], cxs[512], cys[512], czs[512];  // cells, local Morton order
   __shared__ float cmu[512];                                // cell mass, binary32 unit
   const bool quad64 = q64 != nullptr;                       // FP64 quadrupoles
@@ -627,6 +645,7 @@ __global__ void __launch_bounds__(kBlockThreads)
     const float mu = narrow_scaled(mass, ku);
     cm[m] = mass;
     cmu[m] = mu;
+    sib.cmass[(int64_t)p * kCellsPerBlock + m] = mu;
     cxs[m] = ux;
     cys[m] = uy;
     czs[m] = uz;
@@ -662,7 +681,9 @@ __global__ void __launch_bounds__(kBlockThreads)
       accumulate(M, Sx, Sy, Sz, cm[8 * q + o], cxs[8 * q + o], cys[8 * q + o], czs[8 * q + o]);
     const Moment r = finish(M, Sx, Sy, Sz, cx, cy, cz);
     const int64_t id = root + 2 + 73 * (q >> 3) + 9 * (q & 7);
-    store_internal(id, id + 9, lb + 2, r, mom, rec, aux, lvl, ku, inv_theta, quad32);
+    const int64_t sid = (int64_t)kSibsPerBlock * p + 8 + q;
+    store_internal(id, id + 9, lb + 2, r, mom, rec, aux, lvl, ku, inv_theta, sib.sib + sid,
+                   kBottomBit | (unsigned)(64 * p + q), quad32);
     if (quad64) {
       double Q[6] = {0, 0, 0, 0, 0, 0};
       for (int o = 0; o < 8; ++o) {
@@ -680,7 +701,7 @@ __global__ void __launch_bounds__(kBlockThreads)
         add_shifted_ff(Q, nullptr, cmu[8 * q + o], __fsub_rn(dx, ox), __fsub_rn(dy, oy),
                        __fsub_rn(dz, oz));
       }
-      store_quad_f(id, Q, qrec, oz);
+      store_quad_f(id, Q, qrec, sib.quad ? sib.quad + sid : nullptr, oz);
     }
   }
 }
@@ -714,7 +735,8 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
                                                int64_t skip, int64_t first, int ku,
                                                double inv_unit, float inv_theta,
                                                double4_32a *mom, WalkRec *rec, float2 *aux,
-                                               uint8_t *lvl, double *q64, WalkQuad *qrec) {
+                                               uint8_t *lvl, double *q64, WalkQuad *qrec,
+                                               WalkSib *sib, WalkQuad *squad, unsigned kids) {
   constexpr int64_t stride = 9;
   const double cx = centre_coord(ix, lev), cy = centre_coord(iy, lev), cz = centre_coord(iz, lev);
   double4_32a ch[8];
@@ -726,7 +748,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
   for (int o = 1; o < 8; ++o) accumulate(M, Sx, Sy, Sz, ch[o].w, ch[o].x, ch[o].y, ch[o].z);
   const Moment r = finish(M, Sx, Sy, Sz, cx, cy, cz);
   const bool quad32 = qrec && !q64;
-  store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, quad32);
+  store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, sib, kids, quad32);
   if (q64) {
     double Q[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
@@ -753,7 +775,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
                      __fsub_rn(__fadd_rn(dy, cr.pad[1]), oy),
                      __fsub_rn(__fadd_rn(dz, cq.pad[0]), oz));
     }
-    store_quad_f(id, Q, qrec, oz);
+    store_quad_f(id, Q, qrec, squad, oz);
   }
 }
 
@@ -776,7 +798,8 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
                                            int64_t id, int64_t skip, int64_t child, int ku,
                                            double inv_unit, float inv_theta, double4_32a *mom,
                                            WalkRec *rec, float2 *aux, uint8_t *lvl, double *q64,
-                                           WalkQuad *qrec) {
+                                           WalkQuad *qrec, WalkSib *sib, WalkQuad *squad,
+                                           unsigned kids, float spare = 0.0f) {
   const double4_32a c = CG ? ld_mom_cg(mom + child) : mom[child];
   WalkQuad qc = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, {0.0f, 0.0f}};
   float fm = 0.0f, gx = 0.0f, gy = 0.0f;
@@ -815,7 +838,8 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
   r.delta = __dsqrt_rn(__dadd_rn(__dadd_rn(__shfl_sync(gmask, sq, gbase + 1),
                                            __shfl_sync(gmask, sq, gbase + 2)),
                                  __shfl_sync(gmask, sq, gbase + 3)));
-  if (o == 0) store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta);
+  if (o == 0) store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, sib, kids, false,
+                             spare);
   if (q64) {  // FP64 quadrupoles (the FP64 walk): on lane 0, as the one-thread form
     int64_t kids[8];
 #pragma unroll
@@ -859,27 +883,37 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
     add_shifted_ff(Q, Qc, __shfl_sync(gmask, fm, gbase + j), __shfl_sync(gmask, sx, gbase + j),
                    __shfl_sync(gmask, sy, gbase + j), __shfl_sync(gmask, sz, gbase + j));
   }
-  if (o == 0) store_quad_f(id, Q, qrec);
+  if (o == 0) store_quad_f(id, Q, qrec, squad);
 }
 
-// The top node whose slot holds {a, b} (made by k_top_nodes: node, skip, cube,
-// level, field) and whose child o is c, by a group of 8 lanes; its
+// The octant of cube (i, j, k) in its parent.
+__device__ __forceinline__ int octant_of(int i, int j, int k) {
+  return (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
+}
+
+// The top node whose slot s holds {a, b} (made by k_top_nodes: node, skip, cube,
+// level, field), whose parent has slot up (-1: none) and whose child o is c, by a group of 8 lanes; its
 // children -- top nodes one level down or block roots -- were written by
 // other CTAs and are read through L2.  ku: the field's mass-unit exponent.
 // False when the slot is inconsistent (a failed geometry).
-__device__ __forceinline__ bool top_node(unsigned gmask, int gbase, int o, int4 a, int4 b,
+__device__ __forceinline__ bool top_node(unsigned gmask, int gbase, int o, int s, int4 a, int4 b,
                                          int64_t c, int ku, int nb, int nfields,
                                          int64_t n_nodes, double4_32a *mom, WalkRec *rec,
                                          float2 *aux, double *q64, WalkQuad *qrec,
-                                         float inv_theta) {
+                                         float inv_theta, const SibArgs &sib, int up) {
   const int level = b.y;
   if (a.x < 0 || a.x >= n_nodes || level < 0 || level >= kKeyLevels || b.z < 0 ||
       b.z >= nfields || b.w < 0 || b.w >= nb)
     return false;
   if (__any_sync(gmask, c <= 0 || c >= n_nodes)) return false;
+  const bool listed = up >= 0 && up < sib.slots;
+  const int64_t sid = sib.tops + 8 * (int64_t)up + octant_of(a.z, a.w, b.x);
   group_node<false, true>(gmask, gbase, o, level, 0, 0, 0, centre_coord(a.z, level),
                           centre_coord(a.w, level), centre_coord(b.x, level), a.x, a.y, c, ku,
-                          pow2i(ku), inv_theta, mom, rec, aux, nullptr, q64, qrec);
+                          pow2i(ku), inv_theta, mom, rec, aux, nullptr, q64, qrec,
+                          listed ? sib.sib + sid : nullptr,
+                          listed && sib.quad ? sib.quad + sid : nullptr,
+                          (unsigned)(sib.tops + 8 * (int64_t)s), __int_as_float(s));
   return true;
 }
 
@@ -901,7 +935,8 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
                  const int *__restrict__ count, const int *__restrict__ prestart,
                  const int *__restrict__ fid, const unsigned long long *__restrict__ mmax,
                  float inv_theta, int64_t n_nodes, double4_32a *mom, WalkRec *rec, float2 *aux,
-                 uint8_t *lvl, double *q64, WalkQuad *qrec, unsigned *flags, TopArgs top) {
+                 uint8_t *lvl, double *q64, WalkQuad *qrec, unsigned *flags, TopArgs top,
+                 const SibArgs sib) {
   const int p0 = blockIdx.x * kUpperBlocks;
   const int t = threadIdx.x;
   {  // (1) level-one nodes: block p0 + t/8, octant t%8
@@ -912,10 +947,12 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
       const int64_t root = (int64_t)prestart[p] + count[p];
       if (lb >= 0 && lb <= kMaxBlockLevel && root >= 0 && root + kNodesPerBlock <= n_nodes) {
         const int ku = -mass_exponent(mmax[fid[orig[p]]]);
-        const int64_t id = root + 1 + 73 * c;
+        const int64_t id = root + 1 + 73 * c, sid = (int64_t)kSibsPerBlock * p + c;
         level_one_node(lb + 1, 2 * B.y + (c & 1), 2 * B.z + ((c >> 1) & 1),
                        2 * B.w + ((c >> 2) & 1), id, id + 73, id + 1, ku, pow2i(ku), inv_theta,
-                       mom, rec, aux, lvl, q64, qrec);
+                       mom, rec, aux, lvl, q64, qrec, sib.sib + sid,
+                       sib.quad ? sib.quad + sid : nullptr,
+                       (unsigned)(kSibsPerBlock * p + 8 + 8 * c));
       }
     }
   }
@@ -930,12 +967,16 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
   const int64_t root = (int64_t)prestart[p] + count[p];
   if (lb < 0 || lb > kMaxBlockLevel || root < 0 || root + kNodesPerBlock > n_nodes) return;
   const int ku = -mass_exponent(mmax[fid[orig[p]]]);
+  int s = top.bparent[p];  // the slot of the root's parent (-1: a field's only block)
+  const bool listed = s >= 0 && s < top.slots && s < sib.slots;  // (a failed geometry: any s)
+  const int64_t sid = sib.tops + 8 * (int64_t)s + octant_of(B.y, B.z, B.w);
   group_node<true, false>(gmask, gbase, o, lb, B.y, B.z, B.w, centre_coord(B.y, lb),
                           centre_coord(B.z, lb), centre_coord(B.w, lb), root,
                           root + kNodesPerBlock, root + 1 + 73 * o, ku, pow2i(ku), inv_theta, mom,
-                          rec, aux, lvl, q64, qrec);
+                          rec, aux, lvl, q64, qrec, listed ? sib.sib + sid : nullptr,
+                          listed && sib.quad ? sib.quad + sid : nullptr,
+                          (unsigned)(kSibsPerBlock * p));
   // (3) climb: the parent top node of this root, then its parents
-  int s = top.bparent[p];
   while (s >= 0) {
     if (s >= top.slots) {  // a failed geometry
       if (o == 0) atomicOr(flags, kErrIndex);
@@ -959,8 +1000,8 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
     }
     __threadfence();  // the other children's moments after their arrivals
     if (o == 0) top.arrive[s] = 0u;
-    if (!top_node(gmask, gbase, o, a, b, c, kuf, nb, nfields, n_nodes, mom, rec, aux, q64, qrec,
-                  inv_theta)) {
+    if (!top_node(gmask, gbase, o, s, a, b, c, kuf, nb, nfields, n_nodes, mom, rec, aux, q64, qrec,
+                  inv_theta, sib, up)) {
       if (o == 0) atomicOr(flags, kErrIndex);
       return;
     }
@@ -1109,23 +1150,23 @@ cudaError_t launch_moments(cudaStream_t s, int nb, const int4 *blk, const int *o
                            const int *count, const int *prestart, const void *density, int density_is_fp64, const FieldArgs &fa,
                            int64_t n_nodes, double4_32a *mom, WalkRec *rec, float2 *aux,
                            uint8_t *lvl, double *q64, WalkQuad *qrec, unsigned *flags,
-                           const TopArgs &top, cudaEvent_t before_upper) {
+                           const TopArgs &top, const SibArgs &sib, cudaEvent_t before_upper) {
   if (density_is_fp64)
     k_blocks<double><<<nb, kBlockThreads, 0, s>>>(nb, blk, orig, count, prestart,
                                                    (const double *)density, fa.L, fa.fid,
                                                    fa.mmax, fa.inv_theta, n_nodes, mom, rec, aux,
-                                                   lvl, q64, qrec, flags);
+                                                   lvl, q64, qrec, sib, flags);
   else
     k_blocks<float><<<nb, kBlockThreads, 0, s>>>(nb, blk, orig, count, prestart,
                                                   (const float *)density, fa.L, fa.fid, fa.mmax,
                                                   fa.inv_theta, n_nodes, mom, rec, aux, lvl, q64,
-                                                  qrec, flags);
+                                                  qrec, sib, flags);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (before_upper && (e = cudaStreamWaitEvent(s, before_upper, 0)) != cudaSuccess) return e;
   k_upper_tree<<<grid_for(nb, kUpperBlocks), 8 * kUpperBlocks, 0, s>>>(
       nb, fa.nfields, blk, orig, count, prestart, fa.fid, fa.mmax, fa.inv_theta, n_nodes, mom,
-      rec, aux, lvl, q64, qrec, flags, top);
+      rec, aux, lvl, q64, qrec, flags, top, sib);
   return cudaGetLastError();
 }
 

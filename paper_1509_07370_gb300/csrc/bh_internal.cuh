@@ -10,11 +10,27 @@
 //                                 field's binary32 mass unit (below), the
 //                                 squared opening radius s2 for the current
 //                                 theta (0 for cells), and the index of the
-//                                 first node after the subtree; 8 bytes of
-//                                 padding keep records 32-byte aligned
+//                                 first node after the subtree; two spare
+//                                 words keep records 32-byte aligned (a top
+//                                 node's first: its slot)
 //   aux  float2  {l, delta}       node side and |R - centre| in binary32
 //                                 (both 0 for cells)
 //   lvl  uint8                    node level
+// The binary32 walk tests eight siblings at a time, so it reads the internal
+// nodes from a second array in sibling order (sib, squad), where they are
+// neighbours (32 records of four parents lie in 8 lines of 128 bytes instead
+// of 32: the first version read them from rec and was bound by the L1 tag
+// stage), and the cells as bare masses (cmass), their places following from
+// the block:
+//   sib   WalkSib (32 bytes)      at 72 p + c the level-one node c of sorted
+//                                 block p, at 72 p + 8 + q its bottom node q
+//                                 (local Morton order), at 72 nb + 8 s + o the
+//                                 child o of the top node of slot s (a block
+//                                 root or a top node)
+//   squad WalkQuad                the same order (quadrupole option)
+//   cmass float                   at 512 p + m the mass of cell m of sorted
+//                                 block p (local Morton order), in the field's
+//                                 binary32 mass unit
 // Leaf blocks are renumbered in Morton order of their lower corner ("sorted
 // position" p); blk[p] = {level, bi, bj, bk}, orig[p] = caller block index.
 //
@@ -69,6 +85,21 @@ struct __align__(32) WalkRec {
 };
 static_assert(sizeof(WalkRec) == 32, "walk record must be 32 bytes");
 
+// An internal node in sibling order.  kids: where its children start (for a
+// bottom node kBottomBit | 64 p + q, so that its cells' masses are at 8 times
+// that); l, delta: for the squared opening radius of another theta.
+struct __align__(32) WalkSib {
+  float px, py, pz, m;
+  float s2;
+  unsigned kids;
+  float l, delta;
+};
+static_assert(sizeof(WalkSib) == 32, "sibling record must be 32 bytes");
+constexpr unsigned kBottomBit = 0x80000000u;
+constexpr int kSibsPerBlock = 72;
+// Entries of nb blocks: a top node has 8 children and all but the roots are
+// children, so fewer than nb / 7 top nodes have 8 entries each.
+constexpr int64_t sib_entries(int64_t nb) { return kSibsPerBlock * nb + 8 * (nb / 7 + 1); }
 // Quadrupole walk record (quadrupole or learned option), box units and the
 // field's binary32 mass unit: half the diagonal of Q and the off-diagonal
 // terms (read as 24 bytes, like WalkRec), so that
@@ -81,9 +112,18 @@ struct __align__(32) WalkQuad {
 };
 static_assert(sizeof(WalkQuad) == 32, "quadrupole record must be 32 bytes");
 
-// Launch shape of the per-cell binary32 walk: warps per CTA, x-neighbour
-// target pairs per lane (a warp's group of targets: 1 pair = a 4x4x4 octant,
-// 2 pairs = a 8x4x4 slab), and the schedule: ticket = 0 a plain grid of one
+// The walk's arrays (quad null without the quadrupole option).
+struct SibArgs {
+  WalkSib *sib = nullptr;
+  WalkQuad *quad = nullptr;
+  float *cmass = nullptr;
+  int64_t tops = 0;   // where the top nodes' children start: 72 nb
+  int64_t slots = 0;  // top nodes there is room for: nb / 7 + 1
+};
+
+// Launch shape of the binary32 walk: warps per CTA, a warp's group of targets
+// (pairs = 1: a 4x4x4 octant, 2: two x-neighbouring octants one after the
+// other), and the schedule: ticket = 0 a plain grid of one
 // warp per group; ticket = k > 0 a persistent grid (as many CTAs as fit on
 // the GPU at once) whose warps take k groups at a time from `counter` (a
 // device word that the launch resets) until all are taken.  0 = defaults.
@@ -151,9 +191,10 @@ struct Tree {
   int4 *d_fld = nullptr;        // per sorted block
   double *d_invL = nullptr;     // per field
   double *d_L = nullptr;        // per field
+  int *d_flev = nullptr;        // per field
   unsigned long long *d_mmax = nullptr;  // per field, largest cell mass (bits)
   int nf_cap = 0;
-  // d_mmax, d_L, d_invL, d_fstart, d_level and d_ijk live in d_geo, which a
+  // d_mmax, d_L, d_invL, d_fstart, d_flev, d_level and d_ijk live in d_geo, which a
   // build fills from its pinned mirror h_geo in one copy (geo_done: that copy)
   unsigned char *d_geo = nullptr, *h_geo = nullptr;
   int64_t geo_nb_cap = 0;
@@ -181,6 +222,10 @@ struct Tree {
   float2 *d_aux = nullptr;
   uint8_t *d_lvl = nullptr;
   int64_t node_cap = 0;
+  WalkSib *d_sib = nullptr;     // sibling order (capacity sib_cap entries)
+  WalkQuad *d_squad = nullptr;
+  float *d_cmass = nullptr;
+  int64_t sib_cap = 0;
   double *d_q64 = nullptr;      // 6 per node, FP64 quadrupoles (quadrupole option)
   WalkQuad *d_qrec = nullptr;   // binary32 quadrupole walk records
   int64_t quad_cap = 0;
@@ -210,6 +255,7 @@ struct FieldArgs {
   int4 *fld;
   const double *invL;
   const double *L;   // box side per field
+  const int *flev;   // deepest block level per field
   unsigned long long *mmax;  // per field: bits of the largest FP64 cell mass
   // > 0: the moment kernels also write the squared opening radius of every
   // internal node for this 1/theta (as k_prepare_s2 would); 0: they write 0
@@ -270,23 +316,27 @@ cudaError_t launch_moments(cudaStream_t s, int nb, const int4 *blk, const int *o
                            const int *count, const int *prestart, const void *density, int density_is_fp64, const FieldArgs &fa,
                            int64_t n_nodes, double4_32a *mom, WalkRec *rec, float2 *aux,
                            uint8_t *lvl, double *q64, WalkQuad *qrec, unsigned *flags,
-                           const TopArgs &top, cudaEvent_t before_upper = nullptr);
+                           const TopArgs &top, const SibArgs &sib,
+                        cudaEvent_t before_upper = nullptr);
 // Raises the dynamic shared-memory limit of the learned walk (more than 48 KB)
 // on the current device; called once per context, outside any graph capture.
 cudaError_t prepare_learned_kernels();
 
 // ---- walk kernels (bh_walk.cu) ---------------------------------------------
+// s2 of every node of rec and of every entry of sib (entries in all).
 cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux, WalkRec *rec,
-                              float inv_theta);
+                              int64_t entries, WalkSib *sib, float inv_theta);
 // out: float* (F32) or double* (F64); counts: optional per-cell n_int/n_test.
 // Potential scale of field f: -G * invL[f] (times the field's mass unit for
 // the binary32 walk).  shape = the launch shape of the per-cell binary32
 // walk (warps per CTA, target pairs per lane; 0 = defaults), tunable.
 cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
-                        const double4_32a *mom, const WalkQuad *qrec, const double *q64,
-                        const int4 *blk, const int *orig, const FieldArgs &fa, double G,
-                        void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf = nullptr,
+                        const double4_32a *mom, const SibArgs &sib, const double *q64,
+                        const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf = nullptr,
                         WalkShape shape = WalkShape());
+// Raises the dynamic shared-memory limit of the walk kernels on the current
+// device; called once per context, outside any graph capture.
+cudaError_t prepare_walk_kernels();
 
 // ---- small device helpers ---------------------------------------------------
 // Spread the low 21 bits of v so bit b lands at bit 3b.

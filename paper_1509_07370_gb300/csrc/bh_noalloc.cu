@@ -49,7 +49,7 @@ constexpr size_t kOffBlk = up256(kOffPrestart + sizeof(int) * kNoAllocMaxBlocks)
 constexpr size_t kOffOrig = up256(kOffBlk + sizeof(int4) * kNoAllocMaxBlocks);
 constexpr size_t kOffFlags = up256(kOffOrig + sizeof(int) * kNoAllocMaxBlocks);
 constexpr size_t kOffFstart = up256(kOffFlags + 4 * sizeof(unsigned));   // one field
-constexpr size_t kOffFid = up256(kOffFstart + 2 * sizeof(int));
+constexpr size_t kOffFid = up256(kOffFstart + 3 * sizeof(int));  // fstart, then flev
 constexpr size_t kOffFld = up256(kOffFid + sizeof(int) * kNoAllocMaxBlocks);
 constexpr size_t kOffBox = up256(kOffFld + sizeof(int4) * kNoAllocMaxBlocks);  // L, 1/L
 constexpr size_t kOffMmax = up256(kOffBox + 2 * sizeof(double));  // largest cell mass
@@ -58,7 +58,10 @@ constexpr size_t kOffRec = up256(kOffMom + sizeof(double4_32a) * kNoAllocMaxNode
 constexpr size_t kOffAux = up256(kOffRec + sizeof(WalkRec) * kNoAllocMaxNodes);
 constexpr size_t kOffLvl = up256(kOffAux + sizeof(float2) * kNoAllocMaxNodes);
 constexpr size_t kOffTop = up256(kOffLvl + sizeof(uint8_t) * kNoAllocMaxNodes);  // TopArgs
-constexpr size_t kScratchBytes = up256(kOffTop + sizeof(int) * top_ints(kNoAllocMaxBlocks));  // ~2.7 MB
+constexpr size_t kOffSib = up256(kOffTop + sizeof(int) * top_ints(kNoAllocMaxBlocks));
+constexpr size_t kOffCmass = up256(kOffSib + sizeof(WalkSib) * sib_entries(kNoAllocMaxBlocks));
+constexpr size_t kScratchBytes =
+    up256(kOffCmass + sizeof(float) * kCellsPerBlock * kNoAllocMaxBlocks);  // ~3.0 MB
 
 // The fixed scratch.  In host code this name is only a stand-in for the
 // symbol: host code must use the address returned by cudaGetSymbolAddress.
@@ -72,12 +75,14 @@ struct Geometry {  // passed by value as a kernel parameter (1 KB)
 // Copies the block geometry from the kernel parameter into the scratch,
 // describes the single field, and clears the error flags of this call.
 __global__ void k_stage_geometry(Geometry g, int nb, int *level, int *ijk, unsigned *flags,
-                                 int *fstart, double *box, double L, unsigned long long *mmax) {
+                                 int *fstart, int max_level, double *box, double L,
+                                 unsigned long long *mmax) {
   const int t = threadIdx.x;
   if (t < 4) flags[t] = 0u;
   if (t == 0) {
     fstart[0] = 0;
     fstart[1] = nb;
+    fstart[2] = max_level;
     box[0] = L;
     box[1] = 1.0 / L;
     *mmax = 0ull;
@@ -162,11 +167,17 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   float2 *d_aux = (float2 *)(base + kOffAux);
   uint8_t *d_lvl = (uint8_t *)(base + kOffLvl);
   const TopArgs top = top_args((int *)(base + kOffTop), kNoAllocMaxBlocks);
+  SibArgs sib;
+  sib.sib = (WalkSib *)(base + kOffSib);
+  sib.cmass = (float *)(base + kOffCmass);
+  sib.tops = (int64_t)kSibsPerBlock * nb;
+  sib.slots = nb / 7 + 1;
   int *d_fstart = (int *)(base + kOffFstart);
   double *d_box = (double *)(base + kOffBox);
   FieldArgs fa;
   fa.nfields = 1;
   fa.fstart = d_fstart;
+  fa.flev = d_fstart + 2;
   fa.fid = (int *)(base + kOffFid);
   fa.fld = (int4 *)(base + kOffFld);
   fa.L = d_box;
@@ -174,8 +185,8 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   fa.mmax = (unsigned long long *)(base + kOffMmax);
   fa.inv_theta = 0.0f;  // s2 is prepared below
 
-  k_stage_geometry<<<1, 256, 0, s>>>(g, nb, d_level, d_ijk, d_flags, d_fstart, d_box, box_len,
-                                     fa.mmax);
+  k_stage_geometry<<<1, 256, 0, s>>>(g, nb, d_level, d_ijk, d_flags, d_fstart, max_level, d_box,
+                                     box_len, fa.mmax);
   NA_CUDA(cudaGetLastError());
   NA_CUDA(launch_keys_mass(s, nb, d_level, d_ijk, d_key[0], d_idx[0], d_flags, fa, density,
                            density_is_fp64));
@@ -187,7 +198,7 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
                            d_lvl, d_flags, fa, d_orig, max_level, top));
   NA_CUDA(launch_moments(s, nb, d_blk, d_orig, d_count, d_prestart, density,
                          density_is_fp64, fa, n_nodes, d_mom, d_rec, d_aux, d_lvl, nullptr, nullptr,
-                         d_flags, top));
+                         d_flags, top, sib));
   // the walk must only run on a valid tree: check the flags first
   unsigned h_flags[4] = {0, 0, 0, 0};
   NA_CUDA(cudaMemcpyAsync(h_flags, d_flags, sizeof(h_flags), cudaMemcpyDeviceToHost, s));
@@ -195,10 +206,11 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   if (h_flags[0] & (kErrLevel | kErrCoord | kErrTiling | kErrIndex)) return BH_ERR_GEOMETRY;
   if ((int64_t)h_flags[2] != (nb - 1) / 7) return BH_ERR_GEOMETRY;
   if (h_flags[0] & kErrDensity) return BH_ERR_ARG;
-  NA_CUDA(launch_prepare_s2(s, n_nodes, d_aux, d_rec, (float)(1.0 / theta)));
+  NA_CUDA(launch_prepare_s2(s, n_nodes, d_aux, d_rec, kSibsPerBlock * nb + 8 * ((nb - 1) / 7),
+                            sib.sib, (float)(1.0 / theta)));
   bh_options opt;
   bh_default_options(&opt);
-  NA_CUDA(launch_walk(s, opt, nb, d_rec, d_mom, nullptr, nullptr, d_blk, d_orig, fa, G, out,
+  NA_CUDA(launch_walk(s, opt, nb, d_rec, d_mom, sib, nullptr, d_blk, d_orig, fa, G, out,
                       nullptr, nullptr, nullptr, WalkShape()));
   return BH_OK;
 }

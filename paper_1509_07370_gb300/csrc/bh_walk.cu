@@ -1,45 +1,56 @@
 // The Barnes-Hut walk: potential at every cell centre (Sec. 3.3).
 //
-// Traversal.  The paper walks with a shared-memory stack pushed by lane 0 and
-// an all() vote on the opening test (Sec. 3.3).  This walk needs no stack:
-// nodes are stored in pre-order, so a node's first child is the next node and
-// its subtree ends at its skip index.  Every target cell keeps `next`, the
-// first node it still has to visit (0 = the root at the start).  In the
-// one-target-per-lane walk (k_walk_scalar) the warp takes the smallest `next`
-// over its lanes at each step (one __reduce_min_sync), all lanes load that
-// node (one broadcast load), and the targets whose `next` equals it apply the
-// opening test of Eq. 4:
-//   accepted -> add M / d, next = skip (the whole subtree is done)
-//   opened   -> next = node + 1 (descend into the first child)
-// Cells carry s2 = 0: the test accepts every other cell (d2 > 0) and rejects
-// only the target's own cell (d2 = 0), which then adds nothing; for a cell
-// node + 1 is its skip, so no special case is needed.  Each target thus
-// visits exactly the nodes of its own recursive walk, in pre-order, and gets
-// the per-cell result of the recursive definition; targets whose `next` lies
-// further ahead wait (masked) for the warp to get there.  `next` only grows,
-// so a walk ends after at most n_nodes steps.  With the warp vote (paper mode)
-// all lanes share `next`.  The per-cell pair walk (walk_group) takes the same
-// decisions in two modes that need no reduction: one vote per node while all
-// targets sit at the same node, a lazy per-target `next` inside a subtree
-// they disagree on.
+// The paper walks node by node with a shared-memory stack and an all() vote
+// (Sec. 3.3).  Here one warp walks for the 64 cells of a 4x4x4 octant of a
+// block in two alternating phases that need no per-node control flow:
 //
-// Work layout.
-//  * Per-cell binary32 walk (the default, k_walk_pair / k_walk_queue): one
-//    warp per 4x4x4 octant of a block (64 cells, local Morton indices 64o ..
-//    64o+63), lane l owning the two x-neighbours 64o+2l and 64o+2l+1, or per
-//    8x4x4 slab (128 cells, two such pairs per lane).  A lane's targets share
-//    ty, tz and so dy, dz; their dx, d2, 1/d products and Kahan sums run as
-//    packed f32x2 operations (two binary32 results per instruction, each
-//    rounded as its scalar counterpart).  CTAs of 2 to 16 warps, on a plain
-//    grid or a persistent one fed by a work counter (the launch shape).
-//  * binary64 interactions and the paper's warp vote (k_walk_scalar): one
-//    warp per 32-cell brick (4x4x2, local Morton 32q .. 32q+31), one target
-//    per lane, as the paper groups its cells (Sec. 3.1.1, Sec. 3.3).
+// 1. Testing.  The warp pops up to four opened nodes from its stack in shared
+//    memory and tests their 32 children, one child per lane: the lane forms
+//    the opening test of Eq. 4 for all 64 targets and gets a 64-bit mask.
+//    Children are addressed directly (inside a block by the strides of the
+//    585-node pre-order subtree, above it by the top-node child lists).  With
+//    P the targets that opened the parent, the targets accepting the child
+//    are A = P & mask, those opening it O = P & ~mask.  A child with A != 0
+//    is staged in shared memory; a child with O != 0 goes on the stack with P
+//    = O, or, if it is a bottom node (its 8 children are cells), to the list
+//    of opened bottom nodes.  Cells are never tested.
+// 2. Evaluating.  Four sub-bricks of 16 cells (4x2x2) each have a list of the
+//    staged nodes that one of their cells accepts, with the 16-bit mask, and
+//    a list of opened bottom nodes.  8 lanes serve a sub-brick: lane bits 0-1
+//    take every fourth list entry, bit 2 is the cell's z within the sub-brick,
+//    and a lane owns the 8 cells (4 in x, 2 in y) of that z.  So a warp
+//    evaluates 16 different (node, 8 cells) pairs at a time, each lane
+//    loading a record once for 8 interactions.
+//
+// Each target visits exactly the nodes of its own recursive walk and takes
+// the decisions of the per-cell definition (or, with the warp vote, those of
+// its 32-cell brick: the two words of the mask are the octant's two bricks).
+// The order in which a target's terms are added depends on its octant's lists
+// only -- not on the launch shape, the other fields of a batch or timing -- so
+// every launch shape gives the same bits.
+//
+// What bounds it.  An interaction costs one rsqrt on the special-function
+// unit (16 lanes per clock and SM: 4 clocks per 64 interactions) and, packed
+// in f32x2 pairs, about 13 (monopole) or 25 (quadrupole) FMA-pipe clocks per
+// 64 and scheduler.  What the lists save against a walk in which 64 targets
+// share every step: at theta 0.75 on the 2M-cell spheroid a target accepts
+// 401 nodes and opens 11 bottom nodes, its octant's union is 687 nodes and 61
+// bottom nodes, a 16-cell sub-brick's 554 and 35 (groups of 4: 483 and 20,
+// but then every lane reads its own record, and the shared-memory return path
+// bounds the quadrupole walk).
+//
+// Measured (2,039,808-cell spheroid, plain grid of 4-warp CTAs; ms, with in
+// brackets the walk that stepped 64 targets, or 32 with the vote, through the
+// tree together): quadrupole theta 0.75 1.08 (1.85), monopole 0.5 2.07 (3.2)
+// and 0.24 11.0 (15.5), vote with quadrupole 0.8 1.01 (2.49); 16.3M-cell core,
+// monopole 0.5 20.0 (27.4); 32^3 cells 0.106 (0.45): there a warp has a
+// scheduler to itself, and a step tests 32 nodes per chain of dependent loads
+// instead of one.
 //
 // The opening test is evaluated in binary32 with the operation order stated
-// in the public header; the interaction uses the same d2 (binary32, Kahan
-// sum) or recomputes d in binary64 from the FP64 moments.
-#include "bh_walk_common.cuh"
+// in the public header; the interaction uses the same d2 formed again, or
+// recomputes d in binary64 from the FP64 moments (k_walk_scalar).
+#include "bh_lists.cuh"
 
 namespace bhg {
 namespace {
@@ -47,11 +58,17 @@ namespace {
 constexpr int kWalkThreads = 256;               // CTA of the scalar walk: 8 bricks = half a block
 constexpr int kWarpsPerCta = kWalkThreads / 32;
 constexpr int kMaxWalkThreads = 512;            // largest tunable CTA
-// Default launch shape of the per-cell walk (the fastest on GB300 for the
-// spheroid and cloud-core workloads at theta 0.24 - 0.72): one target pair
-// per lane (64-target octants), CTAs of 4 warps.
-constexpr int kDefaultPairs = 1;
+// 80 registers: 24 warps per SM (97 without the bound, 20 warps: 8 % slower;
+// 72: 28 warps, spills: 2-5 % slower).
+constexpr int kWalkRegs = 80;
 constexpr int kDefaultWarps = 4;
+
+__global__ void k_prepare_sib_s2(int64_t n, WalkSib *__restrict__ sib, float inv_theta) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const float s = __fadd_rn(__fmul_rn(sib[i].l, inv_theta), sib[i].delta);
+  sib[i].s2 = __fmul_rn(s, s);
+}
 
 __global__ void k_prepare_s2(int64_t n, const float2 *__restrict__ aux, WalkRec *__restrict__ rec,
                              float inv_theta) {
@@ -62,381 +79,515 @@ __global__ void k_prepare_s2(int64_t n, const float2 *__restrict__ aux, WalkRec 
   rec[i].s2 = __fmul_rn(s, s);
 }
 
-// ---- per-cell binary32 walk, x-neighbour target pairs per lane -------------
-//
-// A warp walks for a group of targets that share every y and z coordinate
-// pattern: lane l owns NP pairs of x-neighbours, pair k at x offset 4k, so
-// all 2 NP targets of a lane have the same (y, z) and share dy, dz and
-// dy^2 + dz^2.  NP = 1: the group is a 4x4x4 octant of a block (64 targets);
-// NP = 2: two x-adjacent octants, a 8x4x4 slab (128 targets).  A larger group
-// walks only a few percent more nodes than a smaller one (the union of its
-// targets' walks), so every record loaded serves more targets: the record's
-// broadcast to all 32 lanes (8 registers each) is what the L1 return path
-// spends most of its time on.
-
-// Per-target state of one lane: NP packed pairs.
-template <int NP>
-struct Lanes {
-  u64 tx2[NP];              // {x_a, x_b} of pair k, box units
-  u64 sum[NP], comp[NP];    // Kahan pair sums
-  unsigned next_a[NP], next_b[NP];
-  int ni[2 * NP], nt[2 * NP], nl[2 * NP];  // counting walk
+// ---- binary32 walk -----------------------------------------------------------
+constexpr int kRing = 64;     // staged nodes, a ring: room for one more chunk is kept
+constexpr int kBottoms = 64;   // opened bottom nodes: evaluated once a chunk might not fit
+struct QuadRest {                    // second half of a staged quadrupole (16-byte stride)
+  float qxz, qyz, unused[2];
+};
+template <bool QUAD>
+struct WalkMem {                     // of one warp
+  Front front;
+  float4 node[kRing];                // px, py, pz, m of the staged nodes
+  float4 quad[QUAD ? kRing : 1];     // Qxx/2, Qyy/2, Qzz/2, Qxy
+  QuadRest quad2[QUAD ? kRing : 1];  // Qxz, Qyz
+  uint32_t list[4][kRing];           // per sub-brick, a ring: 16 slot | mask << 16
+  float4 centre[kBottoms];           // opened bottom nodes: geometric centre, half a cell,
+  uint32_t bottom[3][kBottoms];      // index, O (two words)
 };
 
-// dy, dz and h = fma(dz, dz, dy * dy) of the lane's targets to a record, the
-// shared part of the opening test's distance (fixed rounding: d2 = fma(dx,
-// dx, h)).
-__device__ __forceinline__ float dyz_part(float ty, float tz, u64 q1, float &dy, float &dz) {
-  float py, pz;
-  upk(q1, py, pz);
-  dy = __fsub_rn(ty, py);
-  dz = __fsub_rn(tz, pz);
-  return __fmaf_rn(dz, dz, __fmul_rn(dy, dy));
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
-// The terms of an accepted node for one pair: M/d, or with the quadrupole
-// record w rinv (M + (d^T Q d / 2) rinv^4); qu = Qxy dy + Qxz dz and qc =
-// dy (Qyy/2 dy + Qyz dz) + Qzz/2 dz^2 are shared by all pairs of the lane.
+// Per-lane state of the evaluation: the lane's 8 targets as four x pairs, pair
+// 2 r + k: row r (y = 2 (sub-brick & 1) + r), x = 2 k, 2 k + 1.
+template <bool COUNTS>
+struct Lane {
+  u64 sum[4], comp[4];    // compensated pair sums
+  int na[COUNTS ? 8 : 1], nb[COUNTS ? 8 : 1];  // accepted nodes, opened bottom nodes
+};
+
+// 1/sqrt(d) if m has the bit, else 0.
+__device__ __forceinline__ float rsqrt_if(float d, uint32_t m, uint32_t bit) {
+  float r;
+  asm("{\n.reg .pred p;\n.reg .b32 t;\nand.b32 t, %2, %3;\nsetp.ne.b32 p, t, 0;\n"
+      "mov.f32 %0, 0f00000000;\n@p rsqrt.approx.ftz.f32 %0, %1;\n}"
+      : "=f"(r)
+      : "f"(d), "r"(m), "r"(bit));
+  return r;
+}
+
+// 1/sqrt(d) if d > least, else 0.
+__device__ __forceinline__ float rsqrt_above(float d, float least) {
+  float r;
+  asm("{\n.reg .pred p;\nsetp.gt.f32 p, %1, %2;\nmov.f32 %0, 0f00000000;\n"
+      "@p rsqrt.approx.ftz.f32 %0, %1;\n}"
+      : "=f"(r)
+      : "f"(d), "f"(least));
+  return r;
+}
+
+// Compensated sums of products.  One: s = fl(sum + a b), err = fl((sum - s) +
+// a b); two: s = the sum with both added in turn, err = ((sum - s) + a1 b1) +
+// a0 b0, the products unrounded in both (sum - s is exact while the sum is
+// the larger; all terms are positive).  4 and 6 operations; rounding the
+// products and compensating each (accumulate2) takes 5 and 10, with the same
+// error against binary64 (2.76e-8 of the potential on 32^3 cells at theta
+// 0.5; 2.77e-8 with the two-product form; rounding the result alone gives
+// 2.5e-8).
+template <bool KAHAN>
+__device__ __forceinline__ void accumulate_product2(u64 &sum, u64 &comp, u64 a, u64 b) {
+  const u64 s = fma2(a, b, sum);
+  if (KAHAN) comp = add2(comp, fma2(a, b, sub2(sum, s)));
+  sum = s;
+}
+template <bool KAHAN>
+__device__ __forceinline__ void accumulate_products2(u64 &sum, u64 &comp, u64 a0, u64 b0, u64 a1,
+                                                     u64 b1) {
+  const u64 s = fma2(a1, b1, fma2(a0, b0, sum));
+  if (KAHAN) comp = add2(comp, fma2(a0, b0, fma2(a1, b1, sub2(sum, s))));
+  sum = s;
+}
+
+struct Targets {          // of one lane, read back before every evaluation
+  u64 tx[2];              // {x0, x1}, {x2, x3}
+  float ty[2], tz;
+};
+
+// A list entry as a lane evaluates it: the staged record (mass and x pairs
+// duplicated for the packed operations) and the parts shared by a row.
 template <bool QUAD>
-__device__ __forceinline__ u64 node_term2(u64 mm, u64 rr, u64 dx2, u64 w0, float qu, float qc) {
-  if (!QUAD) return mul2(mm, rr);
-  const u64 hq = fma2(dx2, fma2(w0, dx2, pk(qu, qu)), pk(qc, qc));
-  const u64 r2 = mul2(rr, rr);
-  return mul2(rr, fma2(hq, mul2(r2, r2), mm));
+struct Entry {
+  u64 dx[2], mm;       // {x0, x1} - px, {x2, x3} - px; {m, m}
+  float py, dz;
+  float4 q;            // Qxx/2, Qyy/2, Qzz/2, Qxy
+  float2 q2;           // Qxz, Qyz
+  uint32_t m8;         // bit 4 r + x: target x of row r takes part
+  float h, qu, qc;     // of the current row
+
+  __device__ __forceinline__ void load(const WalkMem<QUAD> &S, uint32_t v, int zsh,
+                                       const Targets &T) {
+    const char *at = reinterpret_cast<const char *>(S.node) + (v & 0xffffu);
+    const float4 n = *reinterpret_cast<const float4 *>(at);
+    if (QUAD) {
+      q = *reinterpret_cast<const float4 *>(reinterpret_cast<const char *>(S.quad) + (v & 0xffffu));
+      q2 = *reinterpret_cast<const float2 *>(reinterpret_cast<const char *>(S.quad2) + (v & 0xffffu));
+    }
+    m8 = v >> zsh;
+    const u64 px = pk(n.x, n.x);
+    dx[0] = sub2(T.tx[0], px);
+    dx[1] = sub2(T.tx[1], px);
+    mm = pk(n.w, n.w);
+    py = n.y;
+    dz = __fsub_rn(T.tz, n.z);
+  }
+  __device__ __forceinline__ void row(float ty) {
+    const float dy = __fsub_rn(ty, py);
+    h = __fmaf_rn(dz, dz, __fmul_rn(dy, dy));
+    if (QUAD) {  // d^T Q d / 2 = dx (Qxx/2 dx + qu) + qc
+      qu = __fmaf_rn(q2.x, dz, __fmul_rn(q.w, dy));
+      const float v = __fmaf_rn(q.y, dy, __fmul_rn(q2.y, dz));
+      qc = __fmaf_rn(dy, v, __fmul_rn(__fmul_rn(q.z, dz), dz));
+    }
+  }
+  // The terms of targets 2 k, 2 k + 1 of row r as products rr t.
+  __device__ __forceinline__ void terms(int r, int k, u64 &rr, u64 &t) const {
+    float da, db;
+    upk(fma2(dx[k], dx[k], pk(h, h)), da, db);
+    rr = pk(rsqrt_if(da, m8, 1u << (4 * r + 2 * k)), rsqrt_if(db, m8, 2u << (4 * r + 2 * k)));
+    t = mm;
+    if (QUAD) {  // M rinv + (d^T Q d / 2) rinv^5
+      const u64 hq = fma2(dx[k], fma2(pk(q.x, q.x), dx[k], pk(qu, qu)), pk(qc, qc));
+      const u64 r2 = mul2(rr, rr);
+      t = fma2(hq, mul2(r2, r2), mm);
+    }
+  }
+};
+
+// 8 entries of every sub-brick's list from ring position `at` (a multiple of
+// 8): the lane takes entries par and par + 4.
+template <bool KAHAN, bool COUNTS, bool QUAD>
+__device__ __forceinline__ void eval_nodes(const WalkMem<QUAD> &S, int sb, unsigned at, int par,
+                                           int zsh, const Targets &T, Lane<COUNTS> &L) {
+  const uint32_t *list = &S.list[sb][(at & (kRing - 1)) + par];
+  const uint32_t v0 = list[0], v1 = list[4];
+  if (COUNTS) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) L.na[i] += ((v0 >> (zsh + i)) & 1u) + ((v1 >> (zsh + i)) & 1u);
+    return;
+  }
+  Entry<QUAD> a, b;
+  if (QUAD) {  // one after the other: together they would take more than 80 registers
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      a.load(S, e ? v1 : v0, zsh, T);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        a.row(T.ty[r]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          u64 rr, t;
+          a.terms(r, k, rr, t);
+          accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], rr, t);
+        }
+      }
+    }
+    return;
+  }
+  a.load(S, v0, zsh, T);
+  b.load(S, v1, zsh, T);
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    a.row(T.ty[r]);
+    b.row(T.ty[r]);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      u64 ra, ta, rb, tb;
+      a.terms(r, k, ra, ta);
+      b.terms(r, k, rb, tb);
+      accumulate_products2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], ra, ta, rb, tb);
+    }
+  }
 }
 
-// The shared parts of a node's quadrupole term from its record (loaded with
-// the node's walk record at the start of the step, so that its latency
-// overlaps the opening test; w0 = {Qxx/2, Qxx/2}, w1 = {Qyy/2, Qzz/2},
-// w2 = {Qxy, Qxz}, w3 = {Qyz, 0}).
-__device__ __forceinline__ void quad_parts(u64 v0, u64 w1, u64 w2, u64 w3, float dy, float dz,
-                                           u64 &w0, float &qu, float &qc) {
-  w0 = v0;
-  float hyy, hzz, qxy, qxz, qyz, unused;
-  upk(w1, hyy, hzz);
-  upk(w2, qxy, qxz);
-  upk(w3, qyz, unused);
-  qu = __fmaf_rn(qxz, dz, __fmul_rn(qxy, dy));
-  const float v = __fmaf_rn(hyy, dy, __fmul_rn(qyz, dz));
-  qc = __fmaf_rn(dy, v, __fmul_rn(__fmul_rn(hzz, dz), dz));
+// TwoSum (Knuth): s + e = a + b exactly.
+__device__ __forceinline__ u64 two_sum2(u64 a, u64 b, u64 &e) {
+  const u64 s = add2(a, b), bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+  return s;
 }
 
-// The 8 cells of a bottom node (node + 1 .. node + 8) for the targets that
-// opened it (oa[k] for target a of pair k, ob[k] for target b; kept as
-// predicates, not packed into a bit mask, which took a few more instructions
-// a step): every cell but the target's own (d2 > 0).
-// Cells 2j and 2j + 1 are x-neighbours with the same y and z, so they share
-// dy, dz and h too.  The 8 positive cell terms are summed plainly (a
-// relative error of at most 7 units in the last place of their sum) and the
-// sum joins the compensated total once.  (A second form of this loop for
-// bottom nodes that hold none of the warp's targets, the openers' mask a
-// factor on the mass instead of a compare and select per cell, took 8 more
-// registers and made the walk slower.)
-template <int NP, bool KAHAN, bool COUNTS>
-__device__ __forceinline__ void bottom_cells(unsigned node, const bool (&oa)[NP],
-                                             const bool (&ob)[NP],
-                                             const WalkRec *__restrict__ rec, float ty,
-                                             float tz, Lanes<NP> &L) {
-  u64 part[NP];
+// The cells of the n opened bottom nodes.  Here a lane serves one row of four
+// targets (row = lane & 15: y = 2 (row >> 2 & 1) + (row & 1), z = 2 (row >> 3)
+// + (row >> 1 & 1)) and four cells of a bottom node (lane >> 4: its z half),
+// and walks through the bottom nodes that a target of its row opened: few
+// targets open a bottom node (19 % of the octant's 64, 32 % of a sub-brick's
+// 16, 56 % of a row's 4 at theta 0.75), and one costs 8 interactions each.
+// Every cell but the target's own (d2 > 0); a node's four terms are added
+// plainly and join a compensated sum, which joins the lanes' totals at the end.
+template <bool KAHAN, bool COUNTS, bool QUAD>
+__device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
+                                           const float4 *__restrict__ cmass, int n, int lane,
+                                           Lane<COUNTS> &L) {
+  constexpr int W = kBottoms / 32;
+  const int row = lane & 15, word = 1 + (row >> 3), sh = 4 * (row & 7), zhalf = lane >> 4;
+  uint32_t mine[W];  // bottom nodes some target of the row opened
 #pragma unroll
-  for (int k = 0; k < NP; ++k) part[k] = 0ull;
-#pragma unroll 1
-  for (unsigned c = node + 1; c < node + 9u; c += 2) {
-    u64 c0, c1, c2, c3, e0, e1, e2, e3;
-    load_rec(rec + c, c0, c1, c2, c3);
-    load_rec(rec + c + 1, e0, e1, e2, e3);
-    float dy, dz;
-    const float h = dyz_part(ty, tz, c1, dy, dz);
+  for (int w = 0; w < W; ++w) {
+    const int j = 32 * w + lane;
+    const uint32_t lo = j < n ? S.bottom[1][j] : 0u, hi = j < n ? S.bottom[2][j] : 0u;
+    mine[w] = 0u;
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const u64 px = j ? e0 : c0, mm = j ? e2 : c2;
-#pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        const u64 dx2 = sub2(L.tx2[k], px);
-        float e2a, e2b;
-        upk(fma2(dx2, dx2, pk(h, h)), e2a, e2b);
-        const bool la = oa[k] && e2a > 0.0f;
-        const bool lb = ob[k] && e2b > 0.0f;
-        if (COUNTS) {
-          L.ni[2 * k] += la;
-          L.ni[2 * k + 1] += lb;
-          L.nl[2 * k] += la;
-          L.nl[2 * k + 1] += lb;
-        } else {
-          float ra = rsqrt_approx(e2a), rb = rsqrt_approx(e2b);
-          ra = la ? ra : 0.0f;
-          rb = lb ? rb : 0.0f;
-          part[k] = fma2(mm, pk(ra, rb), part[k]);
-        }
-      }
+    for (int r = 0; r < 16; ++r) {
+      const unsigned b = __ballot_sync(kFull, (((r < 8 ? lo : hi) >> (4 * (r & 7))) & 15u) != 0u);
+      if (row == r) mine[w] = b;
     }
   }
-  if (!COUNTS) {
+  int left = 0;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) accumulate2<KAHAN>(L.sum[k], L.comp[k], part[k]);
-  }
-}
-
-// Walk of one target group (unit u = (8 / NP) * sorted block + group; group
-// g covers octants NP g .. NP g + NP - 1).
-//
-// Two modes.  While every target of the warp is at the same node (all `next`
-// equal: "converged", as at the root), a step needs no per-target
-// bookkeeping: each target still applies its own test, and one vote tells
-// whether all accepted (add the terms, continue at skip), all opened
-// (continue at node + 1) or they differ.  Where they differ, the targets
-// part, and the subtree of that node is walked per target ("diverged").
-// There a target takes part in the step at `node` when its `next` <= node
-// (`next` is kept lazily: it only moves ahead of the warp when the target
-// accepts a node that another target opens); the warp goes on at node + 1
-// when some taking-part target opened the node, else at its skip index --
-// which is the smallest next of all targets, as the recursive walk requires.
-// Every target leaves a subtree at its skip index, so they all meet again at
-// the end of the parted subtree, and the warp is converged once more.  Both
-// modes take exactly the per-target decisions of the recursive definition;
-// they differ only in the bookkeeping.
-//
-// Bottom nodes (whose 8 children are cells, stored right after them, so
-// skip = node + 9) are taken in one step: the targets that open such a node
-// interact with its 8 cells in an unrolled loop that needs no per-cell
-// bookkeeping (cells are never opened), and every target then continues at
-// node + 9.  Cells are only reached through their bottom node, so the walk
-// never stops at a cell.
-template <int NP, bool KAHAN, bool COUNTS, bool QUAD>
-__device__ __forceinline__ void walk_group(unsigned u, int lane, const WalkRec *__restrict__ rec,
-                                           const WalkQuad *__restrict__ qrec,
-                                           const int4 *__restrict__ blk,
-                                           const int *__restrict__ orig,
-                                           const int4 *__restrict__ fld,
-                                           const double *__restrict__ invL,
-                                           const unsigned long long *__restrict__ mmax, double G,
-                                           float *__restrict__ out, int32_t *__restrict__ n_int,
-                                           int32_t *__restrict__ n_test,
-                                           int32_t *__restrict__ n_leaf) {
-  constexpr unsigned kGroups = 8 / NP;                // groups per block
-  const unsigned p = u / kGroups;                     // sorted block
-  const int4 F = fld[p];                              // this field's node range
-  const unsigned n_nodes = (unsigned)F.y;
-  const int o = (int)(u % kGroups) * NP;              // octant of pair 0
-  const int ma = (o << 6) | (lane << 1);              // local Morton index, even: x bit 0
-  const int4 B = blk[p];
-  const int cx = (int)compact3(ma), cy = (int)compact3(ma >> 1), cz = (int)compact3(ma >> 2);
-  const int lc = B.x + 3;
-  // cell centres in box units, exact in binary32: (2 i + 1) * 2^-(lc+1)
-  const float hh = pow2f(-(lc + 1));
-  const float ty = __fmul_rn((float)(2 * (8 * B.z + cy) + 1), hh);
-  const float tz = __fmul_rn((float)(2 * (8 * B.w + cz) + 1), hh);
-  Lanes<NP> L;
+  for (int w = 0; w < W; ++w) left += __popc(mine[w]);
+  const int steps = (int)__reduce_max_sync(kFull, (unsigned)left);
+  u64 sum[2] = {0ull, 0ull}, comp[2] = {0ull, 0ull};
+  int nb[4] = {0, 0, 0, 0};
+  const u64 tx[2] = {pk(S.front.tx[0].x, S.front.tx[0].z), pk(S.front.tx[1].x, S.front.tx[1].z)};
+  const float ty = S.front.coord(16 + 2 * ((row >> 2) & 1) + (row & 1));
+  const float tz = S.front.coord(8 + 4 * (row >> 3) + (row & 2));
+#pragma unroll 2
+  for (int it = 0; it < steps; ++it) {
+    int j = 0;  // the next of the row's bottom nodes (none left: node 0 with an empty mask)
+    const bool any = it < left;
 #pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    const int ix = 8 * B.y + cx + 4 * k;
-    L.tx2[k] = pk(__fmul_rn((float)(2 * ix + 1), hh), __fmul_rn((float)(2 * ix + 3), hh));
-    L.sum[k] = 0ull;  // (+0.0f, +0.0f)
-    L.comp[k] = 0ull;
-    L.ni[2 * k] = L.ni[2 * k + 1] = L.nt[2 * k] = L.nt[2 * k + 1] = 0;
-    L.nl[2 * k] = L.nl[2 * k + 1] = 0;
-  }
-
-  unsigned node = (unsigned)F.x;  // the field's root
-  while (node < n_nodes) {
-    // ---- converged: every target is at `node`, an internal node ----
-    u64 q0, q1, q2, q3;
-    load_rec(rec + node, q0, q1, q2, q3);
-    u64 p0 = 0ull, p1 = 0ull, p2 = 0ull, p3 = 0ull;
-    if (QUAD && !COUNTS) load_quad(qrec + node, p0, p1, p2, p3);
-    float s2, skf;
-    upk(q3, s2, skf);
-    const unsigned skip = __float_as_uint(skf);
-    float dy, dz;
-    const float h = dyz_part(ty, tz, q1, dy, dz);
-    u64 dx2[NP];
-    float d2a[NP], d2b[NP];
-    bool ta[NP], tb[NP];
-    bool all = true, any = false;
+    for (int w = W - 1; w >= 0; --w) j = mine[w] ? 32 * w + __ffs((int)mine[w]) - 1 : j;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      dx2[k] = sub2(L.tx2[k], q0);
-      upk(fma2(dx2[k], dx2[k], pk(h, h)), d2a[k], d2b[k]);
-      ta[k] = d2a[k] > s2;
-      tb[k] = d2b[k] > s2;
-      all = all && ta[k] && tb[k];
-      any = any || ta[k] || tb[k];
-      if (COUNTS) {
-        ++L.nt[2 * k];
-        ++L.nt[2 * k + 1];
-        L.ni[2 * k] += ta[k];
-        L.ni[2 * k + 1] += tb[k];
-      }
+    for (int w = 0, done = 0; w < W; ++w) {
+      const uint32_t m = mine[w];
+      mine[w] = done ? m : m & (m - 1u);
+      done = done || m != 0u;
     }
-    u64 w0 = 0ull;
-    float qu = 0.0f, qc = 0.0f;
-    if (__all_sync(kFull, all)) {  // every target accepts the node
-      if (!COUNTS) {
-        if (QUAD) quad_parts(p0, p1, p2, p3, dy, dz, w0, qu, qc);
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-          const u64 rr = pk(rsqrt_approx(d2a[k]), rsqrt_approx(d2b[k]));
-          accumulate2<KAHAN>(L.sum[k], L.comp[k], node_term2<QUAD>(q2, rr, dx2[k], w0, qu, qc));
-        }
-      }
-      node = skip;
-      continue;
-    }
-    const bool any_take = __any_sync(kFull, any);
-    if (!COUNTS && any_take) {
-      if (QUAD) quad_parts(p0, p1, p2, p3, dy, dz, w0, qu, qc);
-#pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        float ra = rsqrt_approx(d2a[k]), rb = rsqrt_approx(d2b[k]);
-        ra = ta[k] ? ra : 0.0f;
-        rb = tb[k] ? rb : 0.0f;
-        accumulate2<KAHAN>(L.sum[k], L.comp[k],
-                           node_term2<QUAD>(q2, pk(ra, rb), dx2[k], w0, qu, qc));
-      }
-    }
-    if (skip == node + 9u) {  // bottom node: the openers meet its cells; all go on at skip
-      bool oa[NP], ob[NP];
-#pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        oa[k] = !ta[k];
-        ob[k] = !tb[k];
-      }
-      bottom_cells<NP, KAHAN, COUNTS>(node, oa, ob, rec, ty, tz, L);
-      node = skip;
-      continue;
-    }
-    if (!any_take) {  // every target opens the node
-      node = node + 1;
-      continue;
-    }
-    // ---- diverged: the targets part inside the subtree [node + 1, end) ----
-    const unsigned end = skip;
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      L.next_a[k] = ta[k] ? skip : node + 1;
-      L.next_b[k] = tb[k] ? skip : node + 1;
-    }
-    node = node + 1;  // some target opened the node
-    while (node < end) {
-      load_rec(rec + node, q0, q1, q2, q3);
-      if (QUAD && !COUNTS) load_quad(qrec + node, p0, p1, p2, p3);
-      upk(q3, s2, skf);
-      const unsigned skp = __float_as_uint(skf);
-      const float hd = dyz_part(ty, tz, q1, dy, dz);
-      bool ma_[NP], mb_[NP];
-      bool oa[NP], ob[NP];
-      bool any_tk = false, any_op = false;
-#pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        dx2[k] = sub2(L.tx2[k], q0);
-        upk(fma2(dx2[k], dx2[k], pk(hd, hd)), d2a[k], d2b[k]);
-        ma_[k] = L.next_a[k] <= node;
-        mb_[k] = L.next_b[k] <= node;
-        ta[k] = ma_[k] && d2a[k] > s2;
-        tb[k] = mb_[k] && d2b[k] > s2;
-        oa[k] = ma_[k] && !ta[k];
-        ob[k] = mb_[k] && !tb[k];
-        any_op = any_op || oa[k] || ob[k];
-        any_tk = any_tk || ta[k] || tb[k];
-        if (COUNTS) {  // internal: cells are only reached through bottom nodes
-          L.ni[2 * k] += ta[k];
-          L.ni[2 * k + 1] += tb[k];
-          L.nt[2 * k] += ma_[k];
-          L.nt[2 * k + 1] += mb_[k];
-        }
-      }
-      if (!COUNTS && __any_sync(kFull, any_tk)) {
-        if (QUAD) quad_parts(p0, p1, p2, p3, dy, dz, w0, qu, qc);
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-          float ra = rsqrt_approx(d2a[k]), rb = rsqrt_approx(d2b[k]);
-          ra = ta[k] ? ra : 0.0f;
-          rb = tb[k] ? rb : 0.0f;
-          accumulate2<KAHAN>(L.sum[k], L.comp[k],
-                             node_term2<QUAD>(q2, pk(ra, rb), dx2[k], w0, qu, qc));
-        }
-      }
-      const bool opened = __any_sync(kFull, any_op);
-      if (skp == node + 9u) {  // bottom node: all go on at skip
-        if (opened) bottom_cells<NP, KAHAN, COUNTS>(node, oa, ob, rec, ty, tz, L);
-        node = skp;
-      } else if (opened) {  // takers of a node others open move ahead of the warp
-#pragma unroll
-        for (int k = 0; k < NP; ++k) {
-          L.next_a[k] = ta[k] ? skp : L.next_a[k];
-          L.next_b[k] = tb[k] ? skp : L.next_b[k];
-        }
-        node = node + 1;
-      } else {
-        node = skp;
-      }
-    }
-    node = end;  // every target leaves the subtree at its skip index
-  }
-#pragma unroll
-  for (int k = 0; k < NP; ++k) {
-    const int64_t cell = (int64_t)orig[p] * kCellsPerBlock + cz * 64 + cy * 8 + cx + 4 * k;
+    const uint32_t m4 = any ? S.bottom[word][j] >> sh : 0u;
     if (COUNTS) {
-      n_int[cell] = L.ni[2 * k];
-      n_int[cell + 1] = L.ni[2 * k + 1];
-      n_test[cell] = L.nt[2 * k];
-      n_test[cell + 1] = L.nt[2 * k + 1];
-      if (n_leaf) {
-        n_leaf[cell] = L.nl[2 * k];
-        n_leaf[cell + 1] = L.nl[2 * k + 1];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) nb[i] += (m4 >> i) & 1u;
+      continue;
+    }
+    // masses of the cells (x0, y0), (x1, y0), (x0, y1), (x1, y1) of the lane's z
+    const float4 m = __ldg(cmass + 2 * (size_t)S.bottom[0][j] + zhalf);
+    const float4 c = S.centre[j];
+    float least[4];  // a target takes part where d2 > least: 0, or never
+#pragma unroll
+    for (int i = 0; i < 4; ++i) least[i] = (m4 & (1u << i)) ? 0.0f : __int_as_float(0x7f800000);
+    const float dz = __fsub_rn(tz, zhalf ? __fadd_rn(c.z, c.w) : __fsub_rn(c.z, c.w));
+    const float dzz = __fmul_rn(dz, dz);
+    const float xl = __fsub_rn(c.x, c.w), xh = __fadd_rn(c.x, c.w);
+    const u64 dx[2][2] = {{sub2(tx[0], pk(xl, xl)), sub2(tx[1], pk(xl, xl))},
+                          {sub2(tx[0], pk(xh, xh)), sub2(tx[1], pk(xh, xh))}};
+    u64 part[2] = {0ull, 0ull};
+#pragma unroll
+    for (int y = 0; y < 2; ++y) {
+      const float dy = __fsub_rn(ty, y ? __fadd_rn(c.y, c.w) : __fsub_rn(c.y, c.w));
+      const float h = __fmaf_rn(dy, dy, dzz);
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        const float mc = y ? (x ? m.w : m.z) : (x ? m.y : m.x);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          float da, db;
+          upk(fma2(dx[x][k], dx[x][k], pk(h, h)), da, db);
+          part[k] = fma2(pk(mc, mc), pk(rsqrt_above(da, least[2 * k]), rsqrt_above(db, least[2 * k + 1])),
+                         part[k]);
+        }
       }
+    }
+    accumulate2<KAHAN>(sum[0], comp[0], part[0]);
+    accumulate2<KAHAN>(sum[1], comp[1], part[1]);
+  }
+  // to the lanes that own the targets: rows 2 (lane >> 2) and the next; the
+  // two z halves are added, one lane of the four that share the targets takes them
+  const int from = 2 * (lane >> 2);
+  if (COUNTS) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) L.nb[i] += __shfl_sync(kFull, nb[i & 3], from + (i >> 2));
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    u64 e = 0ull;
+    const u64 o = __shfl_xor_sync(kFull, sum[k], 16);
+    if (KAHAN) {
+      sum[k] = (lane & 16) ? two_sum2(o, sum[k], e) : two_sum2(sum[k], o, e);
+      comp[k] = add2(add2(comp[k], __shfl_xor_sync(kFull, comp[k], 16)), e);
     } else {
-      u64 sm = L.sum[k];
-      sm = finish2<KAHAN>(sm, L.comp[k]);
-      float sa, sb;
-      upk(sm, sa, sb);
-      // -G/L times the field's binary32 mass unit 2^e (exact), rounded once
-      const float scale = (float)(-G * invL[F.w] * pow2i(mass_exponent(mmax[F.w])));
-      out[cell] = __fmul_rn(sa, scale);
-      out[cell + 1] = __fmul_rn(sb, scale);
+      sum[k] = add2(sum[k], o);
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const u64 v = __shfl_sync(kFull, sum[k], from + r);
+      const u64 c = KAHAN ? __shfl_sync(kFull, comp[k], from + r) : 0ull;
+      if ((lane & 3) == 0) {
+        if (KAHAN) {
+          L.sum[2 * r + k] = two_sum2(L.sum[2 * r + k], v, e);
+          L.comp[2 * r + k] = add2(add2(L.comp[2 * r + k], c), e);
+        } else {
+          L.sum[2 * r + k] = add2(L.sum[2 * r + k], v);
+        }
+      }
     }
   }
 }
 
-// One warp per target group (8 / NP groups per block), group order[warp] when
-// an order is given.  (Schedules that keep an SM's warps on neighbouring
-// octants -- SM- or CTA-affine ranges with stealing -- share more of the near
-// field in L1 but ran 2-8 % slower on GB300.)
-template <int NP, bool KAHAN, bool COUNTS, bool QUAD>
-__global__ void __launch_bounds__(kMaxWalkThreads)
-    k_walk_pair(unsigned nunits, const unsigned *__restrict__ order,
-                const WalkRec *__restrict__ rec,
-                const WalkQuad *__restrict__ qrec, const int4 *__restrict__ blk,
-                const int *__restrict__ orig, const int4 *__restrict__ fld,
-                const double *__restrict__ invL, const unsigned long long *__restrict__ mmax,
-                double G, float *__restrict__ out, int32_t *__restrict__ n_int,
-                int32_t *__restrict__ n_test, int32_t *__restrict__ n_leaf) {
+// The sums of the four lanes that share the targets (lane bits 0 and 1).
+template <bool KAHAN>
+__device__ __forceinline__ void merge_lanes(u64 &sum, u64 &comp) {
+#pragma unroll
+  for (int o = 1; o <= 2; o <<= 1) {
+    const u64 v = __shfl_xor_sync(kFull, sum, o);
+    if (KAHAN) {
+      u64 e;  // (exact, so both lanes of a pair get the same)
+      sum = (threadIdx.x & o) ? two_sum2(v, sum, e) : two_sum2(sum, v, e);
+      comp = add2(add2(comp, __shfl_xor_sync(kFull, comp, o)), e);
+    } else {
+      sum = add2(sum, v);
+    }
+  }
+}
+
+struct WalkArgs {
+  const WalkRec *rec;           // (the root's only)
+  SibArgs sib;
+  const int4 *blk;
+  const int *orig;
+  const int4 *fld;
+  const double *invL;
+  const unsigned long long *mmax;
+  double G;
+  float *out;
+  int32_t *n_int, *n_test, *n_leaf;
+  const int *flev;              // deepest block level per field
+};
+
+// Walk of octant u & 7 of sorted block u >> 3.
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+__device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> &S,
+                                            const WalkArgs &A) {
+  const unsigned p = u >> 3;
+  const int o = (int)(u & 7);
+  const int4 B = A.blk[p], F = A.fld[p];
+  const int par = lane & 3, zl = (lane >> 2) & 1, sb = lane >> 3;
+  const unsigned lower = (1u << lane) - 1u;
+  front_start(S.front, octant_at(B, o), F, p, lane, A.rec, A.sib.tops);
+  Lane<COUNTS> L;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) L.sum[i] = L.comp[i] = 0ull;
+#pragma unroll
+  for (int i = 0; i < (COUNTS ? 8 : 1); ++i) L.na[i] = L.nb[i] = 0;
+  const int zsh = 16 + 8 * zl;
+
+  // warp-uniform: stack entries; staged nodes ever and the oldest still needed;
+  // list positions (written ever per sub-brick, evaluated ever); opened bottom nodes
+  int depth = 1, nbot = 0;
+  const int pop4 = stack_pop4(A.flev[F.w]);
+  unsigned staged = 0u, oldest = 0u, head = 0u, tail[4] = {0u, 0u, 0u, 0u};
+  while (depth > 0) {
+    const Tested t = front_step<VOTE>(S.front, depth, pop4, lane, A.sib.sib);
+    const unsigned acc = __ballot_sync(kFull, (t.alo | t.ahi) != 0u);
+    if (acc) {
+      const unsigned slot = (staged + __popc(acc & lower)) & (kRing - 1);
+      if (t.alo | t.ahi) {
+        S.node[slot] = t.rec;
+        if (QUAD) {
+          copy_async<16>(&S.quad[slot], A.sib.quad + t.node);
+          copy_async<8>(&S.quad2[slot], &A.sib.quad[t.node].qxz);
+        }
+      }
+      staged += __popc(acc);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {  // to the lists of the sub-bricks with an accepting cell
+        const uint32_t w = g < 2 ? t.alo : t.ahi;
+        const uint32_t mk = (g & 1) ? (w & 0xffff0000u) : (w << 16);
+        const unsigned c = __ballot_sync(kFull, mk != 0u);
+        if (mk) S.list[g][(tail[g] + __popc(c & lower)) & (kRing - 1)] = mk | (16u * slot);
+        tail[g] += __popc(c);
+      }
+    }
+    const bool bottom = (t.olo | t.ohi) != 0u && (t.kids & kBottomBit) != 0u;
+    const unsigned bot = __ballot_sync(kFull, bottom);
+    if (bot) {
+      const int slot = nbot + __popc(bot & lower);
+      if (bottom) {
+        S.bottom[0][slot] = t.kids & ~kBottomBit;
+        S.bottom[1][slot] = t.olo;
+        S.bottom[2][slot] = t.ohi;
+      }
+      nbot += __popc(bot);
+    }
+    __syncwarp();
+    const bool last = depth == 0;
+    if (staged - oldest > kRing - 32 || last) {
+      // Evaluate listed nodes until a further chunk's fit the ring (at the
+      // end: all).  All lists are read at the same position, 8 entries at a
+      // time: while every list has 8, and then with the short ones filled up
+      // by empty entries.
+      if (QUAD) {
+        copy_async_wait();
+        __syncwarp();
+      }
+      Targets T;
+      T.tx[0] = pk(S.front.tx[0].x, S.front.tx[0].z);
+      T.tx[1] = pk(S.front.tx[1].x, S.front.tx[1].z);
+      T.ty[0] = S.front.coord(16 + 2 * (sb & 1));
+      T.ty[1] = S.front.coord(17 + 2 * (sb & 1));
+      T.tz = S.front.coord(8 + 4 * (sb >> 1) + 2 * zl);
+      for (;;) {
+        const unsigned full = (min(min(tail[0], tail[1]), min(tail[2], tail[3])) - head) / 8u;
+        for (unsigned i = 0; i < full; ++i, head += 8u)
+          eval_nodes<KAHAN, COUNTS, QUAD>(S, sb, head, par, zsh, T, L);
+        const unsigned mine = sb < 2 ? (sb ? tail[1] : tail[0]) : (sb == 2 ? tail[2] : tail[3]);
+        // the oldest staged node still listed
+        unsigned age = staged - oldest;
+        if (mine != head) age = ((S.list[sb][head & (kRing - 1)] >> 4) - oldest) & (kRing - 1);
+        oldest += __reduce_min_sync(kFull, age);
+        if (last ? oldest == staged : staged - oldest <= kRing - 32) break;
+        if ((int)(mine - head) < 8) {  // the 8 lanes of the sub-brick: one entry each
+          const unsigned at = head + (lane & 7);
+          if ((int)(at - mine) >= 0) S.list[sb][at & (kRing - 1)] = 0u;
+        }
+#pragma unroll
+        for (int g = 0; g < 4; ++g) tail[g] = (int)(tail[g] - head) < 8 ? head + 8u : tail[g];
+        __syncwarp();
+      }
+      __syncwarp();
+    }
+    if (nbot > kBottoms - 32 || (last && nbot)) {
+      for (int j = lane; j < nbot; j += 32) S.centre[j] = bottom_centre(S.bottom[0][j], A.blk);
+      __syncwarp();
+      eval_cells<KAHAN, COUNTS, QUAD>(S, reinterpret_cast<const float4 *>(A.sib.cmass), nbot, lane,
+                                      L);
+      nbot = 0;
+      __syncwarp();
+    }
+  }
+  // each of the four lanes writes two of the shared 8 targets: row par >> 1,
+  // x = 2 (par & 1) and the next
+  const int r = par >> 1, k = par & 1;
+  const int64_t cell = (int64_t)A.orig[p] * kCellsPerBlock + (4 * (o >> 2) + 2 * (sb >> 1) + zl) * 64 +
+                       (4 * ((o >> 1) & 1) + 2 * (sb & 1) + r) * 8 + 4 * (o & 1) + 2 * k;
+  if (COUNTS) {
+    int na[2] = {0, 0}, nb[2] = {0, 0};
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      int v = L.na[i];  // every lane of the four counted the entries it took
+      v += __shfl_xor_sync(kFull, v, 1);
+      v += __shfl_xor_sync(kFull, v, 2);
+      if ((i >> 1) == par) {
+        na[i & 1] = v;
+        nb[i & 1] = L.nb[i];
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      // t tests: the root and 8 for every opened node above the bottom ones;
+      // each ends in an accepted, an opened bottom or another opened node:
+      // t = 1 + 8 (t - na - nb)
+      const int cells = 8 * nb[i] - 1;  // not its own
+      A.n_int[cell + i] = na[i] + cells;
+      A.n_test[cell + i] = (8 * (na[i] + nb[i]) - 1) / 7;
+      if (A.n_leaf) A.n_leaf[cell + i] = cells;
+    }
+  } else {
+    // -G/L times the field's binary32 mass unit 2^e (exact), rounded once
+    const float scale = (float)(-A.G * A.invL[F.w] * pow2i(mass_exponent(A.mmax[F.w])));
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      merge_lanes<KAHAN>(L.sum[i], L.comp[i]);
+      if (i == par) {
+        float sa, sb_;
+        upk(finish2<KAHAN>(L.sum[i], L.comp[i]), sa, sb_);
+        A.out[cell] = __fmul_rn(sa, scale);
+        A.out[cell + 1] = __fmul_rn(sb_, scale);
+      }
+    }
+  }
+}
+
+// A unit of work is one octant (np = 1) or two neighbouring ones, walked one
+// after the other (np = 2).  Plain grid: warp i walks unit order[i] (or i).
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+__global__ void __maxnreg__(kWalkRegs)
+    k_walk_lists(unsigned nunits, int np, const unsigned *__restrict__ order, const WalkArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  WalkMem<QUAD> &S = reinterpret_cast<WalkMem<QUAD> *>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   const unsigned warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (warp >= nunits) return;  // whole warps only
   const unsigned u = order ? order[warp] : warp;
-  walk_group<NP, KAHAN, COUNTS, QUAD>(u, lane, rec, qrec, blk, orig, fld, invL, mmax, G, out,
-                                      n_int, n_test, n_leaf);
+  for (int k = 0; k < np; ++k) walk_octant<KAHAN, COUNTS, QUAD, VOTE>(u * np + k, lane, S, A);
 }
 
 // The same walk on a persistent grid: each warp takes `per_ticket`
-// consecutive groups at a time from the work counter (one atomic add by lane
-// 0; no waiting on other warps) until every group is taken.  In the groups'
-// own order, consecutive groups are neighbouring octants; with `order` (the
-// groups sorted by the time of their walks, longest first) the long walks
+// consecutive units at a time from the work counter (one atomic add by lane
+// 0; no waiting on other warps) until every unit is taken.  In the units'
+// own order, consecutive units are neighbouring octants; with `order` (the
+// units sorted by the time of their walks, longest first) the long walks
 // start first and the short ones fill the end, so that fewer warps are left
 // running alone at the end of the launch.  cycles (or null): the SM clock
-// cycles of each group's walk, the measurement that order is made from.
-template <int NP, bool KAHAN, bool COUNTS, bool QUAD>
-__global__ void __launch_bounds__(kMaxWalkThreads)
-    k_walk_queue(unsigned nunits, unsigned per_ticket, unsigned *__restrict__ counter,
+// cycles of each unit's walk, the measurement that order is made from.
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+__global__ void __maxnreg__(kWalkRegs)
+    k_walk_queue(unsigned nunits, int np, unsigned per_ticket, unsigned *__restrict__ counter,
                  const unsigned *__restrict__ order, unsigned long long *__restrict__ cycles,
-                 const WalkRec *__restrict__ rec, const WalkQuad *__restrict__ qrec,
-                 const int4 *__restrict__ blk, const int *__restrict__ orig,
-                 const int4 *__restrict__ fld, const double *__restrict__ invL,
-                 const unsigned long long *__restrict__ mmax, double G, float *__restrict__ out,
-                 int32_t *__restrict__ n_int, int32_t *__restrict__ n_test,
-                 int32_t *__restrict__ n_leaf) {
+                 const WalkArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  WalkMem<QUAD> &S = reinterpret_cast<WalkMem<QUAD> *>(smem_raw)[threadIdx.x >> 5];
   const int lane = threadIdx.x & 31;
   for (;;) {
     unsigned u0 = 0u;
@@ -447,24 +598,27 @@ __global__ void __launch_bounds__(kMaxWalkThreads)
     for (unsigned i = u0; i < u1; ++i) {
       const unsigned u = order ? order[i] : i;
       const long long c0 = cycles ? clock64() : 0;
-      walk_group<NP, KAHAN, COUNTS, QUAD>(u, lane, rec, qrec, blk, orig, fld, invL, mmax, G, out,
-                                          n_int, n_test, n_leaf);
+      for (int k = 0; k < np; ++k) walk_octant<KAHAN, COUNTS, QUAD, VOTE>(u * np + k, lane, S, A);
       if (cycles && lane == 0) cycles[u] = (unsigned long long)(clock64() - c0);
     }
   }
 }
 
-// ---- one target per lane: binary64 interactions and/or the warp vote --------
-template <bool F64, bool VOTE, bool KAHAN, bool COUNTS, bool QUAD>
+// ---- binary64 interactions, one target per lane -------------------------------
+//
+// One warp per 32-cell brick (4x4x2, local Morton 32q .. 32q+31), as the paper
+// groups its cells (Sec. 3.1.1, Sec. 3.3).  Every target keeps `next`, the
+// first node it still has to visit; the warp takes the smallest over its
+// lanes, all lanes load that node, and the targets whose `next` equals it
+// apply the test: accepted -> next = skip, opened -> node + 1.  With the warp
+// vote all lanes share `next`.
+template <bool VOTE, bool QUAD>
 __global__ void __launch_bounds__(kWalkThreads)
     k_walk_scalar(int nbricks, const WalkRec *__restrict__ rec,
-                  const double4_32a *__restrict__ mom, const WalkQuad *__restrict__ qrec,
-                  const double *__restrict__ q64, const int4 *__restrict__ blk,
-                  const int *__restrict__ orig, const int4 *__restrict__ fld,
-                  const double *__restrict__ invL, const unsigned long long *__restrict__ mmax,
-                  double G, void *__restrict__ out,
-                  int32_t *__restrict__ n_int, int32_t *__restrict__ n_test,
-                  int32_t *__restrict__ n_leaf) {
+                  const double4_32a *__restrict__ mom, const double *__restrict__ q64,
+                  const int4 *__restrict__ blk, const int *__restrict__ orig,
+                  const int4 *__restrict__ fld, const double *__restrict__ invL, double G,
+                  double *__restrict__ out) {
   const int warp = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
   const int lane = threadIdx.x & 31;
   if (warp >= nbricks) return;  // whole warps only
@@ -473,111 +627,66 @@ __global__ void __launch_bounds__(kWalkThreads)
   const int4 B = blk[p];
   const int4 F = fld[p];        // this field's node range
   const unsigned n_nodes = (unsigned)F.y;
-  const double scale_d = -G * invL[F.w];  // FP64 walk: physical FP64 moments
-  // binary32 walk: the records' masses are in the field's unit 2^e
-  const float scale_f = (float)(scale_d * pow2i(mass_exponent(mmax[F.w])));
   const int cx = (int)compact3(m), cy = (int)compact3(m >> 1), cz = (int)compact3(m >> 2);
-  const int lc = B.x + 3;
-  const float hh = pow2f(-(lc + 1));
+  const float hh = pow2f(-(B.x + 3 + 1));
   const float tx = __fmul_rn((float)(2 * (8 * B.y + cx) + 1), hh);
   const float ty = __fmul_rn((float)(2 * (8 * B.z + cy) + 1), hh);
   const float tz = __fmul_rn((float)(2 * (8 * B.w + cz) + 1), hh);
-
-  float sum = 0.0f, comp = 0.0f;
   double sumd = 0.0;
-  int ni = 0, nt = 0, nl = 0;
   unsigned next = (unsigned)F.x;  // the field's root
   unsigned node = (unsigned)F.x;
   while (node < n_nodes) {
-    u64 q0, q1, q2, q3;
-    load_rec(rec + node, q0, q1, q2, q3);
-    float px, px2, py, pz, mf, mf2, s2, skf;
-    upk(q0, px, px2);
-    upk(q1, py, pz);
-    upk(q2, mf, mf2);
-    upk(q3, s2, skf);
-    const unsigned skip = __float_as_uint(skf);
-    const float dx = __fsub_rn(tx, px);
-    const float dy = __fsub_rn(ty, py);
-    const float dz = __fsub_rn(tz, pz);
+    const float4 a = __ldg(reinterpret_cast<const float4 *>(rec + node));
+    const float s2 = __ldg(&rec[node].s2);
+    const unsigned skip = __ldg(&rec[node].skip);
+    const float dx = __fsub_rn(tx, a.x);
+    const float dy = __fsub_rn(ty, a.y);
+    const float dz = __fsub_rn(tz, a.z);
     const float d2 = __fmaf_rn(dx, dx, __fmaf_rn(dz, dz, __fmul_rn(dy, dy)));
     const bool internal = s2 > 0.0f;
-    bool mine = true, take;
+    bool take;
     if (VOTE) {
       const bool acc = d2 > s2;
       take = internal ? (__all_sync(kFull, acc) != 0) : acc;
       next = (internal && !take) ? node + 1 : skip;
     } else {
-      mine = next == node;
+      const bool mine = next == node;
       take = mine && d2 > s2;
       next = max(next, take ? skip : node + 1);
     }
-    if (COUNTS) {
-      nt += (mine && internal) ? 1 : 0;
-      ni += take ? 1 : 0;
-      nl += (take && !internal) ? 1 : 0;
-    } else if (F64) {
-      if (take) {
-        const double4_32a md = mom[node];
-        const double ex = (double)tx - md.x, ey = (double)ty - md.y, ez = (double)tz - md.z;
-        const double dd = ex * ex + ey * ey + ez * ez;
-        const double rinv = 1.0 / sqrt(dd);
-        double t = md.w * rinv;
-        if (QUAD && internal) {
-          const double *Q = q64 + 6 * (size_t)node;
-          const double hq = 0.5 * (Q[0] * ex * ex + Q[1] * ey * ey + Q[2] * ez * ez) +
-                            Q[3] * ex * ey + Q[4] * ex * ez + Q[5] * ey * ez;
-          t += hq * rinv * rinv * rinv * rinv * rinv;
-        }
-        sumd += t;
+    if (take) {
+      const double4_32a md = mom[node];
+      const double ex = (double)tx - md.x, ey = (double)ty - md.y, ez = (double)tz - md.z;
+      const double dd = ex * ex + ey * ey + ez * ez;
+      const double rinv = 1.0 / sqrt(dd);
+      double t = md.w * rinv;
+      if (QUAD && internal) {
+        const double *Q = q64 + 6 * (size_t)node;
+        const double hq = 0.5 * (Q[0] * ex * ex + Q[1] * ey * ey + Q[2] * ez * ez) +
+                          Q[3] * ex * ey + Q[4] * ex * ez + Q[5] * ey * ez;
+        t += hq * rinv * rinv * rinv * rinv * rinv;
       }
-    } else {
-      float r = rsqrt_approx(d2);
-      r = take ? r : 0.0f;
-      float term = __fmul_rn(mf, r);
-      if (QUAD && internal) {  // cells carry no quadrupole (and have no record)
-        const WalkQuad w = qrec[node];
-        const float hq = dx * (w.hxx * dx + w.qxy * dy + w.qxz * dz) +
-                         dy * (w.hyy * dy + w.qyz * dz) + w.hzz * dz * dz;
-        const float r2 = r * r;
-        term = r * (mf + hq * r2 * r2);
-      }
-      if (KAHAN) {  // compensated as accumulate2 (bh_walk_common.cuh)
-        const float t = __fadd_rn(sum, term);
-        comp = __fadd_rn(comp, __fadd_rn(__fsub_rn(sum, t), term));
-        sum = t;
-      } else {
-        sum = __fadd_rn(sum, term);
-      }
+      sumd += t;
     }
     node = VOTE ? next : __reduce_min_sync(kFull, next);
   }
   const int64_t cell = (int64_t)orig[p] * kCellsPerBlock + cz * 64 + cy * 8 + cx;
-  if (COUNTS) {
-    n_int[cell] = ni;
-    n_test[cell] = nt;
-    if (n_leaf) n_leaf[cell] = nl;
-  } else if (F64) {
-    reinterpret_cast<double *>(out)[cell] = sumd * scale_d;
-  } else {
-    const float total = KAHAN ? __fadd_rn(sum, comp) : sum;
-    reinterpret_cast<float *>(out)[cell] = __fmul_rn(total, scale_f);
-  }
+  out[cell] = sumd * (-G * invL[F.w]);  // physical FP64 moments
 }
 
-template <int NP, bool KAHAN, bool COUNTS, bool QUAD>
-cudaError_t go_pair_np(cudaStream_t s, int nb, const WalkRec *rec, const WalkQuad *qrec,
-                       const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out,
-                       int32_t *ni, int32_t *nt, int32_t *nl, const WalkShape &shape) {
-  const unsigned nunits = (unsigned)nb * (8u / NP);
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+cudaError_t go_lists(cudaStream_t s, int nb, const WalkArgs &a, const WalkShape &shape) {
+  const int np = shape.pairs > 0 ? shape.pairs : 1;
+  const unsigned nunits = (unsigned)nb * (8u / (unsigned)np);
   const int w = shape.warps > 0 ? shape.warps : kDefaultWarps;
+  const int smem = w * (int)sizeof(WalkMem<QUAD>);
   if (shape.ticket > 0 && shape.counter) {  // persistent: the CTAs that fit at once
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-          &per_sm, k_walk_queue<NP, KAHAN, COUNTS, QUAD>, 32 * w, 0);
+          &per_sm, k_walk_queue<KAHAN, COUNTS, QUAD, VOTE>, 32 * w, smem);
     if (e != cudaSuccess) return e;
     const unsigned warps_needed = (nunits + (unsigned)shape.ticket - 1) / (unsigned)shape.ticket;
     const unsigned ctas_needed = (warps_needed + (unsigned)w - 1) / (unsigned)w;
@@ -585,94 +694,105 @@ cudaError_t go_pair_np(cudaStream_t s, int nb, const WalkRec *rec, const WalkQua
     const unsigned grid = ctas_needed < resident ? ctas_needed : resident;
     e = cudaMemsetAsync(shape.counter, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    k_walk_queue<NP, KAHAN, COUNTS, QUAD><<<grid, 32 * w, 0, s>>>(
-        nunits, (unsigned)shape.ticket, shape.counter, shape.order, shape.cycles, rec, qrec, blk,
-        orig, fa.fld, fa.invL, fa.mmax, G, (float *)out, ni, nt, nl);
+    k_walk_queue<KAHAN, COUNTS, QUAD, VOTE><<<grid, 32 * w, smem, s>>>(
+        nunits, np, (unsigned)shape.ticket, shape.counter, shape.order, shape.cycles, a);
     return cudaGetLastError();
   }
   const int grid = (int)((nunits + w - 1) / w);
-  k_walk_pair<NP, KAHAN, COUNTS, QUAD><<<grid, 32 * w, 0, s>>>(
-      nunits, shape.order, rec, qrec, blk, orig, fa.fld, fa.invL, fa.mmax, G, (float *)out, ni,
-      nt, nl);
+  k_walk_lists<KAHAN, COUNTS, QUAD, VOTE><<<grid, 32 * w, smem, s>>>(nunits, np, shape.order, a);
+  return cudaGetLastError();
+}
+
+template <bool QUAD>
+cudaError_t go_f64(cudaStream_t s, bool vote, int nb, const WalkRec *rec, const double4_32a *mom,
+                   const double *q64, const WalkArgs &a, void *out) {
+  const int nbricks = nb * 16;
+  const int grid = (nbricks + kWarpsPerCta - 1) / kWarpsPerCta;
+  if (vote)
+    k_walk_scalar<true, QUAD><<<grid, kWalkThreads, 0, s>>>(nbricks, rec, mom, q64, a.blk, a.orig,
+                                                            a.fld, a.invL, a.G, (double *)out);
+  else
+    k_walk_scalar<false, QUAD><<<grid, kWalkThreads, 0, s>>>(nbricks, rec, mom, q64, a.blk, a.orig,
+                                                             a.fld, a.invL, a.G, (double *)out);
   return cudaGetLastError();
 }
 
 template <bool KAHAN, bool COUNTS, bool QUAD>
-cudaError_t go_pair(cudaStream_t s, int nb, const WalkRec *rec, const WalkQuad *qrec,
-                    const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out,
-                    int32_t *ni, int32_t *nt, int32_t *nl, WalkShape shape) {
-  const int np = shape.pairs > 0 ? shape.pairs : kDefaultPairs;
-  if (np == 2)
-    return go_pair_np<2, KAHAN, COUNTS, QUAD>(s, nb, rec, qrec, blk, orig, fa, G, out, ni, nt, nl,
-                                              shape);
-  return go_pair_np<1, KAHAN, COUNTS, QUAD>(s, nb, rec, qrec, blk, orig, fa, G, out, ni, nt, nl,
-                                            shape);
+cudaError_t go_criterion(cudaStream_t s, bool vote, int nb, const WalkArgs &a,
+                         const WalkShape &shape) {
+  return vote ? go_lists<KAHAN, COUNTS, QUAD, true>(s, nb, a, shape)
+              : go_lists<KAHAN, COUNTS, QUAD, false>(s, nb, a, shape);
 }
 
-template <bool F64, bool VOTE, bool KAHAN, bool COUNTS, bool QUAD>
-cudaError_t go_scalar(cudaStream_t s, int nb, const WalkRec *rec, const double4_32a *mom,
-                      const WalkQuad *qrec, const double *q64, const int4 *blk,
-                      const int *orig, const FieldArgs &fa, double G, void *out, int32_t *ni,
-                      int32_t *nt, int32_t *nl) {
-  const int nbricks = nb * 16;
-  const int grid = (nbricks + kWarpsPerCta - 1) / kWarpsPerCta;
-  k_walk_scalar<F64, VOTE, KAHAN, COUNTS, QUAD><<<grid, kWalkThreads, 0, s>>>(
-      nbricks, rec, mom, qrec, q64, blk, orig, fa.fld, fa.invL, fa.mmax, G, out, ni, nt, nl);
+// CTAs of up to 16 warps take more dynamic shared memory than the default limit.
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+cudaError_t raise_smem() {
+  const int bytes = (kMaxWalkThreads / 32) * (int)sizeof(WalkMem<QUAD>);
+  cudaError_t e = cudaFuncSetAttribute(k_walk_lists<KAHAN, COUNTS, QUAD, VOTE>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_walk_queue<KAHAN, COUNTS, QUAD, VOTE>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  return e;
+}
+
+}  // namespace
+
+cudaError_t prepare_walk_kernels() {
+  cudaError_t e = raise_smem<true, false, false, false>();
+  if (e == cudaSuccess) e = raise_smem<true, false, false, true>();
+  if (e == cudaSuccess) e = raise_smem<true, false, true, false>();
+  if (e == cudaSuccess) e = raise_smem<true, false, true, true>();
+  if (e == cudaSuccess) e = raise_smem<false, false, false, false>();
+  if (e == cudaSuccess) e = raise_smem<false, false, false, true>();
+  if (e == cudaSuccess) e = raise_smem<false, false, true, false>();
+  if (e == cudaSuccess) e = raise_smem<false, false, true, true>();
+  if (e == cudaSuccess) e = raise_smem<false, true, false, false>();
+  if (e == cudaSuccess) e = raise_smem<false, true, false, true>();
+  return e;
+}
+
+cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux, WalkRec *rec,
+                              int64_t entries, WalkSib *sib, float inv_theta) {
+  const int threads = 256;
+  k_prepare_s2<<<(unsigned)((n_nodes + threads - 1) / threads), threads, 0, s>>>(n_nodes, aux, rec,
+                                                                               inv_theta);
+  k_prepare_sib_s2<<<(unsigned)((entries + threads - 1) / threads), threads, 0, s>>>(entries, sib,
+                                                                                   inv_theta);
   return cudaGetLastError();
 }
 
 // Picks the kernel instance for the options.  The counting walk takes the
 // same decisions as every walk of the same criterion (the opening test does
 // not depend on precision, summation or the quadrupole term).
-template <bool QUAD>
-cudaError_t launch_walk_q(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
-                          const double4_32a *mom, const WalkQuad *qrec, const double *q64,
-                          const int4 *blk, const int *orig, const FieldArgs &fa, double G,
-                          void *out, WalkShape shape) {
-  const bool vote = opt.criterion == BH_CRIT_WARP_VOTE;
-  if (opt.precision == BH_PREC_F64)
-    return vote ? go_scalar<true, true, false, false, QUAD>(s, nb, rec, mom, qrec, q64, blk, orig,
-                                                            fa, G, out, nullptr, nullptr, nullptr)
-                : go_scalar<true, false, false, false, QUAD>(s, nb, rec, mom, qrec, q64, blk,
-                                                             orig, fa, G, out, nullptr, nullptr,
-                                                             nullptr);
-  if (vote)
-    return opt.kahan ? go_scalar<false, true, true, false, QUAD>(s, nb, rec, mom, qrec, q64, blk,
-                                                                 orig, fa, G, out, nullptr,
-                                                                 nullptr, nullptr)
-                     : go_scalar<false, true, false, false, QUAD>(s, nb, rec, mom, qrec, q64,
-                                                                  blk, orig, fa, G, out, nullptr,
-                                                                  nullptr, nullptr);
-  return opt.kahan ? go_pair<true, false, QUAD>(s, nb, rec, qrec, blk, orig, fa, G, out, nullptr,
-                                                nullptr, nullptr, shape)
-                   : go_pair<false, false, QUAD>(s, nb, rec, qrec, blk, orig, fa, G, out,
-                                                 nullptr, nullptr, nullptr, shape);
-}
-
-}  // namespace
-
-cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux, WalkRec *rec,
-                              float inv_theta) {
-  const int threads = 256;
-  const int64_t grid = (n_nodes + threads - 1) / threads;
-  k_prepare_s2<<<(unsigned)grid, threads, 0, s>>>(n_nodes, aux, rec, inv_theta);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
-                        const double4_32a *mom, const WalkQuad *qrec, const double *q64,
-                        const int4 *blk, const int *orig, const FieldArgs &fa, double G,
-                        void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf,
-                        WalkShape shape) {
-  if (n_int)  // counting walk
-    return opt.criterion == BH_CRIT_WARP_VOTE
-               ? go_scalar<false, true, false, true, false>(s, nb, rec, mom, qrec, q64, blk, orig,
-                                                           fa, G, out, n_int, n_test, n_leaf)
-               : go_pair<false, true, false>(s, nb, rec, qrec, blk, orig, fa, G, out, n_int,
-                                             n_test, n_leaf, shape);
+                        const double4_32a *mom, const SibArgs &sib, const double *q64,
+                        const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out,
+                        int32_t *n_int, int32_t *n_test, int32_t *n_leaf, WalkShape shape) {
+  WalkArgs a;
+  a.rec = rec;
+  a.sib = sib;
+  a.blk = blk;
+  a.orig = orig;
+  a.fld = fa.fld;
+  a.invL = fa.invL;
+  a.mmax = fa.mmax;
+  a.G = G;
+  a.out = (float *)out;
+  a.n_int = n_int;
+  a.n_test = n_test;
+  a.n_leaf = n_leaf;
+  a.flev = fa.flev;
+  const bool vote = opt.criterion == BH_CRIT_WARP_VOTE;
+  if (n_int) return go_criterion<false, true, false>(s, vote, nb, a, shape);
+  if (opt.precision == BH_PREC_F64)
+    return opt.quadrupole ? go_f64<true>(s, vote, nb, rec, mom, q64, a, out)
+                          : go_f64<false>(s, vote, nb, rec, mom, q64, a, out);
   if (opt.quadrupole)
-    return launch_walk_q<true>(s, opt, nb, rec, mom, qrec, q64, blk, orig, fa, G, out, shape);
-  return launch_walk_q<false>(s, opt, nb, rec, mom, qrec, q64, blk, orig, fa, G, out, shape);
+    return opt.kahan ? go_criterion<true, false, true>(s, vote, nb, a, shape)
+                     : go_criterion<false, false, true>(s, vote, nb, a, shape);
+  return opt.kahan ? go_criterion<true, false, false>(s, vote, nb, a, shape)
+                   : go_criterion<false, false, false>(s, vote, nb, a, shape);
 }
 
 }  // namespace bhg

@@ -1,0 +1,71 @@
+"""The list walk (siblings tested eight at a time, accepted nodes and opened
+bottom nodes collected per sub-brick and row) where its stack, rings and lists
+run full or nearly empty: meshes refined about one corner (deep, ragged trees),
+small opening angles (many opened nodes per octant), one block.
+
+Bars: opening decisions equal the oracle's exactly; potentials within 1e-5 of
+the oracle's walk (the binary32 bar of the parity tests) or 1e-12 (binary64);
+a field in a batch keeps the bits of its own solve, whatever the depth of the
+others."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import oracle as O  # noqa: E402
+from paper_1509_07370_gb300 import bhgrav as B  # noqa: E402
+from paper_1509_07370_gb300 import meshgen as mg  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def corner(level, extra):
+    return mg.refined_mesh(level, level + extra, lambda lev, ijk: np.all(ijk == 0, axis=1))
+
+
+def field(level, extra, seed):
+    m = corner(level, extra)
+    rng = np.random.Generator(np.random.PCG64(seed))
+    return m, rng.lognormal(0.0, 1.5, size=(m.nblocks, 8, 8, 8)).astype(np.float32)
+
+
+CASES = [(0, 0, 0.3), (0, 4, 0.12), (1, 2, 0.25), (2, 1, 1.0), (1, 9, 0.6)]
+
+
+@pytest.mark.parametrize("level,extra,theta", CASES)
+@pytest.mark.parametrize("vote", [False, True])
+def test_decisions_and_potentials_match_oracle(level, extra, theta, vote):
+    m, rho = field(level, extra, 10 * level + extra)
+    t = O.Tree(m.level, m.ijk, rho.astype(np.float64))
+    for quad in (False, True):
+        s = B.Solver(criterion=B.BH_CRIT_WARP_VOTE if vote else B.BH_CRIT_PER_CELL,
+                     quadrupole=quad)
+        s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+        got = s.potential(theta).cpu().numpy().astype(np.float64)
+        ni, nt = (x.cpu().numpy() for x in s.walk_counts(theta))
+        if vote:  # (32 cells per brick in local Morton order)
+            got, ni, nt = (x.reshape(-1, 512)[:, O.local_morton_order()].reshape(-1)
+                           for x in (got, ni, nt))
+            want, wi, wt = t.walk_vote(theta, quad=quad)
+        else:
+            want, wi, wt = t.walk(theta, quad=quad)
+        assert np.array_equal(ni, wi) and np.array_equal(nt, wt)
+        assert np.max(np.abs(got / want - 1.0)) <= 1e-5
+
+
+@pytest.mark.parametrize("quad", [False, True])
+def test_deep_and_shallow_fields_keep_their_bits_in_a_batch(quad):
+    fs = [field(1, 14, 1), field(0, 0, 2), field(1, 1, 3), field(0, 5, 4)]
+    nb = [m.nblocks for m, _ in fs]
+    s = B.Solver(quadrupole=quad)
+    rho = torch.as_tensor(np.concatenate([r.reshape(-1) for _, r in fs])).cuda()
+    s.build_batch(nb, np.concatenate([m.level for m, _ in fs]),
+                  np.concatenate([m.ijk for m, _ in fs]), rho)
+    got = s.potential(0.4).cpu().numpy()
+    at = 0
+    for m, r in fs:
+        a = B.Solver(quadrupole=quad)
+        a.build(m.level, m.ijk, torch.as_tensor(r.reshape(-1)).cuda())
+        want = a.potential(0.4).cpu().numpy()
+        assert np.array_equal(got[at:at + want.size], want)
+        at += want.size
