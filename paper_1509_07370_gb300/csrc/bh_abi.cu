@@ -98,6 +98,9 @@ void free_nodes(bhg::Tree &t) {
   release(t.d_sib);
   release(t.d_squad);
   release(t.d_cmass);
+  release(t.d_smom);
+  release(t.d_sq64);
+  release(t.d_cmass64);
   t.sib_cap = 0;
   release(t.d_q64);
   release(t.d_qrec);
@@ -145,9 +148,14 @@ bh_status ensure_nodes(bh_ctx *ctx, int64_t n_nodes, int64_t nb) {
   BH_CUDA(bhg::dev_malloc(&t.d_lvl, n * sizeof(uint8_t)));
   t.node_cap = n_nodes;
   BH_CUDA(bhg::dev_malloc(&t.d_sib, (size_t)entries * sizeof(bhg::WalkSib)));
-  if (ctx->opt.quadrupole)
+  if (ctx->opt.quadrupole && !quad64)
     BH_CUDA(bhg::dev_malloc(&t.d_squad, (size_t)entries * sizeof(bhg::WalkQuad)));
   BH_CUDA(bhg::dev_malloc(&t.d_cmass, (size_t)nb * bhg::kCellsPerBlock * sizeof(float)));
+  if (ctx->opt.precision == BH_PREC_F64) {
+    BH_CUDA(bhg::dev_malloc(&t.d_smom, (size_t)entries * sizeof(double4_32a)));
+    if (quad64) BH_CUDA(bhg::dev_malloc(&t.d_sq64, (size_t)entries * 6 * sizeof(double)));
+    BH_CUDA(bhg::dev_malloc(&t.d_cmass64, (size_t)nb * bhg::kCellsPerBlock * sizeof(double)));
+  }
   t.sib_cap = entries;
   return BH_OK;
 }
@@ -236,6 +244,9 @@ bhg::SibArgs sib_args(const bhg::Tree &t) {
   a.sib = t.d_sib;
   a.quad = t.d_squad;
   a.cmass = t.d_cmass;
+  a.mom = t.d_smom;
+  a.q64 = t.d_sq64;
+  a.cmass64 = t.d_cmass64;
   a.tops = (int64_t)bhg::kSibsPerBlock * t.nb;
   a.slots = t.nb / 7 + 1;
   return a;
@@ -529,8 +540,8 @@ static cudaError_t enqueue_walk(bh_ctx *ctx, cudaStream_t s, double G, void *out
     shape.order = (shape.longest && np <= 2 && t.order_n[np - 1] == groups) ? t.d_order[np - 1]
                                                                              : nullptr;
   }
-  return bhg::launch_walk(s, ctx->opt, t.nb, t.d_rec, t.d_mom, sib_args(t), t.d_q64, t.d_blk,
-                          t.d_orig, field_args(t), G, out, n_int, n_test, n_leaf, shape);
+  return bhg::launch_walk(s, ctx->opt, t.nb, t.d_rec, sib_args(t), t.d_blk, t.d_orig,
+                          field_args(t), G, out, n_int, n_test, n_leaf, shape);
 }
 
 bh_status bh_create(bh_ctx **out, const bh_options *opt, int device, void *cuda_stream) {
@@ -1141,8 +1152,10 @@ bh_status bh_stats(const bh_ctx *ctx, bh_stats_t *out) {
   // pos, fld, and 8 bytes of top-node child lists
   int64_t b = t.nb_cap * (int64_t)(4 + 12 + 8 + 8 + 4 + 4 + 4 + 4 + 16 + 4 + 4 + 4 + 16 + 8);
   b += t.node_cap * (int64_t)(sizeof(double4_32a) + sizeof(bhg::WalkRec) + sizeof(float2) + 1);
-  b += t.sib_cap * (int64_t)(sizeof(bhg::WalkSib) + (t.d_squad ? sizeof(bhg::WalkQuad) : 0));
-  if (t.d_cmass) b += t.sib_cap / bhg::kSibsPerBlock * bhg::kCellsPerBlock * (int64_t)sizeof(float);
+  b += t.sib_cap * (int64_t)(sizeof(bhg::WalkSib) + (t.d_squad ? sizeof(bhg::WalkQuad) : 0) +
+                            (t.d_smom ? sizeof(double4_32a) : 0) + (t.d_sq64 ? 48 : 0));
+  b += t.sib_cap / bhg::kSibsPerBlock * bhg::kCellsPerBlock *
+       (int64_t)(sizeof(float) + (t.d_cmass64 ? sizeof(double) : 0));
   b += t.quad_cap * (int64_t)sizeof(bhg::WalkQuad) + (t.d_q64 ? t.quad_cap * 48 : 0);
   b += t.nf_cap * (int64_t)(2 * sizeof(int) + 2 * sizeof(double)) + (t.nf_cap ? 4 : 0);
   b += t.stage_in_bytes + t.stage_out_bytes + 4 * sizeof(unsigned);

@@ -450,6 +450,28 @@ __device__ __forceinline__ WalkRec make_rec(double x, double y, double z, double
   return w;
 }
 
+// A node's places in the arrays in sibling order (null where it has none or
+// the walk does not need it) and where its children start.
+struct SibOut {
+  WalkSib *rec = nullptr;
+  WalkQuad *quad = nullptr;
+  double4_32a *mom = nullptr;
+  double *q64 = nullptr;
+  unsigned kids = 0u;
+};
+__device__ __forceinline__ SibOut sib_out(const SibArgs &s, int64_t sid, unsigned kids,
+                                          bool listed = true) {
+  SibOut o;
+  if (listed) {
+    o.rec = s.sib + sid;
+    o.quad = s.quad ? s.quad + sid : nullptr;
+    o.mom = s.mom ? s.mom + sid : nullptr;
+    o.q64 = s.q64 ? s.q64 + 6 * sid : nullptr;
+  }
+  o.kids = kids;
+  return o;
+}
+
 // ku = -e for the field's binary32 mass unit 2^e (the record's mass).
 // inv_theta > 0: also the squared opening radius s2 = fl(fl(l fl(1/theta)) +
 // delta)^2 from the same binary32 l and delta as k_prepare_s2 (identical).
@@ -458,12 +480,11 @@ __device__ __forceinline__ WalkRec make_rec(double x, double y, double z, double
 // the geometric centre, x and y in the record's two spare words (z goes
 // into the quadrupole record's, store_quad_f), for the parent's quadrupole
 // shift.  spare: the record's first spare word otherwise (a top node's slot).
-// sib: the node's place in sibling order (null: a field's root), kids its
-// children's.
+// out: the node's places in sibling order (none: a field's root).
 __device__ __forceinline__ float store_internal(int64_t id, int64_t skip, int level,
                                                 const Moment &r, double4_32a *mom, WalkRec *rec,
                                                 float2 *aux, uint8_t *lvl, int ku,
-                                                float inv_theta, WalkSib *sib, unsigned kids,
+                                                float inv_theta, const SibOut &out,
                                                 bool keep_off = false, float spare = 0.0f) {
   mom[id] = make_double4_32a(r.x, r.y, r.z, r.m);
   WalkRec w = make_rec(r.x, r.y, r.z, r.m, ku, skip);
@@ -478,17 +499,18 @@ __device__ __forceinline__ float store_internal(int64_t id, int64_t skip, int le
     w.s2 = __fmul_rn(s, s);
   }
   rec[id] = w;
-  if (sib) {
+  if (out.rec) {
     WalkSib b;
     b.px = w.px;
     b.py = w.py;
     b.pz = w.pz;
     b.m = w.m;
     b.s2 = w.s2;
-    b.kids = kids;
+    b.kids = out.kids;
     b.l = l;
     b.delta = delta;
-    *sib = b;
+    *out.rec = b;
+    if (out.mom) *out.mom = make_double4_32a(r.x, r.y, r.z, r.m);
   }
   aux[id] = make_float2(l, delta);
   if (lvl) lvl[id] = (uint8_t)level;
@@ -511,26 +533,12 @@ __device__ __forceinline__ void add_shifted(double Q[6], const double *Qc, doubl
     for (int a = 0; a < 6; ++a) Q[a] += Qc[a];
 }
 
-// Binary32 version, used when the walk is binary32: the quadrupole term is a
+// Binary32 version, used when the walk is binary32 (the quadrupole term is a
 // small correction rounded to binary32 anyway, and GB300 runs FP64 far slower
-// than FP32.  fm is the child's mass in the field's binary32 mass unit; the
-// shift s is formed in FP64 (a difference of nearby centres of mass) and
-// then rounded (top nodes), or inside a block from binary32 offsets (below).
-__device__ __forceinline__ void add_shifted_f(float Q[6], const float *Qc, float fm, double sx,
-                                              double sy, double sz) {
-  const float x = narrow(sx), y = narrow(sy), z = narrow(sz);
-  const float s2 = x * x + y * y + z * z;
-  Q[0] += fm * (3.0f * x * x - s2);
-  Q[1] += fm * (3.0f * y * y - s2);
-  Q[2] += fm * (3.0f * z * z - s2);
-  Q[3] += fm * (3.0f * x * y);
-  Q[4] += fm * (3.0f * x * z);
-  Q[5] += fm * (3.0f * y * z);
-  if (Qc)
-    for (int a = 0; a < 6; ++a) Q[a] += Qc[a];
-}
-
-// The same with the shift given in binary32.  Inside a block it is formed as
+// than FP32).  fm is the child's mass in the field's binary32 mass unit, x, y,
+// z its shift: formed in FP64 (a difference of nearby centres of mass) and
+// rounded for top nodes, or from binary32 offsets inside a block.
+// Inside a block it is formed as
 // s = (c_child - c_parent) + (o_child - o_parent), o = R - c the binary32
 // offsets of the centres of mass from the geometric centres c: c_child -
 // c_parent is +-l/4 (exact) and every term is of the node's size, so s
@@ -581,8 +589,11 @@ __device__ __forceinline__ void load_quad_f(const WalkQuad &w, float Q[6]) {
 // Qzz/2, Qxy, Qxz, Qyz} in the field's mass unit (inv_unit = 2^-e):
 // the halves fold the 1/2 of the quadrupole term.
 __device__ __forceinline__ void store_quad(int64_t id, const double Q[6], double *q64,
-                                           WalkQuad *qrec, double inv_unit) {
-  for (int a = 0; a < 6; ++a) q64[6 * id + a] = Q[a];
+                                           WalkQuad *qrec, double *sq64, double inv_unit) {
+  for (int a = 0; a < 6; ++a) {
+    q64[6 * id + a] = Q[a];
+    if (sq64) sq64[a] = Q[a];
+  }
   const double u = inv_unit;
   WalkQuad w;
   w.hxx = __double2float_rn(0.5 * Q[0] * u);
@@ -646,6 +657,7 @@ __global__ void __launch_bounds__(kBlockThreads)
     cm[m] = mass;
     cmu[m] = mu;
     sib.cmass[(int64_t)p * kCellsPerBlock + m] = mu;
+    if (sib.cmass64) sib.cmass64[(int64_t)p * kCellsPerBlock + m] = mass;
     cxs[m] = ux;
     cys[m] = uy;
     czs[m] = uz;
@@ -681,16 +693,16 @@ __global__ void __launch_bounds__(kBlockThreads)
       accumulate(M, Sx, Sy, Sz, cm[8 * q + o], cxs[8 * q + o], cys[8 * q + o], czs[8 * q + o]);
     const Moment r = finish(M, Sx, Sy, Sz, cx, cy, cz);
     const int64_t id = root + 2 + 73 * (q >> 3) + 9 * (q & 7);
-    const int64_t sid = (int64_t)kSibsPerBlock * p + 8 + q;
-    store_internal(id, id + 9, lb + 2, r, mom, rec, aux, lvl, ku, inv_theta, sib.sib + sid,
-                   kBottomBit | (unsigned)(64 * p + q), quad32);
+    const SibOut out = sib_out(sib, (int64_t)kSibsPerBlock * p + 8 + q,
+                               kBottomBit | (unsigned)(64 * p + q));
+    store_internal(id, id + 9, lb + 2, r, mom, rec, aux, lvl, ku, inv_theta, out, quad32);
     if (quad64) {
       double Q[6] = {0, 0, 0, 0, 0, 0};
       for (int o = 0; o < 8; ++o) {
         const int k = 8 * q + o;
         add_shifted(Q, nullptr, cm[k], cxs[k] - r.x, cys[k] - r.y, czs[k] - r.z);
       }
-      store_quad(id, Q, q64, qrec, inv_unit);
+      store_quad(id, Q, q64, qrec, out.q64, inv_unit);
     } else if (quad32) {
       // children: cells at c +- h/2 (h = 2^-(lb+3)) with o = 0
       const float ox = narrow(r.ox), oy = narrow(r.oy), oz = narrow(r.oz);
@@ -701,7 +713,7 @@ __global__ void __launch_bounds__(kBlockThreads)
         add_shifted_ff(Q, nullptr, cmu[8 * q + o], __fsub_rn(dx, ox), __fsub_rn(dy, oy),
                        __fsub_rn(dz, oz));
       }
-      store_quad_f(id, Q, qrec, sib.quad ? sib.quad + sid : nullptr, oz);
+      store_quad_f(id, Q, qrec, out.quad, oz);
     }
   }
 }
@@ -736,7 +748,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
                                                double inv_unit, float inv_theta,
                                                double4_32a *mom, WalkRec *rec, float2 *aux,
                                                uint8_t *lvl, double *q64, WalkQuad *qrec,
-                                               WalkSib *sib, WalkQuad *squad, unsigned kids) {
+                                               const SibOut &out) {
   constexpr int64_t stride = 9;
   const double cx = centre_coord(ix, lev), cy = centre_coord(iy, lev), cz = centre_coord(iz, lev);
   double4_32a ch[8];
@@ -748,7 +760,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
   for (int o = 1; o < 8; ++o) accumulate(M, Sx, Sy, Sz, ch[o].w, ch[o].x, ch[o].y, ch[o].z);
   const Moment r = finish(M, Sx, Sy, Sz, cx, cy, cz);
   const bool quad32 = qrec && !q64;
-  store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, sib, kids, quad32);
+  store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, out, quad32);
   if (q64) {
     double Q[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll
@@ -756,7 +768,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
       const int64_t k = first + stride * o;
       add_shifted(Q, q64 + 6 * k, ch[o].w, ch[o].x - r.x, ch[o].y - r.y, ch[o].z - r.z);
     }
-    store_quad(id, Q, q64, qrec, inv_unit);
+    store_quad(id, Q, q64, qrec, out.q64, inv_unit);
   } else if (qrec) {
     const float ox = narrow(r.ox), oy = narrow(r.oy), oz = narrow(r.oz);
     const float hc = pow2f(-(lev + 2));  // child centre - centre: +-2^-(lev+2)
@@ -775,7 +787,7 @@ __device__ __forceinline__ void level_one_node(int lev, int ix, int iy, int iz, 
                      __fsub_rn(__fadd_rn(dy, cr.pad[1]), oy),
                      __fsub_rn(__fadd_rn(dz, cq.pad[0]), oz));
     }
-    store_quad_f(id, Q, qrec, squad, oz);
+    store_quad_f(id, Q, qrec, out.quad, oz);
   }
 }
 
@@ -798,8 +810,8 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
                                            int64_t id, int64_t skip, int64_t child, int ku,
                                            double inv_unit, float inv_theta, double4_32a *mom,
                                            WalkRec *rec, float2 *aux, uint8_t *lvl, double *q64,
-                                           WalkQuad *qrec, WalkSib *sib, WalkQuad *squad,
-                                           unsigned kids, float spare = 0.0f) {
+                                           WalkQuad *qrec, const SibOut &out,
+                                           float spare = 0.0f) {
   const double4_32a c = CG ? ld_mom_cg(mom + child) : mom[child];
   WalkQuad qc = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, {0.0f, 0.0f}};
   float fm = 0.0f, gx = 0.0f, gy = 0.0f;
@@ -838,7 +850,7 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
   r.delta = __dsqrt_rn(__dadd_rn(__dadd_rn(__shfl_sync(gmask, sq, gbase + 1),
                                            __shfl_sync(gmask, sq, gbase + 2)),
                                  __shfl_sync(gmask, sq, gbase + 3)));
-  if (o == 0) store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, sib, kids, false,
+  if (o == 0) store_internal(id, skip, lev, r, mom, rec, aux, lvl, ku, inv_theta, out, false,
                              spare);
   if (q64) {  // FP64 quadrupoles (the FP64 walk): on lane 0, as the one-thread form
     int64_t kids[8];
@@ -853,7 +865,7 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
         for (int a = 0; a < 6; ++a) Qc[a] = CG ? __ldcg(q64 + 6 * kj + a) : q64[6 * kj + a];
         add_shifted(Q, Qc, cj.w, cj.x - r.x, cj.y - r.y, cj.z - r.z);
       }
-      store_quad(id, Q, q64, qrec, inv_unit);
+      store_quad(id, Q, q64, qrec, out.q64, inv_unit);
     }
     return;
   }
@@ -883,7 +895,7 @@ __device__ __forceinline__ void group_node(unsigned gmask, int gbase, int o, int
     add_shifted_ff(Q, Qc, __shfl_sync(gmask, fm, gbase + j), __shfl_sync(gmask, sx, gbase + j),
                    __shfl_sync(gmask, sy, gbase + j), __shfl_sync(gmask, sz, gbase + j));
   }
-  if (o == 0) store_quad_f(id, Q, qrec, squad);
+  if (o == 0) store_quad_f(id, Q, qrec, out.quad);
 }
 
 // The octant of cube (i, j, k) in its parent.
@@ -911,9 +923,8 @@ __device__ __forceinline__ bool top_node(unsigned gmask, int gbase, int o, int s
   group_node<false, true>(gmask, gbase, o, level, 0, 0, 0, centre_coord(a.z, level),
                           centre_coord(a.w, level), centre_coord(b.x, level), a.x, a.y, c, ku,
                           pow2i(ku), inv_theta, mom, rec, aux, nullptr, q64, qrec,
-                          listed ? sib.sib + sid : nullptr,
-                          listed && sib.quad ? sib.quad + sid : nullptr,
-                          (unsigned)(sib.tops + 8 * (int64_t)s), __int_as_float(s));
+                          sib_out(sib, sid, (unsigned)(sib.tops + 8 * (int64_t)s), listed),
+                          __int_as_float(s));
   return true;
 }
 
@@ -950,9 +961,8 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
         const int64_t id = root + 1 + 73 * c, sid = (int64_t)kSibsPerBlock * p + c;
         level_one_node(lb + 1, 2 * B.y + (c & 1), 2 * B.z + ((c >> 1) & 1),
                        2 * B.w + ((c >> 2) & 1), id, id + 73, id + 1, ku, pow2i(ku), inv_theta,
-                       mom, rec, aux, lvl, q64, qrec, sib.sib + sid,
-                       sib.quad ? sib.quad + sid : nullptr,
-                       (unsigned)(kSibsPerBlock * p + 8 + 8 * c));
+                       mom, rec, aux, lvl, q64, qrec,
+                       sib_out(sib, sid, (unsigned)(kSibsPerBlock * p + 8 + 8 * c)));
       }
     }
   }
@@ -973,9 +983,8 @@ __global__ void __launch_bounds__(8 * kUpperBlocks)
   group_node<true, false>(gmask, gbase, o, lb, B.y, B.z, B.w, centre_coord(B.y, lb),
                           centre_coord(B.z, lb), centre_coord(B.w, lb), root,
                           root + kNodesPerBlock, root + 1 + 73 * o, ku, pow2i(ku), inv_theta, mom,
-                          rec, aux, lvl, q64, qrec, listed ? sib.sib + sid : nullptr,
-                          listed && sib.quad ? sib.quad + sid : nullptr,
-                          (unsigned)(kSibsPerBlock * p));
+                          rec, aux, lvl, q64, qrec,
+                          sib_out(sib, sid, (unsigned)(kSibsPerBlock * p), listed));
   // (3) climb: the parent top node of this root, then its parents
   while (s >= 0) {
     if (s >= top.slots) {  // a failed geometry

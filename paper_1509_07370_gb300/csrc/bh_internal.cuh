@@ -117,6 +117,11 @@ struct SibArgs {
   WalkSib *sib = nullptr;
   WalkQuad *quad = nullptr;
   float *cmass = nullptr;
+  // the same in binary64, for the binary64 walk only (else null): moments,
+  // quadrupoles (6 each, quadrupole option) and cell masses
+  double4_32a *mom = nullptr;
+  double *q64 = nullptr;
+  double *cmass64 = nullptr;
   int64_t tops = 0;   // where the top nodes' children start: 72 nb
   int64_t slots = 0;  // top nodes there is room for: nb / 7 + 1
 };
@@ -225,6 +230,8 @@ struct Tree {
   WalkSib *d_sib = nullptr;     // sibling order (capacity sib_cap entries)
   WalkQuad *d_squad = nullptr;
   float *d_cmass = nullptr;
+  double4_32a *d_smom = nullptr;  // binary64 walk
+  double *d_sq64 = nullptr, *d_cmass64 = nullptr;
   int64_t sib_cap = 0;
   double *d_q64 = nullptr;      // 6 per node, FP64 quadrupoles (quadrupole option)
   WalkQuad *d_qrec = nullptr;   // binary32 quadrupole walk records
@@ -331,9 +338,13 @@ cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux
 // the binary32 walk).  shape = the launch shape of the per-cell binary32
 // walk (warps per CTA, target pairs per lane; 0 = defaults), tunable.
 cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
-                        const double4_32a *mom, const SibArgs &sib, const double *q64,
-                        const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf = nullptr,
-                        WalkShape shape = WalkShape());
+                        const SibArgs &sib, const int4 *blk, const int *orig, const FieldArgs &fa,
+                        double G, void *out, int32_t *n_int, int32_t *n_test,
+                        int32_t *n_leaf = nullptr, WalkShape shape = WalkShape());
+// Its binary64 form (bh_walk_f64.cu).
+cudaError_t launch_walk_f64(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
+                            const SibArgs &sib, const int4 *blk, const int *orig,
+                            const FieldArgs &fa, double G, void *out);
 // Raises the dynamic shared-memory limit of the walk kernels on the current
 // device; called once per context, outside any graph capture.
 cudaError_t prepare_walk_kernels();

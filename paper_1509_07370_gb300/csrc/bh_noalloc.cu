@@ -210,7 +210,6 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
                             sib.sib, (float)(1.0 / theta)));
   bh_options opt;
   bh_default_options(&opt);
-  NA_CUDA(launch_walk(s, opt, nb, d_rec, d_mom, sib, nullptr, d_blk, d_orig, fa, G, out,
-                      nullptr, nullptr, nullptr, WalkShape()));
+  NA_CUDA(launch_walk(s, opt, nb, d_rec, sib, d_blk, d_orig, fa, G, out, nullptr, nullptr, nullptr, WalkShape()));
   return BH_OK;
 }

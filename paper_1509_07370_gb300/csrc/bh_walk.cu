@@ -48,16 +48,14 @@
 // instead of one.
 //
 // The opening test is evaluated in binary32 with the operation order stated
-// in the public header; the interaction uses the same d2 formed again, or
-// recomputes d in binary64 from the FP64 moments (k_walk_scalar).
+// in the public header; the interaction uses the same d2 formed again.  (The
+// binary64 walk, bh_walk_f64.cu, and the periodic one share the traversal.)
 #include "bh_lists.cuh"
 
 namespace bhg {
 namespace {
 
-constexpr int kWalkThreads = 256;               // CTA of the scalar walk: 8 bricks = half a block
-constexpr int kWarpsPerCta = kWalkThreads / 32;
-constexpr int kMaxWalkThreads = 512;            // largest tunable CTA
+constexpr int kMaxWalkThreads = 512;  // largest tunable CTA
 // 80 registers: 24 warps per SM (97 without the bound, 20 warps: 8 % slower;
 // 72: 28 warps, spills: 2-5 % slower).
 constexpr int kWalkRegs = 80;
@@ -95,19 +93,6 @@ struct WalkMem {                     // of one warp
   float4 centre[kBottoms];           // opened bottom nodes: geometric centre, half a cell,
   uint32_t bottom[3][kBottoms];      // index, O (two words)
 };
-
-__device__ __forceinline__ uint32_t smem_addr(const void *p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-template <int BYTES>
-__device__ __forceinline__ void copy_async(void *dst, const void *src) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src),
-               "n"(BYTES)
-               : "memory");
-}
-__device__ __forceinline__ void copy_async_wait() {
-  asm volatile("cp.async.wait_all;" ::: "memory");
-}
 
 // Per-lane state of the evaluation: the lane's 8 targets as four x pairs, pair
 // 2 r + k: row r (y = 2 (sub-brick & 1) + r), x = 2 k, 2 k + 1.
@@ -604,76 +589,6 @@ __global__ void __maxnreg__(kWalkRegs)
   }
 }
 
-// ---- binary64 interactions, one target per lane -------------------------------
-//
-// One warp per 32-cell brick (4x4x2, local Morton 32q .. 32q+31), as the paper
-// groups its cells (Sec. 3.1.1, Sec. 3.3).  Every target keeps `next`, the
-// first node it still has to visit; the warp takes the smallest over its
-// lanes, all lanes load that node, and the targets whose `next` equals it
-// apply the test: accepted -> next = skip, opened -> node + 1.  With the warp
-// vote all lanes share `next`.
-template <bool VOTE, bool QUAD>
-__global__ void __launch_bounds__(kWalkThreads)
-    k_walk_scalar(int nbricks, const WalkRec *__restrict__ rec,
-                  const double4_32a *__restrict__ mom, const double *__restrict__ q64,
-                  const int4 *__restrict__ blk, const int *__restrict__ orig,
-                  const int4 *__restrict__ fld, const double *__restrict__ invL, double G,
-                  double *__restrict__ out) {
-  const int warp = blockIdx.x * kWarpsPerCta + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (warp >= nbricks) return;  // whole warps only
-  const int p = warp >> 4;      // sorted block
-  const int m = ((warp & 15) << 5) | lane;  // local Morton index of this lane's cell
-  const int4 B = blk[p];
-  const int4 F = fld[p];        // this field's node range
-  const unsigned n_nodes = (unsigned)F.y;
-  const int cx = (int)compact3(m), cy = (int)compact3(m >> 1), cz = (int)compact3(m >> 2);
-  const float hh = pow2f(-(B.x + 3 + 1));
-  const float tx = __fmul_rn((float)(2 * (8 * B.y + cx) + 1), hh);
-  const float ty = __fmul_rn((float)(2 * (8 * B.z + cy) + 1), hh);
-  const float tz = __fmul_rn((float)(2 * (8 * B.w + cz) + 1), hh);
-  double sumd = 0.0;
-  unsigned next = (unsigned)F.x;  // the field's root
-  unsigned node = (unsigned)F.x;
-  while (node < n_nodes) {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(rec + node));
-    const float s2 = __ldg(&rec[node].s2);
-    const unsigned skip = __ldg(&rec[node].skip);
-    const float dx = __fsub_rn(tx, a.x);
-    const float dy = __fsub_rn(ty, a.y);
-    const float dz = __fsub_rn(tz, a.z);
-    const float d2 = __fmaf_rn(dx, dx, __fmaf_rn(dz, dz, __fmul_rn(dy, dy)));
-    const bool internal = s2 > 0.0f;
-    bool take;
-    if (VOTE) {
-      const bool acc = d2 > s2;
-      take = internal ? (__all_sync(kFull, acc) != 0) : acc;
-      next = (internal && !take) ? node + 1 : skip;
-    } else {
-      const bool mine = next == node;
-      take = mine && d2 > s2;
-      next = max(next, take ? skip : node + 1);
-    }
-    if (take) {
-      const double4_32a md = mom[node];
-      const double ex = (double)tx - md.x, ey = (double)ty - md.y, ez = (double)tz - md.z;
-      const double dd = ex * ex + ey * ey + ez * ez;
-      const double rinv = 1.0 / sqrt(dd);
-      double t = md.w * rinv;
-      if (QUAD && internal) {
-        const double *Q = q64 + 6 * (size_t)node;
-        const double hq = 0.5 * (Q[0] * ex * ex + Q[1] * ey * ey + Q[2] * ez * ez) +
-                          Q[3] * ex * ey + Q[4] * ex * ez + Q[5] * ey * ez;
-        t += hq * rinv * rinv * rinv * rinv * rinv;
-      }
-      sumd += t;
-    }
-    node = VOTE ? next : __reduce_min_sync(kFull, next);
-  }
-  const int64_t cell = (int64_t)orig[p] * kCellsPerBlock + cz * 64 + cy * 8 + cx;
-  out[cell] = sumd * (-G * invL[F.w]);  // physical FP64 moments
-}
-
 template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
 cudaError_t go_lists(cudaStream_t s, int nb, const WalkArgs &a, const WalkShape &shape) {
   const int np = shape.pairs > 0 ? shape.pairs : 1;
@@ -700,20 +615,6 @@ cudaError_t go_lists(cudaStream_t s, int nb, const WalkArgs &a, const WalkShape 
   }
   const int grid = (int)((nunits + w - 1) / w);
   k_walk_lists<KAHAN, COUNTS, QUAD, VOTE><<<grid, 32 * w, smem, s>>>(nunits, np, shape.order, a);
-  return cudaGetLastError();
-}
-
-template <bool QUAD>
-cudaError_t go_f64(cudaStream_t s, bool vote, int nb, const WalkRec *rec, const double4_32a *mom,
-                   const double *q64, const WalkArgs &a, void *out) {
-  const int nbricks = nb * 16;
-  const int grid = (nbricks + kWarpsPerCta - 1) / kWarpsPerCta;
-  if (vote)
-    k_walk_scalar<true, QUAD><<<grid, kWalkThreads, 0, s>>>(nbricks, rec, mom, q64, a.blk, a.orig,
-                                                            a.fld, a.invL, a.G, (double *)out);
-  else
-    k_walk_scalar<false, QUAD><<<grid, kWalkThreads, 0, s>>>(nbricks, rec, mom, q64, a.blk, a.orig,
-                                                             a.fld, a.invL, a.G, (double *)out);
   return cudaGetLastError();
 }
 
@@ -766,9 +667,9 @@ cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux
 // same decisions as every walk of the same criterion (the opening test does
 // not depend on precision, summation or the quadrupole term).
 cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
-                        const double4_32a *mom, const SibArgs &sib, const double *q64,
-                        const int4 *blk, const int *orig, const FieldArgs &fa, double G, void *out,
-                        int32_t *n_int, int32_t *n_test, int32_t *n_leaf, WalkShape shape) {
+                        const SibArgs &sib, const int4 *blk, const int *orig, const FieldArgs &fa,
+                        double G, void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf,
+                        WalkShape shape) {
   WalkArgs a;
   a.rec = rec;
   a.sib = sib;
@@ -786,8 +687,7 @@ cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const Wal
   const bool vote = opt.criterion == BH_CRIT_WARP_VOTE;
   if (n_int) return go_criterion<false, true, false>(s, vote, nb, a, shape);
   if (opt.precision == BH_PREC_F64)
-    return opt.quadrupole ? go_f64<true>(s, vote, nb, rec, mom, q64, a, out)
-                          : go_f64<false>(s, vote, nb, rec, mom, q64, a, out);
+    return launch_walk_f64(s, opt, nb, rec, sib, blk, orig, fa, G, out);
   if (opt.quadrupole)
     return opt.kahan ? go_criterion<true, false, true>(s, vote, nb, a, shape)
                      : go_criterion<false, false, true>(s, vote, nb, a, shape);

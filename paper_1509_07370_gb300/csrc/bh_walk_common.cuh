@@ -78,6 +78,21 @@ __device__ __forceinline__ void load_quad(const WalkQuad *p, u64 &w0, u64 &w1, u
   w3 = pk(qyz, 0.0f);
 }
 
+// Asynchronous copies from global to shared memory (visible to the copying
+// thread after copy_async_wait, to others after a barrier then).
+__device__ __forceinline__ uint32_t smem_addr(const void *p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_addr(dst)), "l"(src),
+               "n"(BYTES)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
 // ---- pair walk arithmetic ---------------------------------------------------
 // Compensated summation of the pair `term` into the running pair sums: the
 // rounding error of each addition, err = (sum - t) + term with t = sum + term
