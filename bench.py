@@ -260,7 +260,8 @@ def captured_traffic(workload_name, theta, mode):
         "monopole": ("walk_queue_monopole_theta0.24_maclaurin_2M.md",
                      ("bh_walk.cu", "bh_lists.cuh", "bh_walk_common.cuh")),
         "periodic64": ("walk_periodic_theta0.7_maclaurin_2M.md",
-                       ("bh_walk_periodic.cu", "bh_ewald.cuh", "bh_walk_common.cuh")),
+                       ("bh_walk_periodic.cu", "bh_ewald.cuh", "bh_rows.cuh", "bh_lists.cuh",
+                        "bh_walk_common.cuh")),
         "batched_monopole": ("walk_queue_batched64_theta0.5.md",
                              ("bh_walk.cu", "bh_lists.cuh", "bh_walk_common.cuh")),
     }.get(mode, (None, None))

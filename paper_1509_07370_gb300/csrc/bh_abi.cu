@@ -527,7 +527,7 @@ static cudaError_t enqueue_walk(bh_ctx *ctx, cudaStream_t s, double G, void *out
   if (ctx->opt.periodic) {  // one pair per lane, a plain grid, optionally longest first
     const int64_t groups = (int64_t)t.nb * 8;
     const unsigned *order = shape.longest && t.order_n[0] == groups ? t.d_order[0] : nullptr;
-    return bhg::launch_walk_periodic(s, ctx->opt, t.nb, t.d_rec, t.d_blk, t.d_orig,
+    return bhg::launch_walk_periodic(s, ctx->opt, t.nb, t.d_rec, sib_args(t), t.d_blk, t.d_orig,
                                      field_args(t), ctx->d_ewald, ctx->ewald_n, G, out, n_int,
                                      n_test, n_leaf, shape.warps, order, shape.cycles);
   }
@@ -576,6 +576,7 @@ bh_status bh_create(bh_ctx **out, const bh_options *opt, int device, void *cuda_
   ctx->device = device;
   ctx->stream = (cudaStream_t)cuda_stream;
   if (cudaSetDevice(device) != cudaSuccess || bhg::prepare_walk_kernels() != cudaSuccess ||
+      bhg::prepare_periodic_kernels() != cudaSuccess ||
       bhg::prepare_learned_kernels() != cudaSuccess ||
       bhg::prepare_mlp_tc_kernel() != cudaSuccess ||
       bhg::prepare_learned_tc_kernel() != cudaSuccess ||

@@ -25,9 +25,10 @@
 //                 points), so their half-precision rounding changes chi by
 //                 less than 3e-7, far below the interpolation error;
 //   bytes 62..63  zero.
-// A lookup is two 32-byte loads (the L1 data stage, one wavefront per
-// distinct line and load, bounds the periodic walk) and 26 FMAs in Horner
-// form.
+// A lookup is two 32-byte loads (the L1 data stage takes one wavefront per
+// distinct line and load) and 26 FMAs in Horner form, z and y first: the 24 of
+// these that x does not enter are shared by targets with the same y, z and
+// centre.
 #pragma once
 #include <cuda_fp16.h>
 
@@ -64,19 +65,6 @@ __device__ __forceinline__ float half_hi(uint32_t w) {
   return __half2float(__ushort_as_half((unsigned short)(w >> 16)));
 }
 
-// The 64-byte entry of centre (cx, cy, cz), as two 32-byte loads (raw words).
-__device__ __forceinline__ void ewald_load(const unsigned char *tab, int n, int cx, int cy, int cz,
-                                           uint32_t w[16]) {
-  const unsigned char *e = tab + (size_t)kEwaldEntryBytes *
-                                     (unsigned)(((cz - 1) * n + (cy - 1)) * n + (cx - 1));
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-        : "=r"(w[8 * q]), "=r"(w[8 * q + 1]), "=r"(w[8 * q + 2]), "=r"(w[8 * q + 3]),
-          "=r"(w[8 * q + 4]), "=r"(w[8 * q + 5]), "=r"(w[8 * q + 6]), "=r"(w[8 * q + 7])
-        : "l"(e + 32 * q));
-}
-
 // Coefficient K(k, j, i) of an entry, widened to binary32 where it is used.
 __device__ __forceinline__ float ewald_coef(const uint32_t w[16], int k, int j, int i) {
   const int f = 9 * k + 3 * j + i;
@@ -88,31 +76,38 @@ __device__ __forceinline__ float ewald_coef(const uint32_t w[16], int k, int j, 
   return (slot & 1) ? half_hi(w[4 + (slot >> 1)]) : half_lo(w[4 + (slot >> 1)]);
 }
 
-// The interpolant at (fx, fy, fz) from an entry, in Horner form: x first (9
-// quadratics), then y (3), then z.
-__device__ __forceinline__ float ewald_poly(const uint32_t w[16], float fx, float fy, float fz) {
-  float px[9];
+// Entry e (two 32-byte loads) contracted over z and y at (fy, fz), in Horner
+// form: the interpolant k[0] + fx (k[1] + fx k[2]) along x.
+__device__ __forceinline__ void ewald_row(const unsigned char *tab, unsigned e, float fy, float fz,
+                                          float k[3]) {
+  const unsigned char *at = tab + (size_t)kEwaldEntryBytes * e;
+  uint32_t w[16];
 #pragma unroll
-  for (int r = 0; r < 9; ++r)
-    px[r] = __fmaf_rn(fx, __fmaf_rn(fx, ewald_coef(w, r / 3, r % 3, 2), ewald_coef(w, r / 3, r % 3, 1)),
-                      ewald_coef(w, r / 3, r % 3, 0));
-  float py[3];
+  for (int q = 0; q < 2; ++q)
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(w[8 * q]), "=r"(w[8 * q + 1]), "=r"(w[8 * q + 2]), "=r"(w[8 * q + 3]),
+          "=r"(w[8 * q + 4]), "=r"(w[8 * q + 5]), "=r"(w[8 * q + 6]), "=r"(w[8 * q + 7])
+        : "l"(at + 32 * q));
 #pragma unroll
-  for (int k = 0; k < 3; ++k)
-    py[k] = __fmaf_rn(fy, __fmaf_rn(fy, px[3 * k + 2], px[3 * k + 1]), px[3 * k]);
-  return __fmaf_rn(fz, __fmaf_rn(fz, py[2], py[1]), py[0]);
+  for (int i = 0; i < 3; ++i) {
+    float y[3];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+      y[j] = __fmaf_rn(fz, __fmaf_rn(fz, ewald_coef(w, 2, j, i), ewald_coef(w, 1, j, i)),
+                       ewald_coef(w, 0, j, i));
+    k[i] = __fmaf_rn(fy, __fmaf_rn(fy, y[2], y[1]), y[0]);
+  }
 }
 
 // chi at |displacement| (ax, ay, az), each >= 0.
 __device__ __forceinline__ float ewald_chi(const unsigned char *tab, int n, float s, float ax,
                                            float ay, float az) {
-  float fx, fy, fz;
-  uint32_t w[16];
+  float fx, fy, fz, k[3];
   const int cx = ewald_axis(ax, s, n, fx);
   const int cy = ewald_axis(ay, s, n, fy);
   const int cz = ewald_axis(az, s, n, fz);
-  ewald_load(tab, n, cx, cy, cz, w);
-  return ewald_poly(w, fx, fy, fz);
+  ewald_row(tab, (unsigned)(((cz - 1) * n + (cy - 1)) * n + (cx - 1)), fy, fz, k);
+  return __fmaf_rn(fx, __fmaf_rn(fx, k[2], k[1]), k[0]);
 }
 
 }  // namespace

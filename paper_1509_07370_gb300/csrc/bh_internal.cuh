@@ -453,12 +453,12 @@ cudaError_t launch_ewald_eval(cudaStream_t s, int64_t npts, const float *r,
 // wpc: warps per CTA (0 = default); order: the octants' walk order or null;
 // cycles (potential only, else null): each octant's walk time in SM cycles.
 cudaError_t launch_walk_periodic(cudaStream_t s, const bh_options &opt, int nb,
-                                 const WalkRec *rec, const int4 *blk, const int *orig,
-                                 const FieldArgs &fa, const unsigned char *tab, int n,
-                                 double G,
-                                 void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf,
+                                 const WalkRec *rec, const SibArgs &sib, const int4 *blk,
+                                 const int *orig, const FieldArgs &fa, const unsigned char *tab,
+                                 int n, double G, void *out, int32_t *n_int, int32_t *n_test, int32_t *n_leaf,
                                  int wpc, const unsigned *order = nullptr,
                                  unsigned long long *cycles = nullptr);
+cudaError_t prepare_periodic_kernels();  // as prepare_walk_kernels
 
 }  // namespace bhg
 

@@ -34,22 +34,41 @@ __device__ __forceinline__ uint32_t push_sign(uint32_t mask, float v) {
   return __funnelshift_l(__float_as_uint(v), mask, 1);
 }
 
+// The minimum image of a pair of box-unit displacements in (-1, 1): d minus the
+// nearest whole number (the two magic additions round to even at one half, so
+// +-1/2 stay; all three steps are exact for what they are used for).
+__device__ __forceinline__ u64 wrap2(u64 d) {
+  const u64 magic = pk(12582912.0f, 12582912.0f);  // 1.5 2^23
+  return sub2(d, sub2(add2(d, magic), magic));
+}
+
 // The opening test of one node for the 64 targets: bit 16 (y >> 1) + 8 (z & 1)
 // + 4 (y & 1) + x of m[z >> 1] is set iff d2 > s2, d2 = fma(dx, dx, fma(dz,
 // dz, dy dy)) (the header's rounding), read off the sign of s2 - d2, which
 // rounding to nearest keeps exact (and which a NaN has clear: not accepted).
 // 4 dx, 4 dz, 2 pairs of dy; 8 packed FMAs give the 16 (y, z) parts, then a
 // packed FMA, a packed subtraction and two funnel shifts per two targets:
-// 148 instructions for 32 nodes x 64 targets.
+// 148 instructions for 32 nodes x 64 targets (WRAP, minimum-image
+// displacements: 178).
+template <bool WRAP>
 __device__ __forceinline__ void test64(const Front &S, float px, float py, float pz,
                                        float s2, uint32_t m[2]) {
   const float4 x01 = S.tx[0], x23 = S.tx[1], z01 = S.tz[0], z23 = S.tz[1], yy = S.ty;
   const u64 pxx = pk(px, px), pyy = pk(py, py), pzz = pk(pz, pz), ss = pk(s2, s2);
-  const u64 dx[4] = {sub2(pk(x01.x, x01.y), pxx), sub2(pk(x01.z, x01.w), pxx),
+  u64 dx[4] = {sub2(pk(x01.x, x01.y), pxx), sub2(pk(x01.z, x01.w), pxx),
                      sub2(pk(x23.x, x23.y), pxx), sub2(pk(x23.z, x23.w), pxx)};
-  const u64 dz[4] = {sub2(pk(z01.x, z01.y), pzz), sub2(pk(z01.z, z01.w), pzz),
+  u64 dz[4] = {sub2(pk(z01.x, z01.y), pzz), sub2(pk(z01.z, z01.w), pzz),
                      sub2(pk(z23.x, z23.y), pzz), sub2(pk(z23.z, z23.w), pzz)};
-  const u64 dya = sub2(pk(yy.x, yy.y), pyy), dyb = sub2(pk(yy.z, yy.w), pyy);
+  u64 dya = sub2(pk(yy.x, yy.y), pyy), dyb = sub2(pk(yy.z, yy.w), pyy);
+  if (WRAP) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      dx[i] = wrap2(dx[i]);
+      dz[i] = wrap2(dz[i]);
+    }
+    dya = wrap2(dya);
+    dyb = wrap2(dyb);
+  }
   const u64 ya = mul2(dya, dya), yb = mul2(dyb, dyb);
 #pragma unroll
   for (int w = 0; w < 2; ++w) {
@@ -118,7 +137,7 @@ struct Tested {
 // Pops up to four opened nodes, tests their children, and pushes those that
 // some target opens (bottom nodes excepted).  With VOTE the targets of each
 // 32-cell brick (a word of the mask) accept only together.
-template <bool VOTE>
+template <bool VOTE, bool WRAP = false>
 __device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int lane,
                                              const WalkSib *__restrict__ sib) {
   const int pop = depth > pop4 ? 1 : (depth < 4 ? depth : 4);
@@ -136,7 +155,7 @@ __device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int
   }
   depth -= pop;
   uint32_t m[2];
-  test64(S, a.x, a.y, a.z, b.x, m);
+  test64<WRAP>(S, a.x, a.y, a.z, b.x, m);
   if (VOTE) {
     m[0] = m[0] == kFull ? kFull : 0u;
     m[1] = m[1] == kFull ? kFull : 0u;
