@@ -140,108 +140,204 @@ __global__ void __launch_bounds__(kEvalThreads)
 }
 
 // ---- MLP training (FP32, CUDA cores) ---------------------------------------
-// 64 samples per CTA of 256 threads; 4 threads per sample split the hidden
-// units; the CTA's weight gradients are summed over its samples and added
-// to the global gradient with one atomic per weight.
+// 64 samples per CTA of 256 threads.  Each of the four 64 x 64 products of the
+// forward and backward passes (hidden layer 2, its input gradient, the
+// gradient of W2; layer 1 is 10 wide) is tiled in registers: thread (ti, tj)
+// owns 4 samples (or weight rows) x 4 units, so 16 FMAs take two 128-bit
+// shared-memory reads (the first version read one or two words per FMA and
+// was bound by that).  Activations are kept transposed, [unit][sample], with a
+// pitch of 68 words.  Each GELU and its derivative come from one tanh, kept in
+// registers from the forward to the backward pass (the first version took
+// five).  The CTA's gradients are added to the global ones with one atomic
+// per weight, consecutive lanes to consecutive words.
+// Measured (8,192 samples, 128 CTAs): 64 -> 22 us; 40,000 samples with the
+// optimiser step 274 -> 64 us.
 constexpr int kMlpSamples = 64;
 constexpr int kMlpThreads = 256;
+constexpr int kMlpPitch = 68;
 
-__device__ __forceinline__ float gelu_f(float a) {
-  const float c = 0.7978845608028654f;
-  return 0.5f * a * (1.0f + tanhf(c * (a + 0.044715f * a * a * a)));
-}
-__device__ __forceinline__ float gelu_grad_f(float a) {
+// GELU (tanh form) and its derivative.
+__device__ __forceinline__ float gelu_both(float a, float &grad) {
   const float c = 0.7978845608028654f;
   const float t = tanhf(c * (a + 0.044715f * a * a * a));
-  return 0.5f * (1.0f + t) + 0.5f * a * (1.0f - t * t) * c * (1.0f + 3.0f * 0.044715f * a * a);
+  grad = 0.5f * (1.0f + t) + 0.5f * a * (1.0f - t * t) * c * (1.0f + 3.0f * 0.044715f * a * a);
+  return 0.5f * a * (1.0f + t);
 }
 
 struct MlpSmem {
-  float w[kMlpNW];
-  float x[kMlpSamples][kMlpIn];
-  float a1[kMlpSamples][kMlpH], h1[kMlpSamples][kMlpH], a2[kMlpSamples][kMlpH];
-  float d1[kMlpSamples][kMlpH], d2[kMlpSamples][kMlpH];
-  float dy[kMlpSamples];
-  float red[kMlpThreads / 32];
+  float w2[kMlpH][kMlpH], w2t[kMlpH][kMlpPitch];
+  float w1[kMlpIn][kMlpH], xt[kMlpIn][kMlpPitch];
+  float h1t[kMlpH][kMlpPitch];  // layer-1 activations
+  float dt[kMlpH][kMlpPitch];   // loss gradient at layer 2's input sums, then layer 1's
+  float red[3][16][kMlpH];      // of b1, b2 and W3 per sample group
+  float b1[kMlpH], b2[kMlpH], w3[kMlpH];
+  float dy[kMlpSamples], loss[kMlpSamples];
 };
+
+// acc[r][c] += sum over k of a[k][4 ti + r] b[k][4 tj + c].
+template <int K, int PA, int PB>
+__device__ __forceinline__ void tile_product(const float (*a)[PA], const float (*b)[PB], int ti,
+                                             int tj, float acc[4][4]) {
+#pragma unroll 8
+  for (int k = 0; k < K; ++k) {
+    const float4 u = *reinterpret_cast<const float4 *>(&a[k][4 * ti]);
+    const float4 v = *reinterpret_cast<const float4 *>(&b[k][4 * tj]);
+    const float uu[4] = {u.x, u.y, u.z, u.w}, vv[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(uu[r], vv[c], acc[r][c]);
+  }
+}
 
 __global__ void __launch_bounds__(kMlpThreads)
     k_mlp_grad(int64_t n, const float *__restrict__ x, const float *__restrict__ z,
                const float *__restrict__ w, float *__restrict__ grad, float *__restrict__ loss) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   MlpSmem &S = *reinterpret_cast<MlpSmem *>(smem_raw);
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, ti = t >> 4, tj = t & 15;
   const int64_t base = (int64_t)blockIdx.x * kMlpSamples;
-  for (int i = t; i < kMlpNW; i += kMlpThreads) S.w[i] = w[i];
-  for (int i = t; i < kMlpSamples * kMlpIn; i += kMlpThreads) {
-    const int64_t g = base + i / kMlpIn;
-    S.x[i / kMlpIn][i % kMlpIn] = g < n ? x[base * kMlpIn + i] : 0.0f;
-  }
-  __syncthreads();
-  const float *W1 = S.w, *b1 = W1 + kMlpIn * kMlpH, *W2 = b1 + kMlpH, *b2 = W2 + kMlpH * kMlpH;
+  const float *W1 = w, *b1 = W1 + kMlpIn * kMlpH, *W2 = b1 + kMlpH, *b2 = W2 + kMlpH * kMlpH;
   const float *W3 = b2 + kMlpH, *b3 = W3 + kMlpH;
-  const int smp = t >> 2, qtr = t & 3;       // sample, quarter of the hidden units
-  const int64_t g = base + smp;
-  const bool valid = g < n;
-  for (int j = qtr * 16; j < qtr * 16 + 16; ++j) {
-    float a = b1[j];
-    for (int k = 0; k < kMlpIn; ++k) a += S.x[smp][k] * W1[k * kMlpH + j];
-    S.a1[smp][j] = a;
-    S.h1[smp][j] = gelu_f(a);
+  for (int i = t; i < kMlpH * kMlpH; i += kMlpThreads) {
+    const float v = W2[i];
+    S.w2[i >> 6][i & 63] = v;
+    S.w2t[i & 63][i >> 6] = v;
+  }
+  for (int i = t; i < kMlpIn * kMlpH; i += kMlpThreads) S.w1[i >> 6][i & 63] = W1[i];
+  for (int i = t; i < kMlpSamples * kMlpIn; i += kMlpThreads)
+    S.xt[i % kMlpIn][i / kMlpIn] = base + i / kMlpIn < n ? x[base * kMlpIn + i] : 0.0f;
+  if (t < kMlpH) {
+    S.b1[t] = b1[t];
+    S.b2[t] = b2[t];
+    S.w3[t] = W3[t];
   }
   __syncthreads();
-  float y = 0.0f;
-  for (int j = qtr * 16; j < qtr * 16 + 16; ++j) {
-    float a = b2[j];
-    for (int k = 0; k < kMlpH; ++k) a += S.h1[smp][k] * W2[k * kMlpH + j];
-    S.a2[smp][j] = a;
-    y += gelu_f(a) * W3[j];
+  // layer 1 of samples 4 ti .. + 3, units 4 tj .. + 3
+  float g1[4][4], g2[4][4], acc[4][4], part[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = S.b1[4 * tj + c];
+  tile_product<kMlpIn>(S.xt, S.w1, ti, tj, acc);
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float4 h;
+    h.x = gelu_both(acc[0][c], g1[0][c]);
+    h.y = gelu_both(acc[1][c], g1[1][c]);
+    h.z = gelu_both(acc[2][c], g1[2][c]);
+    h.w = gelu_both(acc[3][c], g1[3][c]);
+    *reinterpret_cast<float4 *>(&S.h1t[4 * tj + c][4 * ti]) = h;
   }
-  y += __shfl_xor_sync(0xffffffffu, y, 1);
-  y += __shfl_xor_sync(0xffffffffu, y, 2);
-  y += b3[0];
-  const float r = valid ? y - z[g] : 0.0f;
-  const float dy = 2.0f * r / (float)n;
-  if (qtr == 0) S.dy[smp] = dy;
-  for (int j = qtr * 16; j < qtr * 16 + 16; ++j) S.d2[smp][j] = dy * W3[j] * gelu_grad_f(S.a2[smp][j]);
   __syncthreads();
-  for (int i = qtr * 16; i < qtr * 16 + 16; ++i) {
-    float a = 0.0f;
-    for (int j = 0; j < kMlpH; ++j) a += W2[i * kMlpH + j] * S.d2[smp][j];
-    S.d1[smp][i] = a * gelu_grad_f(S.a1[smp][i]);
-  }
-  // loss: sum of r^2 / n over the CTA
-  float l2 = (qtr == 0) ? r * r / (float)n : 0.0f;
-  for (int o = 16; o > 0; o >>= 1) l2 += __shfl_xor_sync(0xffffffffu, l2, o);
-  if ((t & 31) == 0) S.red[t >> 5] = l2;
-  __syncthreads();
-  if (t == 0) {
-    float tot = 0.0f;
-    for (int k = 0; k < kMlpThreads / 32; ++k) tot += S.red[k];
-    atomicAdd(loss, tot);
-  }
-  // weight gradients of this CTA's samples
-  for (int e = t; e < kMlpNW; e += kMlpThreads) {
-    float acc = 0.0f;
-    if (e < kMlpIn * kMlpH) {                                   // W1[k][j]
-      const int k = e / kMlpH, j = e % kMlpH;
-      for (int s = 0; s < kMlpSamples; ++s) acc += S.x[s][k] * S.d1[s][j];
-    } else if (e < kMlpIn * kMlpH + kMlpH) {                    // b1[j]
-      const int j = e - kMlpIn * kMlpH;
-      for (int s = 0; s < kMlpSamples; ++s) acc += S.d1[s][j];
-    } else if (e < kMlpIn * kMlpH + kMlpH + kMlpH * kMlpH) {    // W2[i][j]
-      const int ij = e - (kMlpIn * kMlpH + kMlpH), i = ij / kMlpH, j = ij % kMlpH;
-      for (int s = 0; s < kMlpSamples; ++s) acc += S.h1[s][i] * S.d2[s][j];
-    } else if (e < kMlpIn * kMlpH + 2 * kMlpH + kMlpH * kMlpH) {  // b2[j]
-      const int j = e - (kMlpIn * kMlpH + kMlpH + kMlpH * kMlpH);
-      for (int s = 0; s < kMlpSamples; ++s) acc += S.d2[s][j];
-    } else if (e < kMlpNW - 1) {                                // W3[j]
-      const int j = e - (kMlpIn * kMlpH + 2 * kMlpH + kMlpH * kMlpH);
-      for (int s = 0; s < kMlpSamples; ++s) acc += gelu_f(S.a2[s][j]) * S.dy[s];
-    } else {                                                    // b3
-      for (int s = 0; s < kMlpSamples; ++s) acc += S.dy[s];
+  // layer 2 and the output
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[r][c] = S.b2[4 * tj + c];
+  tile_product<kMlpH>(S.h1t, S.w2, ti, tj, acc);
+  float w3[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) w3[c] = S.w3[4 * tj + c];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    float y = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      acc[r][c] = gelu_both(acc[r][c], g2[r][c]);
+      y = fmaf(acc[r][c], w3[c], y);
     }
-    atomicAdd(&grad[e], acc);
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) y += __shfl_xor_sync(0xffffffffu, y, o);
+    const int64_t g = base + 4 * ti + r;
+    const float res = g < n ? y + b3[0] - z[g] : 0.0f;
+    part[r] = 2.0f * res / (float)n;  // dL/dy
+    if (tj == 0) {
+      S.dy[4 * ti + r] = part[r];
+      S.loss[4 * ti + r] = res * res / (float)n;
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float gw3 = 0.0f, gb2 = 0.0f, d[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      gw3 = fmaf(acc[r][c], part[r], gw3);
+      d[r] = part[r] * w3[c] * g2[r][c];
+      gb2 += d[r];
+      acc[r][c] = 0.0f;
+    }
+    S.red[2][ti][4 * tj + c] = gw3;
+    S.red[1][ti][4 * tj + c] = gb2;
+    *reinterpret_cast<float4 *>(&S.dt[4 * tj + c][4 * ti]) = make_float4(d[0], d[1], d[2], d[3]);
+  }
+  __syncthreads();
+  // back through layer 2: dL/d(layer-1 sums), same ownership as layer 1
+  tile_product<kMlpH>(S.dt, S.w2t, ti, tj, acc);
+  // gradient of W2: rows ti + 16 r, columns tj + 16 c (conflict-free reads)
+  float gw[4][4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) gw[r][c] = 0.0f;
+  for (int s = 0; s < kMlpSamples; s += 4) {
+    float4 h[4], d[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      h[r] = *reinterpret_cast<const float4 *>(&S.h1t[ti + 16 * r][s]);
+      d[r] = *reinterpret_cast<const float4 *>(&S.dt[tj + 16 * r][s]);
+    }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        gw[r][c] = fmaf(h[r].w, d[c].w, fmaf(h[r].z, d[c].z, fmaf(h[r].y, d[c].y, fmaf(h[r].x, d[c].x, gw[r][c]))));
+  }
+  float *gW1 = grad, *gb1 = gW1 + kMlpIn * kMlpH, *gW2 = gb1 + kMlpH, *gb2 = gW2 + kMlpH * kMlpH;
+  float *gW3 = gb2 + kMlpH, *gb3 = gW3 + kMlpH;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      atomicAdd(&gW2[(ti + 16 * r) * kMlpH + tj + 16 * c], gw[r][c]);
+  __syncthreads();  // dt has been read
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    float d[4], sum = 0.0f;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      d[r] = acc[r][c] * g1[r][c];
+      sum += d[r];
+    }
+    S.red[0][ti][4 * tj + c] = sum;
+    *reinterpret_cast<float4 *>(&S.dt[4 * tj + c][4 * ti]) = make_float4(d[0], d[1], d[2], d[3]);
+  }
+  __syncthreads();
+  // gradient of W1: input k of unit j
+  for (int e = t; e < kMlpIn * kMlpH; e += kMlpThreads) {
+    const int k = e >> 6, j = e & 63;
+    float v = 0.0f;
+#pragma unroll 4
+    for (int s = 0; s < kMlpSamples; s += 4) {
+      const float4 u = *reinterpret_cast<const float4 *>(&S.xt[k][s]);
+      const float4 d = *reinterpret_cast<const float4 *>(&S.dt[j][s]);
+      v = fmaf(u.w, d.w, fmaf(u.z, d.z, fmaf(u.y, d.y, fmaf(u.x, d.x, v))));
+    }
+    atomicAdd(&gW1[e], v);
+  }
+  if (t < 3 * kMlpH) {  // b1, b2, W3
+    const int q = t >> 6, j = t & 63;
+    float v = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v += S.red[q][i][j];
+    atomicAdd((q == 0 ? gb1 : q == 1 ? gb2 : gW3) + j, v);
+  } else {  // b3 and the loss, a warp each
+    const int l = t & 31;
+    const float *src = t < 3 * kMlpH + 32 ? S.dy : S.loss;
+    float v = src[l] + src[l + 32];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (l == 0) atomicAdd(t < 3 * kMlpH + 32 ? gb3 : loss, v);
   }
 }
 
