@@ -1160,7 +1160,7 @@ bh_status bh_stats(const bh_ctx *ctx, bh_stats_t *out) {
   b += t.quad_cap * (int64_t)sizeof(bhg::WalkQuad) + (t.d_q64 ? t.quad_cap * 48 : 0);
   b += t.nf_cap * (int64_t)(2 * sizeof(int) + 2 * sizeof(double)) + (t.nf_cap ? 4 : 0);
   b += t.stage_in_bytes + t.stage_out_bytes + 4 * sizeof(unsigned);
-  if (ctx->d_mlp) b += sizeof(bhg::MlpDev) + sizeof(bhg::MlpTc) + sizeof(unsigned);
+  if (ctx->d_mlp) b += sizeof(bhg::MlpDev) + sizeof(bhg::MlpTc);
   if (ctx->d_counts) b += 3 * sizeof(unsigned long long);
   if (ctx->d_ewald) b += (int64_t)ctx->ewald_n * ctx->ewald_n * ctx->ewald_n * 64;
   out->device_bytes = b;
@@ -1211,7 +1211,7 @@ void bh_destroy(bh_ctx *ctx) {
   release(ctx->tree.d_order[1]);
   release(ctx->d_mlp);
   release(ctx->d_mlp_tc);
-  release(ctx->d_tc_flag);
+  if (ctx->h_tc_flag) cudaFreeHost(ctx->h_tc_flag);
   release(ctx->d_counts);
   release(ctx->d_ewald);
   for (cudaEvent_t &e : ctx->ev)

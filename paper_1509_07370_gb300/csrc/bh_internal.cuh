@@ -475,7 +475,7 @@ struct bh_ctx {
   bhg::MlpDev *d_mlp = nullptr;  // learned correction, set by bh_set_mlp
   double mlp_s_min = 0.0;        // its gate (bh_set_mlp_gate): no network below s = l/d
   bhg::MlpTc *d_mlp_tc = nullptr;   // the same network for bh_mlp_eval
-  unsigned *d_tc_flag = nullptr;    // time-out flag of bh_mlp_eval
+  unsigned *h_tc_flag = nullptr;    // time-out flag of bh_mlp_eval (mapped host memory)
   unsigned char *d_ewald = nullptr; // periodic boundaries: the Ewald table
   int ewald_n = 0, ewald_series = 0;
   // statistics (bh_stats): events of the timing option (build start/end,

@@ -515,7 +515,8 @@ bh_status bh_set_mlp(bh_ctx *ctx, const float *w_host) {
   if (cudaSetDevice(ctx->device) != cudaSuccess) return ctx_fail(ctx, BH_ERR_CUDA, "device");
   if ((!ctx->d_mlp && bhg::dev_malloc(&ctx->d_mlp, sizeof(MlpDev)) != cudaSuccess) ||
       (!ctx->d_mlp_tc && bhg::dev_malloc(&ctx->d_mlp_tc, sizeof(MlpTc)) != cudaSuccess) ||
-      (!ctx->d_tc_flag && bhg::dev_malloc(&ctx->d_tc_flag, sizeof(unsigned)) != cudaSuccess)) {
+      (!ctx->h_tc_flag &&
+       cudaHostAlloc((void **)&ctx->h_tc_flag, sizeof(unsigned), cudaHostAllocMapped) != cudaSuccess)) {
     cudaGetLastError();
     return ctx_fail(ctx, BH_ERR_OOM, "bh_set_mlp: no device memory");
   }
@@ -542,16 +543,18 @@ bh_status bh_mlp_eval(bh_ctx *ctx, int64_t n, const float *x, float *y) {
     const long v = std::strtol(env, nullptr, 10);
     probe = v > 0 ? (int)(v < (1L << 20) ? v : (1L << 20)) : 0;
   }
-  unsigned flag = 0;
-  if (cudaMemsetAsync(ctx->d_tc_flag, 0, sizeof(unsigned), ctx->stream) != cudaSuccess ||
-      launch_mlp_tc(ctx->stream, n, x, ctx->d_mlp_tc, y, ctx->d_tc_flag, probe) != cudaSuccess ||
-      cudaMemcpyAsync(&flag, ctx->d_tc_flag, sizeof(unsigned), cudaMemcpyDeviceToHost,
-                      ctx->stream) != cudaSuccess ||
+  // the time-out flag lies in mapped host memory, which the kernel writes only
+  // when a wait gave up: no memset before it and no copy after it
+  volatile unsigned *flag = ctx->h_tc_flag;
+  unsigned *d_flag = nullptr;
+  *flag = 0u;
+  if (cudaHostGetDevicePointer((void **)&d_flag, ctx->h_tc_flag, 0) != cudaSuccess ||
+      launch_mlp_tc(ctx->stream, n, x, ctx->d_mlp_tc, y, d_flag, probe) != cudaSuccess ||
       cudaStreamSynchronize(ctx->stream) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(ctx, BH_ERR_CUDA, "bh_mlp_eval: %s", "launch failed");
   }
-  if (flag) return ctx_fail(ctx, BH_ERR_DEVICE_TIMEOUT, "bh_mlp_eval: a tensor-core wait gave up");
+  if (*flag) return ctx_fail(ctx, BH_ERR_DEVICE_TIMEOUT, "bh_mlp_eval: a tensor-core wait gave up");
   return BH_OK;
 }
 
