@@ -573,6 +573,11 @@ bh_status bh_create(bh_ctx **out, const bh_options *opt, int device, void *cuda_
   bh_ctx *ctx = new (std::nothrow) bh_ctx();
   if (!ctx) return BH_ERR_OOM;
   ctx->opt = o;
+  // The default shape: the persistent grid, one octant per take.  On a plain
+  // grid a 4-warp CTA holds its place until its longest octant is done: 4-6 %
+  // slower on every mesh measured, from 15 blocks (86 against 80 us) to the
+  // 16.3M-cell core (20.0 against 19.2 ms).
+  ctx->tree.shape.ticket = 1;
   ctx->device = device;
   ctx->stream = (cudaStream_t)cuda_stream;
   if (cudaSetDevice(device) != cudaSuccess || bhg::prepare_walk_kernels() != cudaSuccess ||

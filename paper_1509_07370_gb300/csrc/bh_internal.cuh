@@ -213,7 +213,7 @@ struct Tree {
   void *graph_out = nullptr;
   int graph_fp64 = -1;
   double graph_theta = 0.0, graph_G = 0.0;
-  WalkShape shape;              // tuned launch shape of the walk (0 = defaults)
+  WalkShape shape;              // launch shape of the walk (warps 0: not tuned)
   // walk order of the groups made by bh_autotune, longest walk first, for one
   // (np = 1) or two (np = 2) target pairs per lane: d_order[np - 1] holds
   // order_n[np - 1] group indices (0 = none); used while the tree has that
