@@ -407,12 +407,22 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   BH_CUDA(cudaEventRecord(t.geo_done, s));
   BH_CUDA(bhg::launch_keys_mass(s, nb, t.d_level, t.d_ijk, t.d_key[0], t.d_idx[0], t.d_flags, fa,
                                 density, density_is_fp64));
-  BH_CUDA(bhg::launch_sort_blocks(s, t.d_key, t.d_idx, t.d_flags, fa));
-  BH_CUDA(bhg::launch_tile_and_count(s, nb, t.d_key[0], t.d_idx[0], t.d_level, t.d_ijk,
-                                     t.d_count, t.d_blk, t.d_orig, t.d_flags, fa, top, t.d_pos));
-  BH_CUDA(bhg::launch_prestart_scan(s, nb, t.d_count, t.d_prestart, t.d_flags));
+  const bool small = bhg::small_geometry(nb);
+  if (small) {
+    BH_CUDA(bhg::launch_small_geometry(s, nb, t.d_key[0], t.d_idx[0], t.d_level, t.d_ijk,
+                                       t.d_count, t.d_prestart, t.d_blk, t.d_orig, t.d_pos,
+                                       n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa,
+                                       max_level, top));
+  } else {
+    BH_CUDA(bhg::launch_sort_blocks(s, t.d_key, t.d_idx, t.d_flags, fa));
+    BH_CUDA(bhg::launch_tile_and_count(s, nb, t.d_key[0], t.d_idx[0], t.d_level, t.d_ijk,
+                                       t.d_count, t.d_blk, t.d_orig, t.d_flags, fa, top,
+                                       t.d_pos));
+    BH_CUDA(bhg::launch_prestart_scan(s, nb, t.d_count, t.d_prestart, t.d_flags));
+  }
   // the top nodes' records and child lists (needed from k_upper_tree on) on
-  // the side stream, beside k_blocks, which writes only the blocks' nodes
+  // the side stream, beside k_blocks, which writes only the blocks' nodes (a
+  // small list's are done: launch_small_geometry)
   if (!ctx->side || !ctx->fork || !ctx->join) {  // made once, all three or none
     int lo_prio = 0, hi_prio = 0;
     cudaStream_t side = nullptr;
@@ -436,9 +446,10 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   }
   BH_CUDA(cudaEventRecord(ctx->fork, s));
   BH_CUDA(cudaStreamWaitEvent(ctx->side, ctx->fork, 0));
-  BH_CUDA(bhg::launch_top_nodes(ctx->side, nb, t.d_key[0], t.d_blk, t.d_count, t.d_prestart,
-                                n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa, t.d_orig,
-                                max_level, top));
+  if (!small)
+    BH_CUDA(bhg::launch_top_nodes(ctx->side, nb, t.d_key[0], t.d_blk, t.d_count, t.d_prestart,
+                                  n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa, t.d_orig,
+                                  max_level, top));
   // Every check of the input is done by now (levels, coordinates and density
   // in k_keys_mass, the tiling in k_tile_and_count, the top-node count in
   // k_prestart_scan, top indexes in k_top_nodes/k_top_children): the flags go
@@ -450,7 +461,8 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   BH_CUDA(cudaMemcpyAsync(t.h_flags, t.d_flags, 4 * sizeof(unsigned), cudaMemcpyDeviceToHost,
                           ctx->side));
   BH_CUDA(cudaEventRecord(ctx->join, ctx->side));
-  if ((st = enqueue_moments(ctx, density, density_is_fp64, true, ctx->join)) != BH_OK) return st;
+  if ((st = enqueue_moments(ctx, density, density_is_fp64, true, small ? nullptr : ctx->join)) != BH_OK)
+    return st;
   ctx->build_timed = timed && timing_mark(ctx, 1);
   BH_CUDA(cudaEventSynchronize(ctx->join));
   const unsigned e = t.h_flags[0];

@@ -171,15 +171,13 @@ __device__ __forceinline__ int top_start_level(unsigned long long key) {
   return max(0, kKeyLevels - tz / 3);
 }
 
-__global__ void k_tile_and_count(int nb, const unsigned long long *__restrict__ key,
-                                 const int *__restrict__ idx, const int *__restrict__ level,
-                                 const int *__restrict__ ijk, int *__restrict__ count,
-                                 int4 *__restrict__ blk, int *__restrict__ orig,
-                                 unsigned *flags, const int *__restrict__ fstart,
-                                 const int *__restrict__ fid, int *__restrict__ pos,
-                                 int *__restrict__ bparent) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nb) return;
+// Sorted position p: its block, and the top nodes that start at it.  (No
+// restrict here and below: k_small_geometry writes what it then reads.)
+__device__ __forceinline__ void tile_and_count(int p, const unsigned long long *key,
+                                               const int *idx, const int *level, const int *ijk,
+                                               int *count, int4 *blk, int *orig, unsigned *flags,
+                                               const int *fstart, const int *fid, int *pos,
+                                               int *bparent) {
   const int b = idx[p];
   if (pos) pos[b] = p;  // sorted position of caller block b
   bparent[p] = -1;      // a field's only block has no parent; k_top_children sets the rest
@@ -204,6 +202,18 @@ __global__ void k_tile_and_count(int nb, const unsigned long long *__restrict__ 
   count[p] = cnt;
   blk[p] = make_int4(lb, ijk[3 * b], ijk[3 * b + 1], ijk[3 * b + 2]);
   orig[p] = b;
+}
+
+__global__ void k_tile_and_count(int nb, const unsigned long long *__restrict__ key,
+                                 const int *__restrict__ idx, const int *__restrict__ level,
+                                 const int *__restrict__ ijk, int *__restrict__ count,
+                                 int4 *__restrict__ blk, int *__restrict__ orig,
+                                 unsigned *flags, const int *__restrict__ fstart,
+                                 const int *__restrict__ fid, int *__restrict__ pos,
+                                 int *__restrict__ bparent) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= nb) return;
+  tile_and_count(p, key, idx, level, ijk, count, blk, orig, flags, fstart, fid, pos, bparent);
 }
 
 // prestart[p] = 585 p + sum_{q<p} count[q]: pre-order index of the first node
@@ -272,16 +282,12 @@ __device__ __forceinline__ double as_f64(double v) { return v; }
 // Also records, per block, its field's node range: fld[p] = {first node of
 // the field (its root), one past its last node, first block of the next
 // field, field index}.
-__global__ void k_top_nodes(int nb, const unsigned long long *__restrict__ key,
-                            const int4 *__restrict__ blk, const int *__restrict__ count,
-                            const int *__restrict__ prestart, int64_t n_nodes,
-                            WalkRec *__restrict__ rec, float2 *__restrict__ aux,
-                            uint8_t *__restrict__ lvl, unsigned *flags, int nfields,
-                            const int *__restrict__ fstart, const int *__restrict__ fid,
-                            const int *__restrict__ orig, int4 *__restrict__ fld,
-                            TopArgs top) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= nb) return;
+__device__ __forceinline__ void top_nodes_of(int p, int nb, const unsigned long long *key,
+                                             const int4 *blk, const int *count,
+                                             const int *prestart, int64_t n_nodes, WalkRec *rec,
+                                             float2 *aux, uint8_t *lvl, unsigned *flags,
+                                             const int *fstart, const int *fid, const int *orig,
+                                             int4 *fld, const TopArgs &top) {
   const int f = fid[orig[p]];
   const int fend = fstart[f + 1];
   const int64_t node_end = fend < nb ? (int64_t)prestart[fend] : n_nodes;
@@ -318,6 +324,16 @@ __global__ void k_top_nodes(int nb, const unsigned long long *__restrict__ key,
   }
 }
 
+__global__ void k_top_nodes(int nb, const unsigned long long *key, const int4 *blk,
+                            const int *count, const int *prestart, int64_t n_nodes, WalkRec *rec,
+                            float2 *aux, uint8_t *lvl, unsigned *flags, const int *fstart,
+                            const int *fid, const int *orig, int4 *fld, TopArgs top) {
+  const int p = blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= nb) return;
+  top_nodes_of(p, nb, key, blk, count, prestart, n_nodes, rec, aux, lvl, flags, fstart, fid, orig,
+               fld, top);
+}
+
 // Child lists of the top nodes, for the moment pass: entry 8 slot + o holds
 // the pre-order index of child o of the top node with compact index
 // slot = prestart[p] - 585 p + r (the r-th top node that starts at block p,
@@ -329,15 +345,10 @@ __global__ void k_top_nodes(int nb, const unsigned long long *__restrict__ key,
 // directly instead of chasing skip pointers one after another.  Also records
 // each child's parent slot (TopArgs::parent, TopArgs::bparent), by which the
 // moment pass climbs the top tree.
-__global__ void k_top_children(int nb, const unsigned long long *__restrict__ key,
-                               const int4 *__restrict__ blk, const int *__restrict__ count,
-                               const int *__restrict__ prestart, int64_t n_nodes,
-                               const int *__restrict__ fstart, const int *__restrict__ fid,
-                               const int *__restrict__ orig, TopArgs top, unsigned *flags) {
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (int64_t)nb * 8) return;
-  const int p = (int)(tid >> 3), o = (int)(tid & 7);
-  const int r = blockIdx.y;
+__device__ __forceinline__ void top_child(int p, int o, int r, const unsigned long long *key,
+                                          const int4 *blk, const int *count, const int *prestart,
+                                          int64_t n_nodes, const int *fstart, const int *fid,
+                                          const int *orig, const TopArgs &top, unsigned *flags) {
   const int cnt = count[p];
   if (r >= cnt) return;
   const int lb = blk[p].x, k = lb - cnt + r;
@@ -380,6 +391,76 @@ __global__ void k_top_children(int nb, const unsigned long long *__restrict__ ke
   } else {  // block q's root
     top.bparent[q] = (int)slot;
   }
+}
+
+__global__ void k_top_children(int nb, const unsigned long long *key, const int4 *blk,
+                               const int *count, const int *prestart, int64_t n_nodes,
+                               const int *fstart, const int *fid, const int *orig, TopArgs top,
+                               unsigned *flags) {
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid >= (int64_t)nb * 8) return;
+  top_child((int)(tid >> 3), (int)(tid & 7), blockIdx.y, key, blk, count, prestart, n_nodes,
+            fstart, fid, orig, top, flags);
+}
+
+// The geometry of a small block list in one launch, one block per thread:
+// what k_sort_blocks, k_tile_and_count, k_prestart_scan, k_top_nodes and
+// k_top_children do in five (2-5 us each, all launch and memory latency).  The
+// sort, when it is needed, counts for every block how many come before it in
+// its field.  Measured, a whole build:
+// 15 blocks 83 -> 69 us, 64 blocks 88 -> 72 us.
+constexpr int kSmallBlocks = 512;
+__global__ void __launch_bounds__(kSmallBlocks)
+    k_small_geometry(int nb, unsigned long long *key, int *idx, const int *level, const int *ijk,
+                     int *count, int *prestart, int4 *blk, int *orig, int *pos, int64_t n_nodes,
+                     WalkRec *rec, float2 *aux, uint8_t *lvl, unsigned *flags, const int *fstart,
+                     const int *fid, int4 *fld, int max_level, TopArgs top) {
+  __shared__ unsigned long long keys[kSmallBlocks];
+  __shared__ int warp_sum[kSmallBlocks / 32];
+  const int t = threadIdx.x, lane = t & 31;
+  if (flags[1] != 0u) {  // (keys of caller blocks are in caller order so far)
+    int f = 0, to = 0;
+    unsigned long long k = 0ull;
+    if (t < nb) keys[t] = k = key[t];
+    __syncthreads();
+    if (t < nb) {
+      f = fid[t];
+      to = fstart[f];
+      for (int q = fstart[f]; q < fstart[f + 1]; ++q) to += keys[q] < k || (keys[q] == k && q < t);
+      key[to] = k;
+      idx[to] = t;
+    }
+    __syncthreads();
+  }
+  int c = 0;
+  if (t < nb) {
+    tile_and_count(t, key, idx, level, ijk, count, blk, orig, flags, fstart, fid, pos, top.bparent);
+    c = count[t];
+  }
+  int incl = c;  // top nodes before block t: an exclusive scan
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) warp_sum[t >> 5] = incl;
+  __syncthreads();
+  int before = 0, total = 0;
+#pragma unroll
+  for (int w = 0; w < kSmallBlocks / 32; ++w) {
+    before += w < (t >> 5) ? warp_sum[w] : 0;
+    total += warp_sum[w];
+  }
+  if (t < nb) prestart[t] = kNodesPerBlock * t + before + incl - c;
+  if (t == 0) flags[2] = (unsigned)total;
+  __syncthreads();
+  if (t < nb)
+    top_nodes_of(t, nb, key, blk, count, prestart, n_nodes, rec, aux, lvl, flags, fstart, fid, orig,
+                 fld, top);
+  __syncthreads();
+  for (int i = t; i < 8 * nb * max_level; i += kSmallBlocks)  // (top node, octant) pairs
+    top_child((i >> 3) % nb, i & 7, (i >> 3) / nb, key, blk, count, prestart, n_nodes, fstart, fid,
+              orig, top, flags);
 }
 
 // Moments of one internal node from its 8 children (Eq. 5), children in
@@ -1134,13 +1215,26 @@ cudaError_t launch_top_nodes(cudaStream_t s, int nb, const unsigned long long *k
                              unsigned *flags, const FieldArgs &fa, const int *orig,
                              int max_level, const TopArgs &top) {
   k_top_nodes<<<grid_for(nb, 256), 256, 0, s>>>(nb, key, blk, count, prestart, n_nodes, rec,
-                                                 aux, lvl, flags, fa.nfields, fa.fstart, fa.fid,
-                                                 orig, fa.fld, top);
+                                                 aux, lvl, flags, fa.fstart, fa.fid, orig, fa.fld,
+                                                 top);
   if (max_level > 0) {  // a block starts at most max_level top nodes
     const dim3 grid((unsigned)grid_for((int64_t)nb * 8, 256), (unsigned)max_level);
     k_top_children<<<grid, 256, 0, s>>>(nb, key, blk, count, prestart, n_nodes, fa.fstart,
                                          fa.fid, orig, top, flags);
   }
+  return cudaGetLastError();
+}
+
+bool small_geometry(int nb) { return nb <= kSmallBlocks; }
+
+cudaError_t launch_small_geometry(cudaStream_t s, int nb, unsigned long long *key, int *idx,
+                                  const int *level, const int *ijk, int *count, int *prestart,
+                                  int4 *blk, int *orig, int *pos, int64_t n_nodes, WalkRec *rec,
+                                  float2 *aux, uint8_t *lvl, unsigned *flags, const FieldArgs &fa,
+                                  int max_level, const TopArgs &top) {
+  k_small_geometry<<<1, kSmallBlocks, 0, s>>>(nb, key, idx, level, ijk, count, prestart, blk, orig,
+                                              pos, n_nodes, rec, aux, lvl, flags, fa.fstart, fa.fid,
+                                              fa.fld, max_level, top);
   return cudaGetLastError();
 }
 

@@ -184,19 +184,16 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   fa.L = d_box;
   fa.invL = d_box + 1;
   fa.mmax = (unsigned long long *)(base + kOffMmax);
-  fa.inv_theta = 0.0f;  // s2 is prepared below
+  fa.inv_theta = (float)(1.0 / theta);  // the moments come with their opening radii
 
   k_stage_geometry<<<1, 256, 0, s>>>(g, nb, d_level, d_ijk, d_flags, d_fstart, max_level, d_box,
                                      box_len, fa.mmax);
   NA_CUDA(cudaGetLastError());
   NA_CUDA(launch_keys_mass(s, nb, d_level, d_ijk, d_key[0], d_idx[0], d_flags, fa, density,
                            density_is_fp64));
-  NA_CUDA(launch_sort_blocks(s, d_key, d_idx, d_flags, fa));
-  NA_CUDA(launch_tile_and_count(s, nb, d_key[0], d_idx[0], d_level, d_ijk, d_count, d_blk,
-                                d_orig, d_flags, fa, top));
-  NA_CUDA(launch_prestart_scan(s, nb, d_count, d_prestart, d_flags));
-  NA_CUDA(launch_top_nodes(s, nb, d_key[0], d_blk, d_count, d_prestart, n_nodes, d_rec, d_aux,
-                           d_lvl, d_flags, fa, d_orig, max_level, top));
+  NA_CUDA(launch_small_geometry(s, nb, d_key[0], d_idx[0], d_level, d_ijk, d_count, d_prestart,
+                                d_blk, d_orig, nullptr, n_nodes, d_rec, d_aux, d_lvl, d_flags, fa,
+                                max_level, top));
   NA_CUDA(launch_moments(s, nb, d_blk, d_orig, d_count, d_prestart, density,
                          density_is_fp64, fa, n_nodes, d_mom, d_rec, d_aux, d_lvl, nullptr, nullptr,
                          d_flags, top, sib));
@@ -207,8 +204,6 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   if (h_flags[0] & (kErrLevel | kErrCoord | kErrTiling | kErrIndex)) return BH_ERR_GEOMETRY;
   if ((int64_t)h_flags[2] != (nb - 1) / 7) return BH_ERR_GEOMETRY;
   if (h_flags[0] & kErrDensity) return BH_ERR_ARG;
-  NA_CUDA(launch_prepare_s2(s, n_nodes, d_aux, d_rec, kSibsPerBlock * nb + 8 * ((nb - 1) / 7),
-                            sib.sib, (float)(1.0 / theta)));
   bh_options opt;
   bh_default_options(&opt);
   WalkShape shape;

@@ -69,3 +69,19 @@ def test_deep_and_shallow_fields_keep_their_bits_in_a_batch(quad):
         want = a.potential(0.4).cpu().numpy()
         assert np.array_equal(got[at:at + want.size], want)
         at += want.size
+
+
+@pytest.mark.parametrize("level,extra", [(0, 0), (0, 1), (3, 0), (3, 1)])
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_block_lists_around_the_small_geometry_limit(level, extra, shuffled):
+    """1, 8, 512 (the most that one launch takes) and 519 blocks, in Morton
+    order and shuffled: the oracle's tree and masses, bit for bit."""
+    m, rho = field(level, extra, 77)
+    if shuffled:
+        m, rho = mg.shuffled(m, rho, seed=3)
+    t = O.Tree(m.level, m.ijk, rho.astype(np.float64)).export()
+    s = B.Solver()
+    s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+    e = {k: v.cpu().numpy() for k, v in s.export_nodes().items()}
+    assert np.array_equal(e["level"], t["level"]) and np.array_equal(e["M"], t["M"])
+    assert np.array_equal(e["R"], t["R"])
