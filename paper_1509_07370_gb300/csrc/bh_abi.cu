@@ -414,10 +414,9 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
                                        n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa,
                                        max_level, top));
   } else {
-    BH_CUDA(bhg::launch_sort_blocks(s, t.d_key, t.d_idx, t.d_flags, fa));
-    BH_CUDA(bhg::launch_tile_and_count(s, nb, t.d_key[0], t.d_idx[0], t.d_level, t.d_ijk,
-                                       t.d_count, t.d_blk, t.d_orig, t.d_flags, fa, top,
-                                       t.d_pos));
+    BH_CUDA(bhg::launch_sort_blocks(s, nb, t.d_key, t.d_idx, t.d_flags, fa));
+    BH_CUDA(bhg::launch_tile_and_count(s, nb, t.d_key, t.d_idx, t.d_level, t.d_ijk, t.d_count,
+                                       t.d_blk, t.d_orig, t.d_flags, fa, top, t.d_pos));
     BH_CUDA(bhg::launch_prestart_scan(s, nb, t.d_count, t.d_prestart, t.d_flags));
   }
   // the top nodes' records and child lists (needed from k_upper_tree on) on

@@ -103,10 +103,51 @@ __device__ __forceinline__ void key_of_block(int b, int f, const int *__restrict
   }
 }
 
-// Stable LSD radix sort of (key, idx), one CTA per field (its segment of the
-// block list), 4 bits per pass, 16 passes, result back in buffer 0.  Block
-// lists are small (a 16M-cell mesh has ~32k blocks), and the sort only runs
-// when the caller's block order is not already the Morton order.
+// The sort only runs when the caller's block order is not already the Morton
+// order.  Up to kCountBlocks blocks it counts for every block how many of its
+// field come before it (k_rank_blocks: lane = block, the warps of a CTA share
+// the field's keys), into buffer 1; every comparison is independent, so all SMs
+// take part: 3,984 blocks 24 us instead of 234 by the radix sort's one CTA,
+// 31,816 blocks 0.35 ms instead of 1.6.  The count grows with the square
+// of the list: longer ones keep the stable LSD radix sort, one CTA per field
+// (its segment of the block list), 4 bits per pass, 16 passes, result back in
+// buffer 0.
+constexpr int kCountBlocks = 1 << 16;
+constexpr int kRankWarps = 8;
+__global__ void __launch_bounds__(32 * kRankWarps)
+    k_rank_blocks(int nb, const int *__restrict__ fstart, const int *__restrict__ fid,
+                  const unsigned long long *__restrict__ k0, unsigned long long *__restrict__ k1,
+                  int *__restrict__ v1, const unsigned *__restrict__ flags) {
+  if (flags[1] == 0u) return;  // already sorted
+  __shared__ int part[kRankWarps][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int b = blockIdx.x * 32 + lane;
+  int before = 0, from = 0;
+  unsigned long long k = 0ull;
+  if (b < nb) {
+    k = k0[b];
+    const int f = fid[b];
+    from = fstart[f];
+    const int n = fstart[f + 1] - from;
+    const int lo = from + (int)((int64_t)n * w / kRankWarps);
+    const int hi = from + (int)((int64_t)n * (w + 1) / kRankWarps);
+#pragma unroll 8
+    for (int q = lo; q < hi; ++q) {
+      const unsigned long long kq = k0[q];
+      before += kq < k || (kq == k && q < b);
+    }
+  }
+  part[w][lane] = before;
+  __syncthreads();
+  if (w == 0 && b < nb) {
+    int to = from;
+#pragma unroll
+    for (int i = 0; i < kRankWarps; ++i) to += part[i][lane];
+    k1[to] = k;
+    v1[to] = b;
+  }
+}
+
 constexpr int kSortThreads = 512;
 __global__ void __launch_bounds__(kSortThreads)
     k_sort_blocks(const int *__restrict__ fstart, unsigned long long *k0, int *v0,
@@ -204,15 +245,24 @@ __device__ __forceinline__ void tile_and_count(int p, const unsigned long long *
   orig[p] = b;
 }
 
-__global__ void k_tile_and_count(int nb, const unsigned long long *__restrict__ key,
-                                 const int *__restrict__ idx, const int *__restrict__ level,
+__global__ void k_tile_and_count(int nb, unsigned long long *key, int *idx,
+                                 const int *__restrict__ level,
                                  const int *__restrict__ ijk, int *__restrict__ count,
                                  int4 *__restrict__ blk, int *__restrict__ orig,
                                  unsigned *flags, const int *__restrict__ fstart,
                                  const int *__restrict__ fid, int *__restrict__ pos,
-                                 int *__restrict__ bparent) {
+                                 int *__restrict__ bparent,
+                                 const unsigned long long *__restrict__ ranked_key,
+                                 const int *__restrict__ ranked_idx) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= nb) return;
+  if (ranked_key && flags[1] != 0u) {  // k_rank_blocks left the sorted list in buffer 1
+    key[p] = ranked_key[p];
+    idx[p] = ranked_idx[p];
+    tile_and_count(p, ranked_key, ranked_idx, level, ijk, count, blk, orig, flags, fstart, fid,
+                   pos, bparent);
+    return;
+  }
   tile_and_count(p, key, idx, level, ijk, count, blk, orig, flags, fstart, fid, pos, bparent);
 }
 
@@ -1234,19 +1284,25 @@ cudaError_t launch_keys_mass(cudaStream_t s, int nb, const int *level, const int
   return cudaGetLastError();
 }
 
-cudaError_t launch_sort_blocks(cudaStream_t s, unsigned long long *key[2], int *idx[2],
+cudaError_t launch_sort_blocks(cudaStream_t s, int nb, unsigned long long *key[2], int *idx[2],
                                unsigned *flags, const FieldArgs &fa) {
-  k_sort_blocks<<<fa.nfields, kSortThreads, 0, s>>>(fa.fstart, key[0], idx[0], key[1], idx[1],
-                                                     flags);
+  if (nb <= kCountBlocks)
+    k_rank_blocks<<<grid_for(nb, 32), 32 * kRankWarps, 0, s>>>(nb, fa.fstart, fa.fid, key[0], key[1],
+                                                              idx[1], flags);
+  else
+    k_sort_blocks<<<fa.nfields, kSortThreads, 0, s>>>(fa.fstart, key[0], idx[0], key[1], idx[1],
+                                                      flags);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tile_and_count(cudaStream_t s, int nb, const unsigned long long *key,
-                                  const int *idx, const int *level, const int *ijk, int *count,
-                                  int4 *blk, int *orig, unsigned *flags, const FieldArgs &fa,
+cudaError_t launch_tile_and_count(cudaStream_t s, int nb, unsigned long long *key[2], int *idx[2],
+                                  const int *level, const int *ijk, int *count, int4 *blk,
+                                  int *orig, unsigned *flags, const FieldArgs &fa,
                                   const TopArgs &top, int *pos) {
-  k_tile_and_count<<<grid_for(nb, 256), 256, 0, s>>>(nb, key, idx, level, ijk, count, blk, orig,
-                                                      flags, fa.fstart, fa.fid, pos, top.bparent);
+  const bool ranked = nb <= kCountBlocks;  // as launch_sort_blocks chose
+  k_tile_and_count<<<grid_for(nb, 256), 256, 0, s>>>(
+      nb, key[0], idx[0], level, ijk, count, blk, orig, flags, fa.fstart, fa.fid, pos, top.bparent,
+      ranked ? key[1] : nullptr, ranked ? idx[1] : nullptr);
   return cudaGetLastError();
 }
 

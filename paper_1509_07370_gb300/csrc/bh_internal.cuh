@@ -296,12 +296,12 @@ __host__ __device__ inline double pow2i(int e) {
 cudaError_t launch_keys_mass(cudaStream_t s, int nb, const int *level, const int *ijk,
                              unsigned long long *key, int *idx, unsigned *flags,
                              const FieldArgs &fa, const void *density, int density_is_fp64);
-cudaError_t launch_sort_blocks(cudaStream_t s, unsigned long long *key[2], int *idx[2],
+cudaError_t launch_sort_blocks(cudaStream_t s, int nb, unsigned long long *key[2], int *idx[2],
                                unsigned *flags, const FieldArgs &fa);
-cudaError_t launch_tile_and_count(cudaStream_t s, int nb, const unsigned long long *key,
-                                  const int *idx, const int *level, const int *ijk,
-                                  int *count, int4 *blk, int *orig, unsigned *flags,
-                                  const FieldArgs &fa, const TopArgs &top, int *pos = nullptr);
+cudaError_t launch_tile_and_count(cudaStream_t s, int nb, unsigned long long *key[2], int *idx[2],
+                                  const int *level, const int *ijk, int *count, int4 *blk,
+                                  int *orig, unsigned *flags, const FieldArgs &fa,
+                                  const TopArgs &top, int *pos);
 cudaError_t launch_prestart_scan(cudaStream_t s, int nb, const int *count, int *prestart,
                                  unsigned *flags);
 // Skip pointers of the top nodes and their lists (TopArgs); max_level = the

@@ -1,5 +1,5 @@
 """Tree construction where its branches meet: masses and products that are
-exact in binary64 beside ones that round.
+exact in binary64 beside ones that round, and the two block sorts.
 
 Bar: the oracle's masses, centres of mass and extents, bit for bit."""
 import numpy as np
@@ -43,3 +43,52 @@ def test_moments_of_exact_and_rounded_products(box_len, dtype, level, extra):
     t["delta"] = t["delta"].astype(np.float32)
     for k in ("M", "R", "delta"):
         assert np.array_equal(e[k], t[k]), k
+
+
+def test_shuffled_fields_of_a_batch_are_sorted_by_themselves():
+    """1, 519 and 8 blocks, listed in random order, in one batch: the sort
+    counts each field's blocks alone."""
+    rng = np.random.Generator(np.random.PCG64(9))
+    fs = []
+    for i, (level, extra) in enumerate([(0, 0), (3, 1), (1, 0)]):
+        m = corner(level, extra)
+        fs.append(mg.shuffled(m, rng.lognormal(size=(m.nblocks, 8, 8, 8)).astype(np.float32), i))
+    s = B.Solver()
+    s.build_batch([m.nblocks for m, _ in fs], np.concatenate([m.level for m, _ in fs]),
+                  np.concatenate([m.ijk for m, _ in fs]),
+                  torch.as_tensor(np.concatenate([r.reshape(-1) for _, r in fs])).cuda())
+    e = {k: v.cpu().numpy() for k, v in s.export_nodes().items()}
+    at = 0
+    for m, rho in fs:
+        t = O.Tree(m.level, m.ijk, rho.astype(np.float64)).export()
+        n = t["M"].size
+        assert np.array_equal(e["M"][at:at + n], t["M"]) and np.array_equal(e["R"][at:at + n], t["R"])
+        at += n
+    assert at == e["M"].size
+
+
+@pytest.mark.parametrize("split", [4681, 4682])
+def test_both_sorts_restore_the_morton_order(split):
+    """65,535 blocks (sorted by counting) and 65,542 (by radix), listed in
+    random order: the tree of the list in Morton order, whose potentials and
+    masses the other tests compare with the oracle."""
+    ijk = np.stack(np.meshgrid(*[np.arange(32)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    fine = (2 * ijk[:split, None, :] + np.indices((2, 2, 2)).reshape(3, 8).T).reshape(-1, 3)
+    lev = np.r_[np.full(len(ijk) - split, 5), np.full(len(fine), 6)].astype(np.int32)
+    ijk = np.concatenate([ijk[split:], fine]).astype(np.int32)
+    corner_key = np.zeros(len(lev), np.int64)  # Morton key of the lower corner at level 6
+    c = ijk.astype(np.int64) << (6 - lev)[:, None]
+    for b in range(6):
+        for d in range(3):
+            corner_key |= ((c[:, d] >> b) & 1) << (3 * b + d)
+    order = np.argsort(corner_key)
+    lev, ijk = lev[order], ijk[order]
+    rho = torch.rand((len(lev), 512), generator=torch.Generator().manual_seed(1))
+    trees = []
+    for p in (np.arange(len(lev)), np.random.default_rng(2).permutation(len(lev))):
+        s = B.Solver()
+        s.build(np.ascontiguousarray(lev[p]), np.ascontiguousarray(ijk[p]),
+                rho[torch.as_tensor(p)].reshape(-1).cuda())
+        trees.append(s.export_nodes())
+    for k in ("level", "M", "R"):
+        assert torch.equal(trees[0][k], trees[1][k]), k
