@@ -7,20 +7,19 @@
 // 1. Testing.  The warp pops up to four opened nodes from its stack in shared
 //    memory and tests their 32 children, one child per lane: the lane forms
 //    the opening test of Eq. 4 for all 64 targets and gets a 64-bit mask.
-//    Children are addressed directly (inside a block by the strides of the
-//    585-node pre-order subtree, above it by the top-node child lists).  With
+//    Siblings lie together (WalkSib), so that 8 lanes read 8 neighbours.  With
 //    P the targets that opened the parent, the targets accepting the child
 //    are A = P & mask, those opening it O = P & ~mask.  A child with A != 0
 //    is staged in shared memory; a child with O != 0 goes on the stack with P
 //    = O, or, if it is a bottom node (its 8 children are cells), to the list
 //    of opened bottom nodes.  Cells are never tested.
 // 2. Evaluating.  Four sub-bricks of 16 cells (4x2x2) each have a list of the
-//    staged nodes that one of their cells accepts, with the 16-bit mask, and
-//    a list of opened bottom nodes.  8 lanes serve a sub-brick: lane bits 0-1
-//    take every fourth list entry, bit 2 is the cell's z within the sub-brick,
-//    and a lane owns the 8 cells (4 in x, 2 in y) of that z.  So a warp
-//    evaluates 16 different (node, 8 cells) pairs at a time, each lane
-//    loading a record once for 8 interactions.
+//    staged nodes that one of their cells accepts, with the 16-bit mask.  8
+//    lanes serve a sub-brick: lane bits 0-1 take every fourth list entry, bit
+//    2 is the cell's z within the sub-brick, and a lane owns the 8 cells (4 in
+//    x, 2 in y) of that z.  So a warp evaluates 16 different (node, 8 cells)
+//    pairs at a time, each lane loading a record once for 8 interactions.
+//    Opened bottom nodes are met row by row (eval_cells).
 //
 // Each target visits exactly the nodes of its own recursive walk and takes
 // the decisions of the per-cell definition (or, with the warp vote, those of
@@ -39,13 +38,13 @@
 // but then every lane reads its own record, and the shared-memory return path
 // bounds the quadrupole walk).
 //
-// Measured (2,039,808-cell spheroid, plain grid of 4-warp CTAs; ms, with in
-// brackets the walk that stepped 64 targets, or 32 with the vote, through the
-// tree together): quadrupole theta 0.75 1.08 (1.85), monopole 0.5 2.07 (3.2)
-// and 0.24 11.0 (15.5), vote with quadrupole 0.8 1.01 (2.49); 16.3M-cell core,
-// monopole 0.5 20.0 (27.4); 32^3 cells 0.106 (0.45): there a warp has a
-// scheduler to itself, and a step tests 32 nodes per chain of dependent loads
-// instead of one.
+// Measured (2,039,808-cell spheroid, persistent grid of 4-warp CTAs, groups in
+// their own order; ms, with in brackets the walk that stepped 64 targets, or
+// 32 with the vote, through the tree together, on its plain grid): quadrupole
+// theta 0.75 0.96 (1.85), monopole 0.5 1.92 (3.2) and 0.24 10.7 (15.5), vote
+// with quadrupole 0.8 0.91 (2.49); 16.3M-cell core, monopole 0.5 18.6 (27.4);
+// 32^3 cells 0.093 (0.45): there a warp has a scheduler to itself, and a step
+// tests 32 nodes per chain of dependent loads instead of one.
 //
 // The opening test is evaluated in binary32 with the operation order stated
 // in the public header; the interaction uses the same d2 formed again.  (The
@@ -56,9 +55,10 @@ namespace bhg {
 namespace {
 
 constexpr int kMaxWalkThreads = 512;  // largest tunable CTA
-// 80 registers: 24 warps per SM (97 without the bound, 20 warps: 8 % slower;
-// 72: 28 warps, spills: 2-5 % slower).
-constexpr int kWalkRegs = 80;
+// Registers.  Monopole: 80, 24 warps per SM (97 without a bound, 20 warps: 8 %
+// slower; 72 spills: 2-5 % slower).  Quadrupole: shared memory allows 16 warps
+// whatever the registers, so 112 (80: 3.6 % slower; 128: 1 %).
+constexpr int walk_regs(bool quad) { return quad ? 112 : 80; }
 constexpr int kDefaultWarps = 4;
 
 __global__ void k_prepare_sib_s2(int64_t n, WalkSib *__restrict__ sib, float inv_theta) {
@@ -78,8 +78,15 @@ __global__ void k_prepare_s2(int64_t n, const float2 *__restrict__ aux, WalkRec 
 }
 
 // ---- binary32 walk -----------------------------------------------------------
-constexpr int kRing = 64;     // staged nodes, a ring: room for one more chunk is kept
-constexpr int kBottoms = 64;   // opened bottom nodes: evaluated once a chunk might not fit
+// Staged nodes (a ring; room for one more step's is kept) and opened bottom
+// nodes (evaluated once a step's might not fit).  Longer lists lose less where
+// the sub-bricks' or rows' lists differ in length, and are evaluated in fewer
+// and longer runs, which is worth more than the warps per SM that their shared
+// memory costs (quadrupole 24 -> 16): 64 and 64 entries take 5.5 % longer on the
+// core and the spheroid at theta 0.5, 7 % on the quadrupole walk.
+constexpr int kRing = 128;
+constexpr int kBottoms = 96;
+
 struct QuadRest {                    // second half of a staged quadrupole (16-byte stride)
   float qxz, qyz, unused[2];
 };
@@ -122,26 +129,29 @@ __device__ __forceinline__ float rsqrt_above(float d, float least) {
   return r;
 }
 
-// Compensated sums of products.  One: s = fl(sum + a b), err = fl((sum - s) +
-// a b); two: s = the sum with both added in turn, err = ((sum - s) + a1 b1) +
-// a0 b0, the products unrounded in both (sum - s is exact while the sum is
-// the larger; all terms are positive).  4 and 6 operations; rounding the
-// products and compensating each (accumulate2) takes 5 and 10, with the same
-// error against binary64 (2.76e-8 of the potential on 32^3 cells at theta
-// 0.5; 2.77e-8 with the two-product form; rounding the result alone gives
-// 2.5e-8).
+// sum + comp += a b, compensated, the product unrounded: s = the sum with it
+// added, err = (sum - s) + a b, exact where the sum is the larger (all terms
+// are positive).  So that it is from the first term on, a lane's sums start
+// from sum_base, which is taken off before they are merged.  Relative error
+// of the potential against binary64 on 32^3 cells at theta 0.5: 2.757e-8, of
+// which rounding the result is 2.5e-8; from zero 2.763e-8 (the early terms of
+// four lanes' sums, where the walk that kept a target in one lane had 2.762e-8);
+// two products to a compensation, 2 % faster, 2.765e-8.
 template <bool KAHAN>
 __device__ __forceinline__ void accumulate_product2(u64 &sum, u64 &comp, u64 a, u64 b) {
   const u64 s = fma2(a, b, sum);
   if (KAHAN) comp = add2(comp, fma2(a, b, sub2(sum, s)));
   sum = s;
 }
+// Four times the power of two at or below the field's mass: above any term
+// (a mass over a distance) but those of a few cells next to a target that
+// hold most of the field's mass, and a power of two, so that sum - sum_base
+// is exact.
 template <bool KAHAN>
-__device__ __forceinline__ void accumulate_products2(u64 &sum, u64 &comp, u64 a0, u64 b0, u64 a1,
-                                                     u64 b1) {
-  const u64 s = fma2(a1, b1, fma2(a0, b0, sum));
-  if (KAHAN) comp = add2(comp, fma2(a0, b0, fma2(a1, b1, sub2(sum, s))));
-  sum = s;
+__device__ __forceinline__ u64 sum_base(float mass) {
+  if (!KAHAN) return 0ull;
+  const float b = 4.0f * __uint_as_float(__float_as_uint(mass) & 0x7f800000u);
+  return pk(b, b);
 }
 
 struct Targets {          // of one lane, read back before every evaluation
@@ -212,23 +222,6 @@ __device__ __forceinline__ void eval_nodes(const WalkMem<QUAD> &S, int sb, unsig
     return;
   }
   Entry<QUAD> a, b;
-  if (QUAD) {  // one after the other: together they would take more than 80 registers
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      a.load(S, e ? v1 : v0, zsh, T);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        a.row(T.ty[r]);
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          u64 rr, t;
-          a.terms(r, k, rr, t);
-          accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], rr, t);
-        }
-      }
-    }
-    return;
-  }
   a.load(S, v0, zsh, T);
   b.load(S, v1, zsh, T);
 #pragma unroll
@@ -240,7 +233,8 @@ __device__ __forceinline__ void eval_nodes(const WalkMem<QUAD> &S, int sb, unsig
       u64 ra, ta, rb, tb;
       a.terms(r, k, ra, ta);
       b.terms(r, k, rb, tb);
-      accumulate_products2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], ra, ta, rb, tb);
+      accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], ra, ta);
+      accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], rb, tb);
     }
   }
 }
@@ -263,7 +257,7 @@ __device__ __forceinline__ u64 two_sum2(u64 a, u64 b, u64 &e) {
 template <bool KAHAN, bool COUNTS, bool QUAD>
 __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
                                            const float4 *__restrict__ cmass, int n, int lane,
-                                           Lane<COUNTS> &L) {
+                                           u64 base, Lane<COUNTS> &L) {
   constexpr int W = kBottoms / 32;
   const int row = lane & 15, word = 1 + (row >> 3), sh = 4 * (row & 7), zhalf = lane >> 4;
   uint32_t mine[W];  // bottom nodes some target of the row opened
@@ -282,7 +276,7 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
 #pragma unroll
   for (int w = 0; w < W; ++w) left += __popc(mine[w]);
   const int steps = (int)__reduce_max_sync(kFull, (unsigned)left);
-  u64 sum[2] = {0ull, 0ull}, comp[2] = {0ull, 0ull};
+  u64 sum[2] = {base, base}, comp[2] = {0ull, 0ull};
   int nb[4] = {0, 0, 0, 0};
   const u64 tx[2] = {pk(S.front.tx[0].x, S.front.tx[0].z), pk(S.front.tx[1].x, S.front.tx[1].z)};
   const float ty = S.front.coord(16 + 2 * ((row >> 2) & 1) + (row & 1));
@@ -347,6 +341,7 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
 #pragma unroll
   for (int k = 0; k < 2; ++k) {
     u64 e = 0ull;
+    sum[k] = sub2(sum[k], base);
     const u64 o = __shfl_xor_sync(kFull, sum[k], 16);
     if (KAHAN) {
       sum[k] = (lane & 16) ? two_sum2(o, sum[k], e) : two_sum2(sum[k], o, e);
@@ -410,9 +405,13 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
   const int par = lane & 3, zl = (lane >> 2) & 1, sb = lane >> 3;
   const unsigned lower = (1u << lane) - 1u;
   front_start(S.front, octant_at(B, o), F, p, lane, A.rec, A.sib.tops);
+  const u64 base = sum_base<KAHAN>(A.rec[F.x].m);
   Lane<COUNTS> L;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) L.sum[i] = L.comp[i] = 0ull;
+  for (int i = 0; i < 4; ++i) {
+    L.sum[i] = base;
+    L.comp[i] = 0ull;
+  }
 #pragma unroll
   for (int i = 0; i < (COUNTS ? 8 : 1); ++i) L.na[i] = L.nb[i] = 0;
   const int zsh = 16 + 8 * zl;
@@ -496,7 +495,7 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
       for (int j = lane; j < nbot; j += 32) S.centre[j] = bottom_centre(S.bottom[0][j], A.blk);
       __syncwarp();
       eval_cells<KAHAN, COUNTS, QUAD>(S, reinterpret_cast<const float4 *>(A.sib.cmass), nbot, lane,
-                                      L);
+                                      base, L);
       nbot = 0;
       __syncwarp();
     }
@@ -533,6 +532,7 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
     const float scale = (float)(-A.G * A.invL[F.w] * pow2i(mass_exponent(A.mmax[F.w])));
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
+      L.sum[i] = sub2(L.sum[i], base);
       merge_lanes<KAHAN>(L.sum[i], L.comp[i]);
       if (i == par) {
         float sa, sb_;
@@ -547,7 +547,7 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
 // A unit of work is one octant (np = 1) or two neighbouring ones, walked one
 // after the other (np = 2).  Plain grid: warp i walks unit order[i] (or i).
 template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
-__global__ void __maxnreg__(kWalkRegs)
+__global__ void __maxnreg__(walk_regs(QUAD))
     k_walk_lists(unsigned nunits, int np, const unsigned *__restrict__ order, const WalkArgs A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   WalkMem<QUAD> &S = reinterpret_cast<WalkMem<QUAD> *>(smem_raw)[threadIdx.x >> 5];
@@ -567,7 +567,7 @@ __global__ void __maxnreg__(kWalkRegs)
 // running alone at the end of the launch.  cycles (or null): the SM clock
 // cycles of each unit's walk, the measurement that order is made from.
 template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
-__global__ void __maxnreg__(kWalkRegs)
+__global__ void __maxnreg__(walk_regs(QUAD))
     k_walk_queue(unsigned nunits, int np, unsigned per_ticket, unsigned *__restrict__ counter,
                  const unsigned *__restrict__ order, unsigned long long *__restrict__ cycles,
                  const WalkArgs A) {
