@@ -90,6 +90,50 @@ __device__ __forceinline__ void test64(const Front &S, float px, float py, float
   }
 }
 
+// The same test for the part of the targets that one of SPLIT warps holds: x =
+// 2 k0, 2 k0 + 1 and, with SPLIT = 4, y = r0, r0 + 2; the other bits are clear.
+template <int SPLIT>
+__device__ __forceinline__ void test_part(const Front &S, int r0, int k0, float px, float py,
+                                          float pz, float s2, uint32_t m[2]) {
+  const float4 xx = S.tx[k0], z01 = S.tz[0], z23 = S.tz[1];
+  const u64 pyy = pk(py, py), pzz = pk(pz, pz), ss = pk(s2, s2);
+  const u64 dx[2] = {sub2(pk(xx.x, xx.y), pk(px, px)), sub2(pk(xx.z, xx.w), pk(px, px))};
+  const u64 dz[4] = {sub2(pk(z01.x, z01.y), pzz), sub2(pk(z01.z, z01.w), pzz),
+                     sub2(pk(z23.x, z23.y), pzz), sub2(pk(z23.z, z23.w), pzz)};
+  constexpr int NY = SPLIT == 4 ? 1 : 2;  // y pairs {r0, r0 + 2} or {0, 1}, {2, 3}
+  u64 yy[NY];
+#pragma unroll
+  for (int i = 0; i < NY; ++i) {
+    const u64 dy = sub2(SPLIT == 4 ? pk(S.coord(16 + r0), S.coord(18 + r0))
+                                   : pk(S.coord(16 + 2 * i), S.coord(17 + 2 * i)), pyy);
+    yy[i] = mul2(dy, dy);
+  }
+#pragma unroll
+  for (int w = 0; w < 2; ++w) {
+    float v[4][2][2];  // [y][z & 1][x]
+#pragma unroll
+    for (int zl = 0; zl < 2; ++zl)
+#pragma unroll
+      for (int i = 0; i < NY; ++i) {
+        const u64 h = fma2(dz[2 * w + zl], dz[2 * w + zl], yy[i]);
+#pragma unroll
+        for (int x = 0; x < 2; ++x)
+          upk(sub2(ss, fma2(dx[x], dx[x], h)), v[2 * i][zl][x], v[2 * i + 1][zl][x]);
+      }
+    uint32_t b = 0u;
+#pragma unroll
+    for (int yh = 1; yh >= 0; --yh)
+#pragma unroll
+      for (int zl = 1; zl >= 0; --zl)
+#pragma unroll
+        for (int r = NY - 1; r >= 0; --r) {
+          const int y = SPLIT == 4 ? yh : 2 * yh + r;
+          b = push_sign(push_sign(b << (SPLIT == 4 ? 6 : 2), v[y][zl][1]), v[y][zl][0]);
+        }
+    m[w] = b << ((SPLIT == 4 ? 4 * r0 : 0) + 2 * k0);
+  }
+}
+
 // One octant's place in the mesh.
 struct Octant {
   int ox, oy, oz;   // lowest cell of the octant in its level's lattice
@@ -136,10 +180,11 @@ struct Tested {
 
 // Pops up to four opened nodes, tests their children, and pushes those that
 // some target opens (bottom nodes excepted).  With VOTE the targets of each
-// 32-cell brick (a word of the mask) accept only together.
-template <bool VOTE, bool WRAP = false>
+// 32-cell brick (a word of the mask) accept only together.  test(a, s2, m)
+// makes the mask.
+template <bool VOTE, class Test>
 __device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int lane,
-                                             const WalkSib *__restrict__ sib) {
+                                             const WalkSib *__restrict__ sib, const Test &test) {
   const int pop = depth > pop4 ? 1 : (depth < 4 ? depth : 4);
   const bool valid = (lane >> 3) < pop;
   uint2 P = make_uint2(0u, 0u);
@@ -155,7 +200,7 @@ __device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int
   }
   depth -= pop;
   uint32_t m[2];
-  test64<WRAP>(S, a.x, a.y, a.z, b.x, m);
+  test(a, b.x, m);
   if (VOTE) {
     m[0] = m[0] == kFull ? kFull : 0u;
     m[1] = m[1] == kFull ? kFull : 0u;
@@ -176,6 +221,15 @@ __device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int
   }
   depth += __popc(push);
   return t;
+}
+
+template <bool VOTE, bool WRAP = false>
+__device__ __forceinline__ Tested front_step(Front &S, int &depth, int pop4, int lane,
+                                             const WalkSib *__restrict__ sib) {
+  return front_step<VOTE>(S, depth, pop4, lane, sib,
+                          [&](const float4 &a, float s2, uint32_t *m) {
+                            test64<WRAP>(S, a.x, a.y, a.z, s2, m);
+                          });
 }
 
 // Geometric centre and half a cell of the bottom node 64 p + q.

@@ -43,8 +43,8 @@
 // 32 with the vote, through the tree together, on its plain grid): quadrupole
 // theta 0.75 0.96 (1.85), monopole 0.5 1.92 (3.2) and 0.24 10.7 (15.5), vote
 // with quadrupole 0.8 0.91 (2.49); 16.3M-cell core, monopole 0.5 18.6 (27.4);
-// 32^3 cells 0.093 (0.45): there a warp has a scheduler to itself, and a step
-// tests 32 nodes per chain of dependent loads instead of one.
+// 32^3 cells 0.085 (0.45): there a step tests 32 nodes per chain of dependent
+// loads instead of one, and two warps share an octant (k_walk_shared).
 //
 // The opening test is evaluated in binary32 with the operation order stated
 // in the public header; the interaction uses the same d2 formed again.  (The
@@ -102,10 +102,14 @@ struct WalkMem {                     // of one warp
 };
 
 // Per-lane state of the evaluation: the lane's 8 targets as four x pairs, pair
-// 2 r + k: row r (y = 2 (sub-brick & 1) + r), x = 2 k, 2 k + 1.
-template <bool COUNTS>
+// 2 r + k: row r (y = 2 (sub-brick & 1) + r), x = 2 k, 2 k + 1.  A walk shared
+// by SPLIT warps leaves each its x pair k0 of both rows (SPLIT = 2: 4 targets)
+// or of row r0 (SPLIT = 4: 2 targets).
+constexpr int split_rows(int split) { return split == 4 ? 1 : 2; }
+constexpr int split_pairs(int split) { return split == 1 ? 2 : 1; }  // x pairs of a row
+template <bool COUNTS, int SPLIT>
 struct Lane {
-  u64 sum[4], comp[4];    // compensated pair sums
+  u64 sum[4 / SPLIT], comp[4 / SPLIT];    // compensated pair sums
   int na[COUNTS ? 8 : 1], nb[COUNTS ? 8 : 1];  // accepted nodes, opened bottom nodes
 };
 
@@ -154,24 +158,26 @@ __device__ __forceinline__ u64 sum_base(float mass) {
   return pk(b, b);
 }
 
+template <int NR, int NK>  // rows, x pairs of a row
 struct Targets {          // of one lane, read back before every evaluation
-  u64 tx[2];              // {x0, x1}, {x2, x3}
-  float ty[2], tz;
+  u64 tx[NK];             // {x0, x1}, {x2, x3}
+  float ty[NR], tz;
 };
 
 // A list entry as a lane evaluates it: the staged record (mass and x pairs
 // duplicated for the packed operations) and the parts shared by a row.
-template <bool QUAD>
+template <bool QUAD, int NK>
 struct Entry {
-  u64 dx[2], mm;       // {x0, x1} - px, {x2, x3} - px; {m, m}
+  u64 dx[NK], mm;      // {x0, x1} - px, {x2, x3} - px; {m, m}
   float py, dz;
   float4 q;            // Qxx/2, Qyy/2, Qzz/2, Qxy
   float2 q2;           // Qxz, Qyz
   uint32_t m8;         // bit 4 r + x: target x of row r takes part
   float h, qu, qc;     // of the current row
 
+  template <int NR>
   __device__ __forceinline__ void load(const WalkMem<QUAD> &S, uint32_t v, int zsh,
-                                       const Targets &T) {
+                                       const Targets<NR, NK> &T) {
     const char *at = reinterpret_cast<const char *>(S.node) + (v & 0xffffu);
     const float4 n = *reinterpret_cast<const float4 *>(at);
     if (QUAD) {
@@ -180,8 +186,8 @@ struct Entry {
     }
     m8 = v >> zsh;
     const u64 px = pk(n.x, n.x);
-    dx[0] = sub2(T.tx[0], px);
-    dx[1] = sub2(T.tx[1], px);
+#pragma unroll
+    for (int k = 0; k < NK; ++k) dx[k] = sub2(T.tx[k], px);
     mm = pk(n.w, n.w);
     py = n.y;
     dz = __fsub_rn(T.tz, n.z);
@@ -211,9 +217,11 @@ struct Entry {
 
 // 8 entries of every sub-brick's list from ring position `at` (a multiple of
 // 8): the lane takes entries par and par + 4.
-template <bool KAHAN, bool COUNTS, bool QUAD>
-__device__ __forceinline__ void eval_nodes(const WalkMem<QUAD> &S, int sb, unsigned at, int par,
-                                           int zsh, const Targets &T, Lane<COUNTS> &L) {
+template <bool KAHAN, bool COUNTS, bool QUAD, int SPLIT>
+__device__ __forceinline__ void eval_nodes(
+    const WalkMem<QUAD> &S, int sb, unsigned at, int par, int zsh,
+    const Targets<split_rows(SPLIT), split_pairs(SPLIT)> &T, Lane<COUNTS, SPLIT> &L) {
+  constexpr int NR = split_rows(SPLIT), NK = split_pairs(SPLIT);
   const uint32_t *list = &S.list[sb][(at & (kRing - 1)) + par];
   const uint32_t v0 = list[0], v1 = list[4];
   if (COUNTS) {
@@ -221,20 +229,20 @@ __device__ __forceinline__ void eval_nodes(const WalkMem<QUAD> &S, int sb, unsig
     for (int i = 0; i < 8; ++i) L.na[i] += ((v0 >> (zsh + i)) & 1u) + ((v1 >> (zsh + i)) & 1u);
     return;
   }
-  Entry<QUAD> a, b;
+  Entry<QUAD, NK> a, b;
   a.load(S, v0, zsh, T);
   b.load(S, v1, zsh, T);
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < NR; ++r) {
     a.row(T.ty[r]);
     b.row(T.ty[r]);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < NK; ++k) {
       u64 ra, ta, rb, tb;
       a.terms(r, k, ra, ta);
       b.terms(r, k, rb, tb);
-      accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], ra, ta);
-      accumulate_product2<KAHAN>(L.sum[2 * r + k], L.comp[2 * r + k], rb, tb);
+      accumulate_product2<KAHAN>(L.sum[NK * r + k], L.comp[NK * r + k], ra, ta);
+      accumulate_product2<KAHAN>(L.sum[NK * r + k], L.comp[NK * r + k], rb, tb);
     }
   }
 }
@@ -254,12 +262,14 @@ __device__ __forceinline__ u64 two_sum2(u64 a, u64 b, u64 &e) {
 // 16, 56 % of a row's 4 at theta 0.75), and one costs 8 interactions each.
 // Every cell but the target's own (d2 > 0); a node's four terms are added
 // plainly and join a compensated sum, which joins the lanes' totals at the end.
-template <bool KAHAN, bool COUNTS, bool QUAD>
+template <bool KAHAN, bool COUNTS, bool QUAD, int SPLIT>
 __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
                                            const float4 *__restrict__ cmass, int n, int lane,
-                                           u64 base, Lane<COUNTS> &L) {
-  constexpr int W = kBottoms / 32;
-  const int row = lane & 15, word = 1 + (row >> 3), sh = 4 * (row & 7), zhalf = lane >> 4;
+                                           int r0, int k0, u64 base, Lane<COUNTS, SPLIT> &L) {
+  constexpr int W = kBottoms / 32, NR = split_rows(SPLIT), NK = split_pairs(SPLIT);
+  constexpr unsigned row_bits = SPLIT == 1 ? 15u : 3u;
+  const bool serves = SPLIT != 4 || (lane & 1) == r0;  // (the row's y & 1)
+  const int row = lane & 15, word = 1 + (row >> 3), sh = 4 * (row & 7) + 2 * k0, zhalf = lane >> 4;
   uint32_t mine[W];  // bottom nodes some target of the row opened
 #pragma unroll
   for (int w = 0; w < W; ++w) {
@@ -268,17 +278,22 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
     mine[w] = 0u;
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
-      const unsigned b = __ballot_sync(kFull, (((r < 8 ? lo : hi) >> (4 * (r & 7))) & 15u) != 0u);
-      if (row == r) mine[w] = b;
+      const unsigned b = __ballot_sync(kFull, (((r < 8 ? lo : hi) >> (4 * (r & 7) + 2 * k0)) & row_bits) != 0u);
+      if (row == r) mine[w] = serves ? b : 0u;
     }
   }
   int left = 0;
 #pragma unroll
   for (int w = 0; w < W; ++w) left += __popc(mine[w]);
   const int steps = (int)__reduce_max_sync(kFull, (unsigned)left);
-  u64 sum[2] = {base, base}, comp[2] = {0ull, 0ull};
+  u64 sum[NK], comp[NK], tx[NK];
+#pragma unroll
+  for (int k = 0; k < NK; ++k) {
+    sum[k] = base;
+    comp[k] = 0ull;
+    tx[k] = pk(S.front.tx[k0 + k].x, S.front.tx[k0 + k].z);
+  }
   int nb[4] = {0, 0, 0, 0};
-  const u64 tx[2] = {pk(S.front.tx[0].x, S.front.tx[0].z), pk(S.front.tx[1].x, S.front.tx[1].z)};
   const float ty = S.front.coord(16 + 2 * ((row >> 2) & 1) + (row & 1));
   const float tz = S.front.coord(8 + 4 * (row >> 3) + (row & 2));
 #pragma unroll 2
@@ -302,15 +317,19 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
     // masses of the cells (x0, y0), (x1, y0), (x0, y1), (x1, y1) of the lane's z
     const float4 m = __ldg(cmass + 2 * (size_t)S.bottom[0][j] + zhalf);
     const float4 c = S.centre[j];
-    float least[4];  // a target takes part where d2 > least: 0, or never
+    float least[2 * NK];  // a target takes part where d2 > least: 0, or never
 #pragma unroll
-    for (int i = 0; i < 4; ++i) least[i] = (m4 & (1u << i)) ? 0.0f : __int_as_float(0x7f800000);
+    for (int i = 0; i < 2 * NK; ++i) least[i] = (m4 & (1u << i)) ? 0.0f : __int_as_float(0x7f800000);
     const float dz = __fsub_rn(tz, zhalf ? __fadd_rn(c.z, c.w) : __fsub_rn(c.z, c.w));
     const float dzz = __fmul_rn(dz, dz);
     const float xl = __fsub_rn(c.x, c.w), xh = __fadd_rn(c.x, c.w);
-    const u64 dx[2][2] = {{sub2(tx[0], pk(xl, xl)), sub2(tx[1], pk(xl, xl))},
-                          {sub2(tx[0], pk(xh, xh)), sub2(tx[1], pk(xh, xh))}};
-    u64 part[2] = {0ull, 0ull};
+    u64 dx[2][NK], part[NK];
+#pragma unroll
+    for (int k = 0; k < NK; ++k) {
+      dx[0][k] = sub2(tx[k], pk(xl, xl));
+      dx[1][k] = sub2(tx[k], pk(xh, xh));
+      part[k] = 0ull;
+    }
 #pragma unroll
     for (int y = 0; y < 2; ++y) {
       const float dy = __fsub_rn(ty, y ? __fadd_rn(c.y, c.w) : __fsub_rn(c.y, c.w));
@@ -319,7 +338,7 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
       for (int x = 0; x < 2; ++x) {
         const float mc = y ? (x ? m.w : m.z) : (x ? m.y : m.x);
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
+        for (int k = 0; k < NK; ++k) {
           float da, db;
           upk(fma2(dx[x][k], dx[x][k], pk(h, h)), da, db);
           part[k] = fma2(pk(mc, mc), pk(rsqrt_above(da, least[2 * k]), rsqrt_above(db, least[2 * k + 1])),
@@ -327,8 +346,8 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
         }
       }
     }
-    accumulate2<KAHAN>(sum[0], comp[0], part[0]);
-    accumulate2<KAHAN>(sum[1], comp[1], part[1]);
+#pragma unroll
+    for (int k = 0; k < NK; ++k) accumulate2<KAHAN>(sum[k], comp[k], part[k]);
   }
   // to the lanes that own the targets: rows 2 (lane >> 2) and the next; the
   // two z halves are added, one lane of the four that share the targets takes them
@@ -339,7 +358,7 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
     return;
   }
 #pragma unroll
-  for (int k = 0; k < 2; ++k) {
+  for (int k = 0; k < NK; ++k) {
     u64 e = 0ull;
     sum[k] = sub2(sum[k], base);
     const u64 o = __shfl_xor_sync(kFull, sum[k], 16);
@@ -350,15 +369,15 @@ __device__ __forceinline__ void eval_cells(const WalkMem<QUAD> &S,
       sum[k] = add2(sum[k], o);
     }
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const u64 v = __shfl_sync(kFull, sum[k], from + r);
-      const u64 c = KAHAN ? __shfl_sync(kFull, comp[k], from + r) : 0ull;
+    for (int r = 0; r < NR; ++r) {
+      const u64 v = __shfl_sync(kFull, sum[k], from + r0 + r);
+      const u64 c = KAHAN ? __shfl_sync(kFull, comp[k], from + r0 + r) : 0ull;
       if ((lane & 3) == 0) {
         if (KAHAN) {
-          L.sum[2 * r + k] = two_sum2(L.sum[2 * r + k], v, e);
-          L.comp[2 * r + k] = add2(add2(L.comp[2 * r + k], c), e);
+          L.sum[NK * r + k] = two_sum2(L.sum[NK * r + k], v, e);
+          L.comp[NK * r + k] = add2(add2(L.comp[NK * r + k], c), e);
         } else {
-          L.sum[2 * r + k] = add2(L.sum[2 * r + k], v);
+          L.sum[NK * r + k] = add2(L.sum[NK * r + k], v);
         }
       }
     }
@@ -395,10 +414,16 @@ struct WalkArgs {
   const int *flev;              // deepest block level per field
 };
 
-// Walk of octant u & 7 of sorted block u >> 3.
-template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
+// Walk of octant u & 7 of sorted block u >> 3; with SPLIT > 1 by the SPLIT warps
+// of the CTA, each for its part of the targets (r0, k0; else 0).  They test
+// their part alone and join the masks (`joint`: two buffers, of which a warp
+// overwrites one only after a barrier that follows the others' reads), so
+// that all take the same steps and make the same lists.
+template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE, int SPLIT = 1>
 __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> &S,
-                                            const WalkArgs &A) {
+                                            const WalkArgs &A, int r0 = 0, int k0 = 0,
+                                            uint2 (*joint)[SPLIT][32] = nullptr) {
+  constexpr int NR = split_rows(SPLIT), NK = split_pairs(SPLIT), NP = NR * NK;
   const unsigned p = u >> 3;
   const int o = (int)(u & 7);
   const int4 B = A.blk[p], F = A.fld[p];
@@ -406,15 +431,16 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
   const unsigned lower = (1u << lane) - 1u;
   front_start(S.front, octant_at(B, o), F, p, lane, A.rec, A.sib.tops);
   const u64 base = sum_base<KAHAN>(A.rec[F.x].m);
-  Lane<COUNTS> L;
+  Lane<COUNTS, SPLIT> L;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < NP; ++i) {
     L.sum[i] = base;
     L.comp[i] = 0ull;
   }
 #pragma unroll
   for (int i = 0; i < (COUNTS ? 8 : 1); ++i) L.na[i] = L.nb[i] = 0;
-  const int zsh = 16 + 8 * zl;
+  const int zsh = 16 + 8 * zl + 4 * r0 + 2 * k0;
+  unsigned turn = 0u;
 
   // warp-uniform: stack entries; staged nodes ever and the oldest still needed;
   // list positions (written ever per sub-brick, evaluated ever); opened bottom nodes
@@ -422,7 +448,23 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
   const int pop4 = stack_pop4(A.flev[F.w]);
   unsigned staged = 0u, oldest = 0u, head = 0u, tail[4] = {0u, 0u, 0u, 0u};
   while (depth > 0) {
-    const Tested t = front_step<VOTE>(S.front, depth, pop4, lane, A.sib.sib);
+    const Tested t = front_step<VOTE>(
+        S.front, depth, pop4, lane, A.sib.sib, [&](const float4 &a, float s2, uint32_t *m) {
+          if (SPLIT == 1) {
+            test64<false>(S.front, a.x, a.y, a.z, s2, m);
+            return;
+          }
+          test_part<SPLIT>(S.front, r0, k0, a.x, a.y, a.z, s2, m);
+          joint[turn][threadIdx.x >> 5][lane] = make_uint2(m[0], m[1]);
+          __syncthreads();
+#pragma unroll
+          for (int i = 0; i < SPLIT; ++i) {
+            const uint2 o = joint[turn][i][lane];
+            m[0] |= o.x;
+            m[1] |= o.y;
+          }
+          turn ^= 1u;
+        });
     const unsigned acc = __ballot_sync(kFull, (t.alo | t.ahi) != 0u);
     if (acc) {
       const unsigned slot = (staged + __popc(acc & lower)) & (kRing - 1);
@@ -465,16 +507,16 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
         copy_async_wait();
         __syncwarp();
       }
-      Targets T;
-      T.tx[0] = pk(S.front.tx[0].x, S.front.tx[0].z);
-      T.tx[1] = pk(S.front.tx[1].x, S.front.tx[1].z);
-      T.ty[0] = S.front.coord(16 + 2 * (sb & 1));
-      T.ty[1] = S.front.coord(17 + 2 * (sb & 1));
+      Targets<NR, NK> T;
+#pragma unroll
+      for (int k = 0; k < NK; ++k) T.tx[k] = pk(S.front.tx[k0 + k].x, S.front.tx[k0 + k].z);
+#pragma unroll
+      for (int r = 0; r < NR; ++r) T.ty[r] = S.front.coord(16 + 2 * (sb & 1) + r0 + r);
       T.tz = S.front.coord(8 + 4 * (sb >> 1) + 2 * zl);
       for (;;) {
         const unsigned full = (min(min(tail[0], tail[1]), min(tail[2], tail[3])) - head) / 8u;
         for (unsigned i = 0; i < full; ++i, head += 8u)
-          eval_nodes<KAHAN, COUNTS, QUAD>(S, sb, head, par, zsh, T, L);
+          eval_nodes<KAHAN, COUNTS, QUAD, SPLIT>(S, sb, head, par, zsh, T, L);
         const unsigned mine = sb < 2 ? (sb ? tail[1] : tail[0]) : (sb == 2 ? tail[2] : tail[3]);
         // the oldest staged node still listed
         unsigned age = staged - oldest;
@@ -494,15 +536,16 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
     if (nbot > kBottoms - 32 || (last && nbot)) {
       for (int j = lane; j < nbot; j += 32) S.centre[j] = bottom_centre(S.bottom[0][j], A.blk);
       __syncwarp();
-      eval_cells<KAHAN, COUNTS, QUAD>(S, reinterpret_cast<const float4 *>(A.sib.cmass), nbot, lane,
-                                      base, L);
+      eval_cells<KAHAN, COUNTS, QUAD, SPLIT>(S, reinterpret_cast<const float4 *>(A.sib.cmass), nbot,
+                                             lane, r0, k0, base, L);
       nbot = 0;
       __syncwarp();
     }
   }
   // each of the four lanes writes two of the shared 8 targets: row par >> 1,
-  // x = 2 (par & 1) and the next
-  const int r = par >> 1, k = par & 1;
+  // x = 2 (par & 1) and the next (of a shared walk two lanes or one)
+  const int r = SPLIT == 4 ? r0 : (SPLIT == 2 ? par & 1 : par >> 1);
+  const int k = SPLIT == 1 ? par & 1 : k0;
   const int64_t cell = (int64_t)A.orig[p] * kCellsPerBlock + (4 * (o >> 2) + 2 * (sb >> 1) + zl) * 64 +
                        (4 * ((o >> 1) & 1) + 2 * (sb & 1) + r) * 8 + 4 * (o & 1) + 2 * k;
   if (COUNTS) {
@@ -531,7 +574,7 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
     // -G/L times the field's binary32 mass unit 2^e (exact), rounded once
     const float scale = (float)(-A.G * A.invL[F.w] * pow2i(mass_exponent(A.mmax[F.w])));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < NP; ++i) {
       L.sum[i] = sub2(L.sum[i], base);
       merge_lanes<KAHAN>(L.sum[i], L.comp[i]);
       if (i == par) {
@@ -557,6 +600,31 @@ __global__ void __maxnreg__(walk_regs(QUAD))
   const unsigned u = order ? order[warp] : warp;
   for (int k = 0; k < np; ++k) walk_octant<KAHAN, COUNTS, QUAD, VOTE>(u * np + k, lane, S, A);
 }
+
+// The octants of a small mesh, one per CTA of SPLIT warps, each for its part of
+// the targets: every target's terms are added in the same order as by one
+// warp, so the bits are the same.  Where a warp has a scheduler to itself, the
+// chain of a step and of its entries is what takes the time, and most
+// schedulers are idle; a part's tests and evaluations take 1/SPLIT of it.
+template <bool QUAD, int SPLIT>
+struct SharedMem {
+  WalkMem<QUAD> warp[SPLIT];
+  uint2 joint[2][SPLIT][32];
+};
+template <bool KAHAN, bool QUAD, bool VOTE, int SPLIT>
+__global__ void __launch_bounds__(32 * SPLIT) k_walk_shared(const WalkArgs A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SharedMem<QUAD, SPLIT> &S = *reinterpret_cast<SharedMem<QUAD, SPLIT> *>(smem_raw);
+  const int w = threadIdx.x >> 5;
+  walk_octant<KAHAN, false, QUAD, VOTE, SPLIT>(blockIdx.x, threadIdx.x & 31, S.warp[w], A, w >> 1,
+                                               w & 1, S.joint);
+}
+// Octants up to which an octant is shared by 4 or 2 warps: 2 warps to each of
+// the 608 schedulers.  Above, the doubled traversal costs more than the idle
+// schedulers (us, walk alone; persistent grid, 2 warps, 4 warps): 8 octants 36,
+// 29, 27; 64: 67, 55, 50; 120: 80, 67, 60; 512: 93, 85, 83 (quadrupole, 568:
+// 54, 48, 51); 792: 167, 199, 258.
+constexpr unsigned kShare4 = 304, kShare2 = 608;
 
 // The same walk on a persistent grid: each warp takes `per_ticket`
 // consecutive units at a time from the work counter (one atomic add by lane
@@ -595,6 +663,16 @@ cudaError_t go_lists(cudaStream_t s, int nb, const WalkArgs &a, const WalkShape 
   const unsigned nunits = (unsigned)nb * (8u / (unsigned)np);
   const int w = shape.warps > 0 ? shape.warps : kDefaultWarps;
   const int smem = w * (int)sizeof(WalkMem<QUAD>);
+  const unsigned octants = 8u * (unsigned)nb;
+  // (whatever the shape: the bits are the same, and no counter is needed)
+  if (!COUNTS && !shape.cycles && octants <= kShare4) {
+    k_walk_shared<KAHAN, QUAD, VOTE, 4><<<octants, 128, (int)sizeof(SharedMem<QUAD, 4>), s>>>(a);
+    return cudaGetLastError();
+  }
+  if (!COUNTS && !shape.cycles && octants <= kShare2) {
+    k_walk_shared<KAHAN, QUAD, VOTE, 2><<<octants, 64, (int)sizeof(SharedMem<QUAD, 2>), s>>>(a);
+    return cudaGetLastError();
+  }
   if (shape.ticket > 0 && shape.counter) {  // persistent: the CTAs that fit at once
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -634,6 +712,10 @@ cudaError_t raise_smem() {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(k_walk_queue<KAHAN, COUNTS, QUAD, VOTE>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  if (e == cudaSuccess && !COUNTS)
+    e = cudaFuncSetAttribute(k_walk_shared<KAHAN, QUAD, VOTE, 4>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(SharedMem<QUAD, 4>));
   return e;
 }
 

@@ -85,3 +85,24 @@ def test_block_lists_around_the_small_geometry_limit(level, extra, shuffled):
     e = {k: v.cpu().numpy() for k, v in s.export_nodes().items()}
     assert np.array_equal(e["level"], t["level"]) and np.array_equal(e["M"], t["M"])
     assert np.array_equal(e["R"], t["R"])
+
+
+@pytest.mark.parametrize("kahan", [True, False])
+@pytest.mark.parametrize("quad,vote", [(False, False), (True, False), (True, True)])
+def test_octants_shared_by_warps_keep_their_bits(kahan, quad, vote):
+    """1, 15, 36 (4 warps to an octant), 64 and 71 blocks (2 warps) alone: the
+    bits that the fields have in a batch of 187 blocks, a warp to an octant."""
+    fs = [field(0, 0, 1), field(1, 1, 2), field(0, 5, 3), field(2, 0, 4), field(2, 1, 5)]
+    crit = B.BH_CRIT_WARP_VOTE if vote else B.BH_CRIT_PER_CELL
+    s = B.Solver(criterion=crit, quadrupole=quad, kahan=kahan)
+    s.build_batch([m.nblocks for m, _ in fs], np.concatenate([m.level for m, _ in fs]),
+                  np.concatenate([m.ijk for m, _ in fs]),
+                  torch.as_tensor(np.concatenate([r.reshape(-1) for _, r in fs])).cuda())
+    got = s.potential(0.5).cpu().numpy()
+    at = 0
+    for m, r in fs:
+        a = B.Solver(criterion=crit, quadrupole=quad, kahan=kahan)
+        a.build(m.level, m.ijk, torch.as_tensor(r.reshape(-1)).cuda())
+        want = a.potential(0.5).cpu().numpy()
+        assert np.array_equal(got[at:at + want.size], want)
+        at += want.size
