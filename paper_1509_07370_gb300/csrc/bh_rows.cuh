@@ -22,16 +22,17 @@ struct Row {
   }
 };
 
-// Which of n <= 64 entries with masks {lo, hi} have a target of the lane's
+// Which of n <= 64 N entries with masks {lo, hi} have a target of the lane's
 // row, found by ballots; steps: the most that any lane has.
+template <int N>
 struct RowList {
-  unsigned long long left;
+  unsigned long long left[N];
   int mine, steps;
   bool taken;
   __device__ __forceinline__ RowList(const uint32_t *lo, const uint32_t *hi, int n, int lane) {
-    uint32_t m[2];
+    uint32_t m[2 * N];
 #pragma unroll
-    for (int w = 0; w < 2; ++w) {
+    for (int w = 0; w < 2 * N; ++w) {
       const int j = 32 * w + lane;
       const uint32_t l = j < n ? lo[j] : 0u, h = j < n ? hi[j] : 0u;
       m[w] = 0u;
@@ -41,8 +42,12 @@ struct RowList {
         if ((lane & 15) == r) m[w] = b;
       }
     }
-    left = ((unsigned long long)m[1] << 32) | m[0];
-    mine = __popcll(left);
+    mine = 0;
+#pragma unroll
+    for (int w = 0; w < N; ++w) {
+      left[w] = ((unsigned long long)m[2 * w + 1] << 32) | m[2 * w];
+      mine += __popcll(left[w]);
+    }
     steps = (int)__reduce_max_sync(kFull, (unsigned)mine);
     taken = false;
   }
@@ -55,16 +60,32 @@ struct RowList {
   // The next entry (0 with taken = false when the lane has none left).
   __device__ __forceinline__ int from_bottom() {
     taken = mine > 0;
-    const int j = taken ? __ffsll((long long)left) - 1 : 0;
-    left &= left - 1ull;
     --mine;
+    int w = 0;  // the lowest word with an entry left
+#pragma unroll
+    for (int i = N - 1; i >= 0; --i) w = left[i] ? i : w;
+    int j = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (i == w) {
+        j = taken ? 64 * i + __ffsll((long long)left[i]) - 1 : 0;
+        left[i] &= left[i] - 1ull;
+      }
     return j;
   }
   __device__ __forceinline__ int from_top() {
     taken = mine > 0;
-    const int j = taken ? 63 - __clzll((long long)left) : 0;
-    left &= ~(1ull << j);
     --mine;
+    int w = 0;  // the highest
+#pragma unroll
+    for (int i = 0; i < N; ++i) w = left[i] ? i : w;
+    int j = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (i == w) {
+        j = taken ? 64 * i + 63 - __clzll((long long)left[i]) : 0;
+        left[i] &= ~(1ull << (j & 63));
+      }
     return j;
   }
 };

@@ -16,7 +16,7 @@
 //    operations instead of a square root and a division (some 9 each).  The
 //    approximation's 2^-20 leaves e^3 below 2^-60.
 // An interaction then takes 9 operations (7.9 with a cell) instead of 26.
-// Measured (32^3 cells, theta 0.5): 3.07 -> 1.59 ms; error against exact sums
+// Measured (32^3 cells, theta 0.5): 3.07 -> 1.43 ms; error against exact sums
 // 1.12e-15 -> 1.07e-15 of the potential.  That is 36 operations per step of a
 // lane's 4 targets against the FP64 rate's 1.04 ms (four octants on the
 // fullest SM): the rest is rows waiting for the longest list of their warp.
@@ -26,17 +26,24 @@ namespace bhg {
 namespace {
 
 constexpr int kF64Warps = 4;       // per CTA
-constexpr int kF64Stage = 64;      // staged nodes, evaluated once a further step's might not fit
-constexpr int kF64Bottoms = 64;    // opened bottom nodes, likewise
+// Staged nodes and opened bottom nodes, evaluated once a further step's might
+// not fit: rows wait less for the longest list of their warp in long lists.
+// 96 and 128 entries against 64 and 64: 1.59 -> 1.43 ms on 32^3 cells, 13.1 ->
+// 12.2 on a core at theta 0.7; with quadrupoles (more shared memory an entry)
+// 2 % slower.
+template <bool QUAD>
+constexpr int kF64Stage = QUAD ? 64 : 96;
+template <bool QUAD>
+constexpr int kF64Bottoms = QUAD ? 64 : 128;
 
 template <bool QUAD>
 struct F64Mem {                    // of one warp
   Front front;
-  double4_32a node[kF64Stage];     // centre of mass and mass
-  double quad[QUAD ? 6 * kF64Stage : 2];
-  uint32_t mask[2][kF64Stage];     // the accepting targets
-  float4 centre[kF64Bottoms];      // opened bottom nodes: geometric centre, half a cell,
-  uint32_t bottom[3][kF64Bottoms]; // index, O (two words)
+  double4_32a node[kF64Stage<QUAD>];     // centre of mass and mass
+  double quad[QUAD ? 6 * kF64Stage<QUAD> : 2];
+  uint32_t mask[2][kF64Stage<QUAD>];     // the accepting targets
+  float4 centre[kF64Bottoms<QUAD>];      // opened bottom nodes: geometric centre, half a cell,
+  uint32_t bottom[3][kF64Bottoms<QUAD>]; // index, O (two words)
 };
 
 // 1/sqrt(d) for normal d > 0.
@@ -100,11 +107,11 @@ __global__ void __launch_bounds__(32 * kF64Warps)
     nbot += __popc(bot);
     __syncwarp();
     const bool last = depth == 0;
-    if (staged > kF64Stage - 32 || (last && staged)) {
+    if (staged > kF64Stage<QUAD> - 32 || (last && staged)) {
       copy_async_wait();
       __syncwarp();
       double part[4] = {0.0, 0.0, 0.0, 0.0};  // (short sums of their own: less rounding)
-      RowList list(S.mask[0], S.mask[1], staged, lane);
+      RowList<(kF64Stage<QUAD> + 63) / 64> list(S.mask[0], S.mask[1], staged, lane);
       list.halve(R.half);
       for (int it = 0; it < list.steps; ++it) {
         const int j = R.half ? list.from_top() : list.from_bottom();
@@ -136,11 +143,11 @@ __global__ void __launch_bounds__(32 * kF64Warps)
       staged = 0;
       __syncwarp();
     }
-    if (nbot > kF64Bottoms - 32 || (last && nbot)) {
+    if (nbot > kF64Bottoms<QUAD> - 32 || (last && nbot)) {
       for (int j = lane; j < nbot; j += 32) S.centre[j] = bottom_centre(S.bottom[0][j], blk);
       __syncwarp();
       double part[4] = {0.0, 0.0, 0.0, 0.0};
-      RowList list(S.bottom[1], S.bottom[2], nbot, lane);
+      RowList<(kF64Bottoms<QUAD> + 63) / 64> list(S.bottom[1], S.bottom[2], nbot, lane);
       for (int it = 0; it < list.steps; ++it) {  // the lane's half: the four cells of one z
         const int j = list.from_bottom();
         const uint32_t m4 = list.taken ? S.bottom[1 + R.word][j] >> R.shift : 0u;

@@ -143,7 +143,7 @@ __device__ __forceinline__ void walk_octant_periodic(
     __syncwarp();
     const bool last = depth == 0;
     if (staged > kPStage - 32 || (last && staged)) {
-      RowList list(S.mask[0], S.mask[1], staged, lane);
+      RowList<1> list(S.mask[0], S.mask[1], staged, lane);
       list.halve(R.half);
       for (int it = 0; it < list.steps; ++it) {
         const int j = R.half ? list.from_top() : list.from_bottom();
@@ -162,7 +162,7 @@ __device__ __forceinline__ void walk_octant_periodic(
     if (nbot > kPBottoms - 32 || (last && nbot)) {
       for (int j = lane; j < nbot; j += 32) S.centre[j] = bottom_centre(S.bottom[0][j], blk);
       __syncwarp();
-      RowList list(S.bottom[1], S.bottom[2], nbot, lane);
+      RowList<1> list(S.bottom[1], S.bottom[2], nbot, lane);
       for (int it = 0; it < list.steps; ++it) {  // the lane's half: the four cells of one z
         const int j = list.from_bottom();
         const uint32_t m4 = list.taken ? S.bottom[1 + R.word][j] >> R.shift : 0u;
