@@ -183,10 +183,10 @@ bh_status bh_sync_status(bh_ctx *ctx);
  * every launch shape it offers -- CTAs of 2, 4, 8 and 16 warps; warps that
  * walk for 64 targets (a 4x4x4 octant of a block; "one pair per lane") or 128
  * targets (two x-neighbouring octants, one after the other; "two pairs");
- * either a
- * plain grid of one warp per group or a persistent grid (as many CTAs as the
- * GPU holds at once) whose warps take 1, 2 or 4 groups at a time from a work
- * counter; and the groups in their own (Morton) order or longest walk first
+ * either a plain grid of one warp per group or a persistent grid (as many CTAs
+ * as the GPU holds at once; the default, one group at a time, in CTAs of 4
+ * warps) whose warps take 1, 2 or 4 groups at a time from a work counter; and
+ * the groups in their own (Morton) order or longest walk first
  * (the periodic walk: CTA width and order, one octant, plain grid) --
  * each twice, then the four fastest five times more -- and keeps the fastest
  * for later walks.  For the longest-first order it first walks the tree once
@@ -194,8 +194,9 @@ bh_status bh_sync_status(bh_ctx *ctx);
  * recording the SM clock cycles of every group's walk, and
  * sorts the groups by them (on the host); that order is kept with the
  * context, like the shape, and used while the tree has the same number of
- * groups (a permutation of the groups: it can only change the speed).  All shapes
- * give bit-identical potentials.  shape (may be NULL) receives four ints:
+ * groups (a permutation of the groups: it can only change the speed).  Trees
+ * of up to 76 blocks are walked by several warps per octant whatever the
+ * shape.  All shapes give bit-identical potentials.  shape (may be NULL) receives four ints:
  * {warps per CTA, target pairs per lane, groups per take (0 = plain grid),
  * longest first (0/1)}; all 0 for walk modes with a fixed launch shape.
  * Allocates a scratch output once and the order (4 bytes per group). */
@@ -204,8 +205,8 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape);
 /* Sets the launch shape of the binary32 per-cell walk (the four values
  * bh_autotune chooses among), e.g. one found by an earlier bh_autotune on
  * the same kind of mesh: warps per CTA (1..16), octants per group (1 or 2,
- * named target pairs per lane), groups per take of the persistent grid (0 = plain grid, 1..64) and
- * longest_first (1: the walk order made by the last bh_autotune, 0: the
+ * named target pairs per lane), groups per take of the persistent grid (0 =
+ * plain grid, 1..64) and longest_first (1: the walk order made by the last bh_autotune, 0: the
  * groups' own order); 0 for the first two means the default.  Potentials do
  * not depend on the shape (bit for bit).  Drops a captured bh_solve_graph
  * graph.  BH_ERR_ARG for values out of range (the periodic walk: one pair,

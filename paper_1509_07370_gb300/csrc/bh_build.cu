@@ -10,7 +10,8 @@
 //   1. each block gets the Morton key of its lower corner on the level-21
 //      lattice (k_keys_mass, which also finds each field's largest cell
 //      mass, the binary32 mass unit) and blocks are put in key order
-//      (k_sort_blocks, only if the caller's order is not already sorted);
+//      (k_rank_blocks or k_sort_blocks, only if the caller's order is not
+//      already sorted);
 //   2. consecutive keys must abut exactly (k_tile_and_count): this checks that
 //      the blocks tile the box, and the trailing zero bits of a block's key
 //      tell how many internal "top" nodes (cubes above the blocks) start at it

@@ -1,4 +1,5 @@
-// The learned walk: the per-cell binary32 monopole walk of k_walk_pair with
+// The learned walk: the per-cell binary32 monopole walk, the warp's 64 targets
+// stepping through the tree together (skip pointers in pre-order), with
 // the learned residual correction added for every accepted internal node
 // (features and network in bhgrav.h; the correction is not in the paper).
 //
