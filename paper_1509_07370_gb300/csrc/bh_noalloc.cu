@@ -48,8 +48,7 @@ constexpr size_t kOffPrestart = up256(kOffCount + sizeof(int) * kNoAllocMaxBlock
 constexpr size_t kOffBlk = up256(kOffPrestart + sizeof(int) * kNoAllocMaxBlocks);
 constexpr size_t kOffOrig = up256(kOffBlk + sizeof(int4) * kNoAllocMaxBlocks);
 constexpr size_t kOffFlags = up256(kOffOrig + sizeof(int) * kNoAllocMaxBlocks);
-constexpr size_t kOffFstart = up256(kOffFlags + 5 * sizeof(unsigned));   // one field
-// (flags[4]: the work counter of the persistent walk)
+constexpr size_t kOffFstart = up256(kOffFlags + 4 * sizeof(unsigned));   // one field
 constexpr size_t kOffFid = up256(kOffFstart + 3 * sizeof(int));  // fstart, then flev
 constexpr size_t kOffFld = up256(kOffFid + sizeof(int) * kNoAllocMaxBlocks);
 constexpr size_t kOffBox = up256(kOffFld + sizeof(int4) * kNoAllocMaxBlocks);  // L, 1/L
@@ -206,10 +205,7 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
   if (h_flags[0] & kErrDensity) return BH_ERR_ARG;
   bh_options opt;
   bh_default_options(&opt);
-  WalkShape shape;
-  shape.ticket = 1;
-  shape.counter = d_flags + 4;
-  NA_CUDA(launch_walk(s, opt, nb, d_rec, sib, d_blk, d_orig, fa, G, out, nullptr, nullptr, nullptr,
-                      shape));
+  // (up to 64 blocks: several warps share an octant, no work counter)
+  NA_CUDA(launch_walk(s, opt, nb, d_rec, sib, d_blk, d_orig, fa, G, out, nullptr, nullptr));
   return BH_OK;
 }
