@@ -67,22 +67,41 @@ def test_shuffled_fields_of_a_batch_are_sorted_by_themselves():
     assert at == e["M"].size
 
 
+def split_first(level, split):
+    """All cubes of `level` with the first `split` of them refined once, in
+    Morton order."""
+    n = 1 << level
+    ijk = np.stack(np.meshgrid(*[np.arange(n)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    fine = (2 * ijk[:split, None, :] + np.indices((2, 2, 2)).reshape(3, 8).T).reshape(-1, 3)
+    lev = np.r_[np.full(len(ijk) - split, level), np.full(len(fine), level + 1)].astype(np.int32)
+    ijk = np.concatenate([ijk[split:], fine]).astype(np.int32)
+    key = np.zeros(len(lev), np.int64)  # Morton key of the lower corner at the finer level
+    c = ijk.astype(np.int64) << (level + 1 - lev)[:, None]
+    for b in range(level + 1):
+        for d in range(3):
+            key |= ((c[:, d] >> b) & 1) << (3 * b + d)
+    order = np.argsort(key)
+    return lev[order], ijk[order]
+
+
+@pytest.mark.parametrize("split", [585, 586])
+def test_trees_around_one_tile_of_the_scan(split):
+    """8,191 and 8,198 blocks: the scan's tile holds 8,192."""
+    lev, ijk = split_first(4, split)
+    rho = np.random.default_rng(3).random((len(lev), 512), dtype=np.float32)
+    t = O.Tree(lev, ijk, rho.reshape(-1, 8, 8, 8).astype(np.float64)).export()
+    s = B.Solver()
+    s.build(lev, ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+    e = {k: v.cpu().numpy() for k, v in s.export_nodes().items()}
+    assert np.array_equal(e["level"], t["level"]) and np.array_equal(e["M"], t["M"])
+
+
 @pytest.mark.parametrize("split", [4681, 4682])
 def test_both_sorts_restore_the_morton_order(split):
     """65,535 blocks (sorted by counting) and 65,542 (by radix), listed in
     random order: the tree of the list in Morton order, whose potentials and
     masses the other tests compare with the oracle."""
-    ijk = np.stack(np.meshgrid(*[np.arange(32)] * 3, indexing="ij"), -1).reshape(-1, 3)
-    fine = (2 * ijk[:split, None, :] + np.indices((2, 2, 2)).reshape(3, 8).T).reshape(-1, 3)
-    lev = np.r_[np.full(len(ijk) - split, 5), np.full(len(fine), 6)].astype(np.int32)
-    ijk = np.concatenate([ijk[split:], fine]).astype(np.int32)
-    corner_key = np.zeros(len(lev), np.int64)  # Morton key of the lower corner at level 6
-    c = ijk.astype(np.int64) << (6 - lev)[:, None]
-    for b in range(6):
-        for d in range(3):
-            corner_key |= ((c[:, d] >> b) & 1) << (3 * b + d)
-    order = np.argsort(corner_key)
-    lev, ijk = lev[order], ijk[order]
+    lev, ijk = split_first(5, split)
     rho = torch.rand((len(lev), 512), generator=torch.Generator().manual_seed(1))
     trees = []
     for p in (np.arange(len(lev)), np.random.default_rng(2).permutation(len(lev))):
