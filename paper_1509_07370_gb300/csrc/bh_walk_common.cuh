@@ -1,4 +1,4 @@
-// Helpers shared by the walk kernels (bh_walk.cu, bh_walk_learned.cu):
+// Helpers shared by the walk kernels (the list walks, bh_walk_learned.cu):
 // packed binary32 pair arithmetic and raw record loads in inline PTX, the
 // Kahan pair accumulator and the opening-test distance.
 #pragma once
@@ -62,20 +62,6 @@ __device__ __forceinline__ void load_rec(const WalkRec *p, u64 &q0, u64 &q1, u64
   q1 = pk(py, pz);
   q2 = pk(m, m);
   q3 = pk(s2, skf);
-}
-
-// The six fields of a quadrupole record (24 bytes) as w0 = {Qxx/2, Qxx/2},
-// w1 = {Qyy/2, Qzz/2}, w2 = {Qxy, Qxz}, w3 = {Qyz, 0}.
-__device__ __forceinline__ void load_quad(const WalkQuad *p, u64 &w0, u64 &w1, u64 &w2, u64 &w3) {
-  float hxx, hyy, hzz, qxy, qxz, qyz;
-  asm("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
-      : "=f"(hxx), "=f"(hyy), "=f"(hzz), "=f"(qxy)
-      : "l"(p));
-  asm("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(qxz), "=f"(qyz) : "l"(&p->qxz));
-  w0 = pk(hxx, hxx);
-  w1 = pk(hyy, hzz);
-  w2 = pk(qxy, qxz);
-  w3 = pk(qyz, 0.0f);
 }
 
 // Asynchronous copies from global to shared memory (visible to the copying
