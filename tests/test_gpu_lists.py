@@ -111,7 +111,7 @@ def test_octants_shared_by_warps_keep_their_bits(kahan, quad, vote):
 @pytest.mark.parametrize("level,extra", [(1, 0), (2, 0), (2, 3)])
 @pytest.mark.parametrize("quad", [False, True])
 def test_sums_of_a_cell_that_holds_the_mass_stay_compensated(level, extra, quad):
-    """8, 64 and 85 blocks (4, 2 and 1 warps to an octant).  A cell is no term
+    """8, 64 and 239 blocks (4, 2 and 1 warps to an octant).  A cell is no term
     of its own sum and of no node that it accepts, so its potential is the same
     sum of the same terms whether it is empty or holds 10^7 times the mass of
     the others (the mass unit is a power of two).  Compensated sums of some
