@@ -195,8 +195,9 @@ bh_status bh_sync_status(bh_ctx *ctx);
  * sorts the groups by them (on the host); that order is kept with the
  * context, like the shape, and used while the tree has the same number of
  * groups (a permutation of the groups: it can only change the speed).  Trees
- * of up to 76 blocks are walked by several warps per octant whatever the
- * shape.  All shapes give bit-identical potentials.  shape (may be NULL) receives four ints:
+ * of up to 76 blocks (isolated boundaries) are walked by several warps per
+ * octant whatever the shape: there only the order is made, and the shape stays
+ * as it was.  All shapes give bit-identical potentials.  shape (may be NULL) receives four ints:
  * {warps per CTA, target pairs per lane, groups per take (0 = plain grid),
  * longest first (0/1)}; all 0 for walk modes with a fixed launch shape.
  * Allocates a scratch output once and the order (4 bytes per group). */
@@ -216,7 +217,8 @@ bh_status bh_set_walk_shape(bh_ctx *ctx, int warps_per_cta, int pairs_per_lane,
 
 /* bh_update_density + bh_potential as ONE CUDA graph launch: the first call
  * (or a call with a different density/out pointer, density type, theta or G)
- * tunes the walk if it was not tuned yet, captures the sequence on the
+ * tunes the walk if it was not tuned yet and the tree's walk has a shape
+ * (bh_autotune), captures the sequence on the
  * context's stream and instantiates it; later calls replay it.  The context
  * must run on a created (non-default) stream.  Nothing is synchronised:
  * out is ready when the stream reaches the end of the graph; density errors

@@ -910,6 +910,13 @@ static bh_status make_walk_order(bh_ctx *ctx, int npairs) {
   return BH_OK;
 }
 
+// Whether the launch shape has a part in the walks of this tree: not where
+// several warps share an octant (then all shapes are one launch, and the
+// fastest of them chance).
+static bool shape_used(const bh_ctx *ctx) {
+  return ctx->opt.periodic || bhg::walk_split(ctx->tree.nb) == 1;
+}
+
 bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape) {
   const Range range_("bh_autotune");
   if (!ctx) return BH_ERR_ARG;
@@ -930,7 +937,10 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape) {
       BH_CUDA(bhg::dev_malloc(&t.d_stage_out, out_bytes));
       t.stage_out_bytes = out_bytes;
     }
+    drop_graph(t);  // a captured walk holds the old order and shape
     if ((st = make_walk_order(ctx, npairs)) != BH_OK) return st;
+  }
+  if (tunable && shape_used(ctx)) {
     struct Events {  // released on every return
       cudaEvent_t e[2] = {nullptr, nullptr};
       ~Events() {
@@ -983,11 +993,10 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape) {
       if (tmin[rank[i]] < tmin[pick]) pick = rank[i];
     const bhg::WalkShape best_s = shapes[pick];
     t.shape = best_s;
-    drop_graph(t);
   }
   if (shape) {
-    shape[0] = tunable ? t.shape.warps : 0;
-    shape[1] = tunable ? t.shape.pairs : 0;
+    shape[0] = !tunable ? 0 : t.shape.warps > 0 ? t.shape.warps : bhg::kDefaultWalkWarps;
+    shape[1] = !tunable ? 0 : t.shape.pairs > 0 ? t.shape.pairs : 1;
     shape[2] = tunable ? t.shape.ticket : 0;
     shape[3] = tunable ? t.shape.longest : 0;
   }
@@ -1038,7 +1047,9 @@ bh_status bh_solve_graph(bh_ctx *ctx, const void *density, int density_is_fp64, 
                     t.graph_fp64 == density_is_fp64 && t.graph_theta == theta && t.graph_G == G;
   if (!same) {
     drop_graph(t);
-    if (t.shape.warps == 0 && (st = bh_autotune(ctx, theta, nullptr)) != BH_OK) return st;
+    if (t.shape.warps == 0 && shape_used(ctx) &&
+        (st = bh_autotune(ctx, theta, nullptr)) != BH_OK)
+      return st;
     cudaStream_t s = ctx->stream;
     BH_CUDA(cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal));
     bh_status cap = BH_OK;

@@ -354,6 +354,11 @@ cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const Wal
 cudaError_t launch_walk_f64(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
                             const SibArgs &sib, const int4 *blk, const int *orig,
                             const FieldArgs &fa, double G, void *out);
+// Warps by which the binary32 walk shares an octant of a tree of nb blocks on
+// the current device; above 1 the launch shape is not used (the counting walk
+// and the one that records cycles never share).
+int walk_split(int nb);
+constexpr int kDefaultWalkWarps = 4;  // per CTA (shape.warps = 0)
 // Raises the dynamic shared-memory limit of the walk kernels on the current
 // device; called once per context, outside any graph capture.
 cudaError_t prepare_walk_kernels();

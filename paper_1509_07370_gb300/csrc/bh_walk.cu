@@ -59,7 +59,6 @@ constexpr int kMaxWalkThreads = 512;  // largest tunable CTA
 // slower; 72 spills: 2-5 % slower).  Quadrupole: shared memory allows 16 warps
 // whatever the registers, so 112 (80: 3.6 % slower; 128: 1 %).
 constexpr int walk_regs(bool quad) { return quad ? 112 : 80; }
-constexpr int kDefaultWarps = 4;
 
 __global__ void k_prepare_sib_s2(int64_t n, WalkSib *__restrict__ sib, float inv_theta) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -626,13 +625,6 @@ __global__ void __launch_bounds__(32 * SPLIT) k_walk_shared(const WalkArgs A) {
   walk_octant<KAHAN, false, QUAD, VOTE, SPLIT>(blockIdx.x, threadIdx.x & 31, S.warp[w], A, w >> 1,
                                                w & 1, S.joint);
 }
-// Octants up to which an octant is shared by 4 or 2 warps: 2 warps to each of
-// the 608 schedulers.  Above, the doubled traversal costs more than the idle
-// schedulers (us, walk alone; persistent grid, 2 warps, 4 warps): 8 octants 36,
-// 29, 27; 64: 67, 55, 50; 120: 80, 67, 60; 512: 93, 85, 83 (quadrupole, 568:
-// 54, 48, 51); 792: 167, 199, 258.
-constexpr unsigned kShare4 = 304, kShare2 = 608;
-
 // The same walk on a persistent grid: each warp takes `per_ticket`
 // consecutive units at a time from the work counter (one atomic add by lane
 // 0; no waiting on other warps) until every unit is taken.  In the units'
@@ -668,16 +660,16 @@ template <bool KAHAN, bool COUNTS, bool QUAD, bool VOTE>
 cudaError_t go_lists(cudaStream_t s, int nb, const WalkArgs &a, const WalkShape &shape) {
   const int np = shape.pairs > 0 ? shape.pairs : 1;
   const unsigned nunits = (unsigned)nb * (8u / (unsigned)np);
-  const int w = shape.warps > 0 ? shape.warps : kDefaultWarps;
+  const int w = shape.warps > 0 ? shape.warps : kDefaultWalkWarps;
   const int smem = w * (int)sizeof(WalkMem<QUAD>);
-  const unsigned octants = 8u * (unsigned)nb;
   // (whatever the shape: the bits are the same, and no counter is needed)
-  if (!COUNTS && !shape.cycles && octants <= kShare4) {
-    k_walk_shared<KAHAN, QUAD, VOTE, 4><<<octants, 128, (int)sizeof(SharedMem<QUAD, 4>), s>>>(a);
+  const int split = COUNTS || shape.cycles ? 1 : walk_split(nb);
+  if (split == 4) {
+    k_walk_shared<KAHAN, QUAD, VOTE, 4><<<8 * nb, 128, (int)sizeof(SharedMem<QUAD, 4>), s>>>(a);
     return cudaGetLastError();
   }
-  if (!COUNTS && !shape.cycles && octants <= kShare2) {
-    k_walk_shared<KAHAN, QUAD, VOTE, 2><<<octants, 64, (int)sizeof(SharedMem<QUAD, 2>), s>>>(a);
+  if (split == 2) {
+    k_walk_shared<KAHAN, QUAD, VOTE, 2><<<8 * nb, 64, (int)sizeof(SharedMem<QUAD, 2>), s>>>(a);
     return cudaGetLastError();
   }
   if (shape.ticket > 0 && shape.counter) {  // persistent: the CTAs that fit at once
@@ -727,6 +719,24 @@ cudaError_t raise_smem() {
 }
 
 }  // namespace
+
+// Up to two warps to each scheduler an octant is shared by 4 or 2 warps (152
+// SMs: 38 and 76 blocks).  Above, the doubled traversal costs more than the idle
+// schedulers (us, walk alone; persistent grid, 2 warps, 4 warps): 8 octants 36,
+// 29, 27; 64: 67, 55, 50; 120: 80, 67, 60; 512: 93, 85, 83 (quadrupole, 568:
+// 54, 48, 51); 792: 167, 199, 258.
+int walk_split(int nb) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 1;
+  }
+  const int64_t warps = 4 * 2 * (int64_t)sms;
+  for (int split = 4; split > 1; split /= 2)
+    if (8 * (int64_t)nb * split <= warps) return split;
+  return 1;
+}
 
 cudaError_t prepare_walk_kernels() {
   cudaError_t e = raise_smem<true, false, false, false>();
