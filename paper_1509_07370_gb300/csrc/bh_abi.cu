@@ -477,7 +477,7 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   for (int a = 0; a < 3; ++a) t.lo[a] = box_lo[a];
   t.L = box_len[0];
   // the moment kernels prepared s2 for the last walk's theta, if any
-  t.s2_inv_theta = fa.inv_theta > 0.0f ? fa.inv_theta : -1.0f;
+  t.sib_inv_theta = t.rec_inv_theta = fa.inv_theta > 0.0f ? fa.inv_theta : -1.0f;
   t.built = true;
   return BH_OK;
 }
@@ -655,7 +655,7 @@ bh_status bh_update_density(bh_ctx *ctx, const void *density, int density_is_fp6
   // the records are rewritten (s2 included, and delta changes with the
   // density), with s2 for the last walk's theta if there was one
   const float inv_theta = ctx->tree.last_inv_theta;
-  ctx->tree.s2_inv_theta = inv_theta > 0.0f ? inv_theta : -1.0f;
+  ctx->tree.sib_inv_theta = ctx->tree.rec_inv_theta = inv_theta > 0.0f ? inv_theta : -1.0f;
   st = enqueue_moments(ctx, density, density_is_fp64);
   ctx->build_timed = st == BH_OK && timed && timing_mark(ctx, 1);
   return st;
@@ -679,7 +679,7 @@ bh_status bh_sync_status(bh_ctx *ctx) {
   return BH_OK;
 }
 
-static bh_status prepare(bh_ctx *ctx, double theta);
+static bh_status prepare(bh_ctx *ctx, double theta, bool pre_order);
 
 }  // extern "C"
 
@@ -693,20 +693,16 @@ bh_status ctx_fail(bh_ctx *c, bh_status st, const char *fmt, ...) {
   }
   return st;
 }
-bh_status ctx_prepare(bh_ctx *ctx, double theta) { return prepare(ctx, theta); }
+bh_status ctx_prepare(bh_ctx *ctx, double theta) { return prepare(ctx, theta, true); }
 }  // namespace bhg
 
 extern "C" {
 
-// The squared opening radii for 1/theta on the context's stream.
-static cudaError_t enqueue_s2(bh_ctx *ctx, float inv_theta) {
-  bhg::Tree &t = ctx->tree;
-  const int64_t tops = t.n_nodes - (int64_t)bhg::kNodesPerBlock * t.nb;
-  return bhg::launch_prepare_s2(ctx->stream, t.n_nodes, t.d_aux, t.d_rec,
-                                (int64_t)bhg::kSibsPerBlock * t.nb + 8 * tops, t.d_sib, inv_theta);
-}
-
-static bh_status prepare(bh_ctx *ctx, double theta) {
+// Checks theta and makes the squared opening radii for it, unless they are the
+// present ones: those of the records in sibling order, which the list walks
+// test, or (pre_order) of those in pre-order, for the learned walks and the
+// pair listing.  The other records' stay as they are.
+static bh_status prepare(bh_ctx *ctx, double theta, bool pre_order) {
   bhg::Tree &t = ctx->tree;
   if (!t.built) return fail(ctx, BH_ERR_STATE, "no tree: call bh_build first");
   if (!(theta > 0.0) || !(theta <= 1.0))
@@ -715,9 +711,15 @@ static bh_status prepare(bh_ctx *ctx, double theta) {
   if (st != BH_OK) return st;
   const float inv_theta = (float)(1.0 / theta);
   t.last_inv_theta = inv_theta;
-  if (inv_theta != t.s2_inv_theta) {
-    BH_CUDA(enqueue_s2(ctx, inv_theta));
-    t.s2_inv_theta = inv_theta;
+  float &now = pre_order ? t.rec_inv_theta : t.sib_inv_theta;
+  if (inv_theta != now) {
+    const int64_t tops = t.n_nodes - (int64_t)bhg::kNodesPerBlock * t.nb;
+    if (pre_order)
+      BH_CUDA(bhg::launch_prepare_s2(ctx->stream, t.n_nodes, t.d_aux, t.d_rec, inv_theta));
+    else
+      BH_CUDA(bhg::launch_prepare_sib_s2(ctx->stream, (int64_t)bhg::kSibsPerBlock * t.nb + 8 * tops,
+                                         t.d_sib, inv_theta));
+    now = inv_theta;
   }
   return BH_OK;
 }
@@ -735,7 +737,7 @@ bh_status bh_potential(bh_ctx *ctx, double theta, double G, void *out) {
   bh_status st = use_device(ctx);
   if (st != BH_OK) return st;
   const bool timed = timing_mark(ctx, 2);
-  if ((st = prepare(ctx, theta)) != BH_OK) return st;
+  if ((st = prepare(ctx, theta, ctx->opt.learned != 0)) != BH_OK) return st;
   BH_CUDA(enqueue_walk(ctx, ctx->stream, G, out, nullptr, nullptr, nullptr, ctx->tree.shape));
   ctx->potential_timed = timed && timing_mark(ctx, 3);
   ctx->last_theta = theta;
@@ -749,7 +751,7 @@ bh_status bh_walk_counts(bh_ctx *ctx, double theta, int32_t *n_int, int32_t *n_t
   ctx->err[0] = 0;
   if (!ctx->tree.built) return fail(ctx, BH_ERR_STATE, "no tree: call bh_build first");
   if (!n_int || !n_test) return fail(ctx, BH_ERR_ARG, "bh_walk_counts: null output");
-  bh_status st = prepare(ctx, theta);
+  bh_status st = prepare(ctx, theta, false);
   if (st != BH_OK) return st;
   bhg::Tree &t = ctx->tree;
   BH_CUDA(enqueue_walk(ctx, ctx->stream, 0.0, nullptr, n_int, n_test, n_cell, t.shape));
@@ -921,7 +923,7 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape) {
   const Range range_("bh_autotune");
   if (!ctx) return BH_ERR_ARG;
   ctx->err[0] = 0;
-  bh_status st = prepare(ctx, theta);
+  bh_status st = prepare(ctx, theta, ctx->opt.learned != 0);
   if (st != BH_OK) return st;
   bhg::Tree &t = ctx->tree;
   const bool tunable = ctx->opt.precision == BH_PREC_F32 &&
@@ -1055,9 +1057,8 @@ bh_status bh_solve_graph(bh_ctx *ctx, const void *density, int density_is_fp64, 
     bh_status cap = BH_OK;
     cudaError_t e = cudaMemsetAsync(t.d_flags, 0, sizeof(unsigned), s);
     if (e == cudaSuccess) {
+      t.last_inv_theta = (float)(1.0 / theta);  // the moments come with their opening radii
       cap = enqueue_moments(ctx, density, density_is_fp64);
-      if (cap == BH_OK)
-        e = enqueue_s2(ctx, (float)(1.0 / theta));
       if (cap == BH_OK && e == cudaSuccess && ctx->opt.learned && !ctx->d_mlp)
         cap = fail(ctx, BH_ERR_STATE, "learned walk: call bh_set_mlp first");
       if (cap == BH_OK && e == cudaSuccess)
@@ -1081,7 +1082,7 @@ bh_status bh_solve_graph(bh_ctx *ctx, const void *density, int density_is_fp64, 
     t.graph_G = G;
   }
   BH_CUDA(cudaGraphLaunch(t.graph_exec, ctx->stream));
-  t.s2_inv_theta = t.last_inv_theta = (float)(1.0 / theta);
+  t.sib_inv_theta = t.rec_inv_theta = t.last_inv_theta = (float)(1.0 / theta);
   return BH_OK;
 }
 

@@ -246,7 +246,8 @@ struct Tree {
   double lo[3] = {0, 0, 0};
   double L = 1.0;
   bool built = false;
-  float s2_inv_theta = -1.0f;  // inverse theta the s2 field was prepared for
+  // inverse theta that the s2 of d_sib and of d_rec were made for (-1: none)
+  float sib_inv_theta = -1.0f, rec_inv_theta = -1.0f;
   float last_inv_theta = 0.0f; // of the last walk: builds prepare s2 for it
 };
 
@@ -339,9 +340,10 @@ cudaError_t launch_moments(cudaStream_t s, int nb, const int4 *blk, const int *o
 cudaError_t prepare_learned_kernels();
 
 // ---- walk kernels (bh_walk.cu) ---------------------------------------------
-// s2 of every node of rec and of every entry of sib (entries in all).
+// s2 of every node of rec; of every entry of sib.
 cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux, WalkRec *rec,
-                              int64_t entries, WalkSib *sib, float inv_theta);
+                              float inv_theta);
+cudaError_t launch_prepare_sib_s2(cudaStream_t s, int64_t entries, WalkSib *sib, float inv_theta);
 // out: float* (F32) or double* (F64); counts: optional per-cell n_int/n_test.
 // Potential scale of field f: -G * invL[f] (times the field's mass unit for
 // the binary32 walk).  shape = the launch shape of the per-cell binary32

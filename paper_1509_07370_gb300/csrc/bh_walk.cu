@@ -753,10 +753,15 @@ cudaError_t prepare_walk_kernels() {
 }
 
 cudaError_t launch_prepare_s2(cudaStream_t s, int64_t n_nodes, const float2 *aux, WalkRec *rec,
-                              int64_t entries, WalkSib *sib, float inv_theta) {
+                              float inv_theta) {
   const int threads = 256;
   k_prepare_s2<<<(unsigned)((n_nodes + threads - 1) / threads), threads, 0, s>>>(n_nodes, aux, rec,
                                                                                inv_theta);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_prepare_sib_s2(cudaStream_t s, int64_t entries, WalkSib *sib, float inv_theta) {
+  const int threads = 256;
   k_prepare_sib_s2<<<(unsigned)((entries + threads - 1) / threads), threads, 0, s>>>(entries, sib,
                                                                                    inv_theta);
   return cudaGetLastError();
