@@ -452,10 +452,11 @@ __device__ __forceinline__ void walk_octant(unsigned u, int lane, WalkMem<QUAD> 
   // list positions (written ever per sub-brick, evaluated ever); opened bottom nodes
   int depth = 1, nbot = 0;
   const int pop4 = stack_pop4(A.flev[F.w]);
+  const unsigned tops = (unsigned)A.sib.tops;
   unsigned staged = 0u, oldest = 0u, head = 0u, tail[4] = {0u, 0u, 0u, 0u};
   while (depth > 0) {
     const Tested t = front_step<VOTE>(
-        S.front, depth, pop4, lane, A.sib.sib, [&](const float4 &a, float s2, uint32_t *m) {
+        S.front, depth, pop4, tops, lane, A.sib.sib, [&](const float4 &a, float s2, uint32_t *m) {
           if (SPLIT == 1) {
             test64<false>(S.front, a.x, a.y, a.z, s2, m);
             return;

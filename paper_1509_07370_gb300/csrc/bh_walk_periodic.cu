@@ -120,8 +120,9 @@ __device__ __forceinline__ void walk_octant_periodic(
 
   int depth = 1, staged = 0, nbot = 0;
   const int pop4 = stack_pop4(flev[F.w]);
+  const unsigned tops = (unsigned)sib.tops;
   while (depth > 0) {
-    const Tested t = front_step<false, true>(S.front, depth, pop4, lane, sib.sib);
+    const Tested t = front_step<false, true>(S.front, depth, pop4, tops, lane, sib.sib);
     const bool accepted = (t.alo | t.ahi) != 0u;
     const unsigned acc = __ballot_sync(kFull, accepted);
     if (accepted) {

@@ -137,3 +137,26 @@ def test_sums_of_a_cell_that_holds_the_mass_stay_compensated(level, extra, quad)
         assert abs(phi[1] / phi[0] - 1.0) <= 2.0 ** -22
         same += phi[0] == phi[1]
     assert same >= 30
+
+
+@pytest.mark.parametrize("depth", [16, 17, 18])
+@pytest.mark.parametrize("theta", [0.35, 0.8])
+def test_deepest_meshes_match_the_oracle(depth, theta):
+    """Blocks down to levels 16 to 18 about opposite corners of the box, where the
+    stack has little or no room for four nodes of any kind: sampled cells of
+    every level."""
+    m = mg.refined_mesh(1, depth, lambda lev, ijk: np.all(ijk == 0, axis=1) |
+                        np.all(ijk == (1 << lev) - 1, axis=1))
+    rng = np.random.Generator(np.random.PCG64(depth))
+    rho = rng.lognormal(0.0, 1.5, size=(m.nblocks, 8, 8, 8)).astype(np.float32)
+    tg = 512 * np.arange(m.nblocks) + rng.integers(0, 512, m.nblocks)
+    t = O.Tree(m.level, m.ijk, rho.astype(np.float64))
+    for quad in (False, True):
+        want, wi, wt = t.walk(theta, targets=tg, quad=quad)
+        for prec, bar in ((B.BH_PREC_F32, 1e-5), (B.BH_PREC_F64, 1e-12)):
+            s = B.Solver(precision=prec, quadrupole=quad)
+            s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+            got = s.potential(theta).cpu().numpy().astype(np.float64)[tg]
+            ni, nt = (x.cpu().numpy()[tg] for x in s.walk_counts(theta))
+            assert np.array_equal(ni, wi) and np.array_equal(nt, wt)
+            assert np.max(np.abs(got / want - 1.0)) <= bar
