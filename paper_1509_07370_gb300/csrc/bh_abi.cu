@@ -412,7 +412,7 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
     BH_CUDA(bhg::launch_small_geometry(s, nb, t.d_key[0], t.d_idx[0], t.d_level, t.d_ijk,
                                        t.d_count, t.d_prestart, t.d_blk, t.d_orig, t.d_pos,
                                        n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa,
-                                       max_level, top));
+                                       top));
   } else {
     BH_CUDA(bhg::launch_sort_blocks(s, nb, t.d_key, t.d_idx, t.d_flags, fa));
     BH_CUDA(bhg::launch_tile_and_count(s, nb, t.d_key, t.d_idx, t.d_level, t.d_ijk, t.d_count,
@@ -448,7 +448,7 @@ bh_status build_fields(bh_ctx *ctx, int nfields, const int32_t *nblocks, const i
   if (!small)
     BH_CUDA(bhg::launch_top_nodes(ctx->side, nb, t.d_key[0], t.d_blk, t.d_count, t.d_prestart,
                                   n_nodes, t.d_rec, t.d_aux, t.d_lvl, t.d_flags, fa, t.d_orig,
-                                  max_level, top));
+                                  top));
   // Every check of the input is done by now (levels, coordinates and density
   // in k_keys_mass, the tiling in k_tile_and_count, the top-node count in
   // k_prestart_scan, top indexes in k_top_nodes/k_top_children): the flags go

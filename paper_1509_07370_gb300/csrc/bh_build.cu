@@ -246,8 +246,8 @@ __device__ __forceinline__ void tile_and_count(int p, const unsigned long long *
   orig[p] = b;
 }
 
-__global__ void k_tile_and_count(int nb, unsigned long long *key, int *idx,
-                                 const int *__restrict__ level,
+__global__ void k_tile_and_count(int nb, unsigned long long *__restrict__ key,
+                                 int *__restrict__ idx, const int *__restrict__ level,
                                  const int *__restrict__ ijk, int *__restrict__ count,
                                  int4 *__restrict__ blk, int *__restrict__ orig,
                                  unsigned *flags, const int *__restrict__ fstart,
@@ -397,49 +397,57 @@ __device__ __forceinline__ void top_nodes_of(int p, int nb, const unsigned long 
   }
 }
 
-__global__ void k_top_nodes(int nb, const unsigned long long *key, const int4 *blk,
-                            const int *count, const int *prestart, int64_t n_nodes, WalkRec *rec,
-                            float2 *aux, uint8_t *lvl, unsigned *flags, const int *fstart,
-                            const int *fid, const int *orig, int4 *fld, TopArgs top) {
+__global__ void k_top_nodes(int nb, const unsigned long long *__restrict__ key,
+                            const int4 *__restrict__ blk, const int *__restrict__ count,
+                            const int *__restrict__ prestart, int64_t n_nodes,
+                            WalkRec *__restrict__ rec, float2 *__restrict__ aux,
+                            uint8_t *__restrict__ lvl, unsigned *flags,
+                            const int *__restrict__ fstart, const int *__restrict__ fid,
+                            const int *__restrict__ orig, int4 *__restrict__ fld, TopArgs top) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= nb) return;
   top_nodes_of(p, nb, key, blk, count, prestart, n_nodes, rec, aux, lvl, flags, fstart, fid, orig,
                fld, top);
 }
 
-// Child lists of the top nodes, for the moment pass: entry 8 slot + o holds
-// the pre-order index of child o of the top node with compact index
-// slot = prestart[p] - 585 p + r (the r-th top node that starts at block p,
-// level k = j0 + r; prestart[p] - 585 p counts the top nodes before p).
+// Child lists of the top nodes, for the moment pass: entry 8 s + o holds the
+// pre-order index of child o of the top node with slot s (its place among the
+// top nodes; k_top_nodes left its block p, its level k and its field there).
 // Child o's cube starts at key kp + o 8^(21-k-1), so its first block q is
 // found by one binary search, and the child is q's top node of level k + 1
 // or, if q is a block of level k + 1, q's root.  One thread per (top node,
 // octant), all independent: the moment pass then reads its children
 // directly instead of chasing skip pointers one after another.  Also records
 // each child's parent slot (TopArgs::parent, TopArgs::bparent), by which the
-// moment pass climbs the top tree.
-__device__ __forceinline__ void top_child(int p, int o, int r, const unsigned long long *key,
-                                          const int4 *blk, const int *count, const int *prestart,
-                                          int64_t n_nodes, const int *fstart, const int *fid,
-                                          const int *orig, const TopArgs &top, unsigned *flags) {
-  const int cnt = count[p];
-  if (r >= cnt) return;
-  const int lb = blk[p].x, k = lb - cnt + r;
-  const int fend = fstart[fid[orig[p]] + 1];
-  const int64_t slot = (int64_t)prestart[p] - (int64_t)kNodesPerBlock * p + r;
-  if (k < 0 || k >= kKeyLevels || slot < 0 || slot >= top.slots) {
+// moment pass climbs the top tree.  (By slots and not by blocks and levels:
+// only a seventh of the blocks start a top node, and few of those one of every
+// level.)
+__device__ __forceinline__ void top_child(int64_t s, int o, int nb, int nfields,
+                                          const unsigned long long *key, const int4 *blk,
+                                          const int *count, const int *prestart, int64_t n_nodes,
+                                          const int *fstart, const TopArgs &top, unsigned *flags) {
+  if (s >= top.slots) {
     atomicOr(flags, kErrIndex);
     return;
   }
+  const int4 a = top.slot[2 * s], b = top.slot[2 * s + 1];
+  const int p = b.w, k = b.y, f = b.z;
+  // (a failed geometry leaves slots of earlier trees or none)
+  if (p < 0 || p >= nb || k < 0 || k >= kKeyLevels || f < 0 || f >= nfields ||
+      (int64_t)a.x - (int64_t)kNodesPerBlock * p != s) {
+    atomicOr(flags, kErrIndex);
+    return;
+  }
+  const int fend = fstart[f + 1];
   const unsigned long long start = key[p] + (unsigned long long)o * key_span(k + 1);
   int q = p;
   if (o > 0) {
-    int a = p + 1, e = fend;
-    while (a < e) {
-      const int m = (a + e) >> 1;
-      if (key[m] < start) a = m + 1; else e = m;
+    int lo = p + 1, e = fend;
+    while (lo < e) {
+      const int m = (lo + e) >> 1;
+      if (key[m] < start) lo = m + 1; else e = m;
     }
-    q = a;
+    q = lo;
   }
   if (q >= fend || key[q] != start) {  // a complete tiling starts every cube with a block
     atomicOr(flags, kErrIndex);
@@ -453,41 +461,43 @@ __device__ __forceinline__ void top_child(int p, int o, int r, const unsigned lo
     atomicOr(flags, kErrIndex);
     return;
   }
-  top.child[8 * slot + o] = (int)idx;
+  top.child[8 * s + o] = (int)idx;
   if (k + 1 < lq) {  // a top node: its slot
     const int64_t cs = idx - (int64_t)kNodesPerBlock * q;
     if (cs < 0 || cs >= top.slots) {
       atomicOr(flags, kErrIndex);
       return;
     }
-    top.parent[cs] = (int)slot;
+    top.parent[cs] = (int)s;
   } else {  // block q's root
-    top.bparent[q] = (int)slot;
+    top.bparent[q] = (int)s;
   }
 }
 
-__global__ void k_top_children(int nb, const unsigned long long *key, const int4 *blk,
-                               const int *count, const int *prestart, int64_t n_nodes,
-                               const int *fstart, const int *fid, const int *orig, TopArgs top,
-                               unsigned *flags) {
+__global__ void k_top_children(int64_t tops, int nb, int nfields,
+                               const unsigned long long *__restrict__ key,
+                               const int4 *__restrict__ blk, const int *__restrict__ count,
+                               const int *__restrict__ prestart, int64_t n_nodes,
+                               const int *__restrict__ fstart, TopArgs top, unsigned *flags) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (tid >= (int64_t)nb * 8) return;
-  top_child((int)(tid >> 3), (int)(tid & 7), blockIdx.y, key, blk, count, prestart, n_nodes,
-            fstart, fid, orig, top, flags);
+  if (tid >= 8 * tops) return;
+  top_child(tid >> 3, (int)(tid & 7), nb, nfields, key, blk, count, prestart, n_nodes, fstart, top,
+            flags);
 }
 
 // The geometry of a small block list in one launch, one block per thread:
 // what k_sort_blocks, k_tile_and_count, k_prestart_scan, k_top_nodes and
 // k_top_children do in five (2-5 us each, all launch and memory latency).  The
 // sort, when it is needed, counts for every block how many come before it in
-// its field.  Measured, a whole build:
-// 15 blocks 83 -> 69 us, 64 blocks 88 -> 72 us.
+// its field.  Measured, a whole build (us, by the five launches and by one):
+// 15 blocks 89, 68; 239 blocks of 7 levels 111, 91; 463 of 11 levels 128, 114; 512
+// of one level 95, 85 -- up to the most that one CTA of a thread a block takes.
 constexpr int kSmallBlocks = 512;
 __global__ void __launch_bounds__(kSmallBlocks)
     k_small_geometry(int nb, unsigned long long *key, int *idx, const int *level, const int *ijk,
                      int *count, int *prestart, int4 *blk, int *orig, int *pos, int64_t n_nodes,
-                     WalkRec *rec, float2 *aux, uint8_t *lvl, unsigned *flags, const int *fstart,
-                     const int *fid, int4 *fld, int max_level, TopArgs top) {
+                     WalkRec *rec, float2 *aux, uint8_t *lvl, unsigned *flags, int nfields,
+                     const int *fstart, const int *fid, int4 *fld, TopArgs top) {
   __shared__ unsigned long long keys[kSmallBlocks];
   __shared__ int warp_sum[kSmallBlocks / 32];
   const int t = threadIdx.x, lane = t & 31;
@@ -531,9 +541,9 @@ __global__ void __launch_bounds__(kSmallBlocks)
     top_nodes_of(t, nb, key, blk, count, prestart, n_nodes, rec, aux, lvl, flags, fstart, fid, orig,
                  fld, top);
   __syncthreads();
-  for (int i = t; i < 8 * nb * max_level; i += kSmallBlocks)  // (top node, octant) pairs
-    top_child((i >> 3) % nb, i & 7, (i >> 3) / nb, key, blk, count, prestart, n_nodes, fstart, fid,
-              orig, top, flags);
+  const int tops = (int)(n_nodes - (int64_t)kNodesPerBlock * nb);
+  for (int i = t; i < 8 * tops; i += kSmallBlocks)  // (top node, octant) pairs
+    top_child(i >> 3, i & 7, nb, nfields, key, blk, count, prestart, n_nodes, fstart, top, flags);
 }
 
 // Moments of one internal node from its 8 children (Eq. 5), children in
@@ -1339,15 +1349,14 @@ cudaError_t launch_top_nodes(cudaStream_t s, int nb, const unsigned long long *k
                              const int4 *blk, const int *count, const int *prestart,
                              int64_t n_nodes, WalkRec *rec, float2 *aux, uint8_t *lvl,
                              unsigned *flags, const FieldArgs &fa, const int *orig,
-                             int max_level, const TopArgs &top) {
+                             const TopArgs &top) {
   k_top_nodes<<<grid_for(nb, 256), 256, 0, s>>>(nb, key, blk, count, prestart, n_nodes, rec,
                                                  aux, lvl, flags, fa.fstart, fa.fid, orig, fa.fld,
                                                  top);
-  if (max_level > 0) {  // a block starts at most max_level top nodes
-    const dim3 grid((unsigned)grid_for((int64_t)nb * 8, 256), (unsigned)max_level);
-    k_top_children<<<grid, 256, 0, s>>>(nb, key, blk, count, prestart, n_nodes, fa.fstart,
-                                         fa.fid, orig, top, flags);
-  }
+  const int64_t tops = n_nodes - (int64_t)kNodesPerBlock * nb;
+  if (tops > 0)
+    k_top_children<<<(unsigned)grid_for(8 * tops, 256), 256, 0, s>>>(
+        tops, nb, fa.nfields, key, blk, count, prestart, n_nodes, fa.fstart, top, flags);
   return cudaGetLastError();
 }
 
@@ -1357,10 +1366,10 @@ cudaError_t launch_small_geometry(cudaStream_t s, int nb, unsigned long long *ke
                                   const int *level, const int *ijk, int *count, int *prestart,
                                   int4 *blk, int *orig, int *pos, int64_t n_nodes, WalkRec *rec,
                                   float2 *aux, uint8_t *lvl, unsigned *flags, const FieldArgs &fa,
-                                  int max_level, const TopArgs &top) {
+                                  const TopArgs &top) {
   k_small_geometry<<<1, kSmallBlocks, 0, s>>>(nb, key, idx, level, ijk, count, prestart, blk, orig,
-                                              pos, n_nodes, rec, aux, lvl, flags, fa.fstart, fa.fid,
-                                              fa.fld, max_level, top);
+                                              pos, n_nodes, rec, aux, lvl, flags, fa.nfields,
+                                              fa.fstart, fa.fid, fa.fld, top);
   return cudaGetLastError();
 }
 

@@ -305,13 +305,12 @@ cudaError_t launch_tile_and_count(cudaStream_t s, int nb, unsigned long long *ke
                                   const TopArgs &top, int *pos);
 cudaError_t launch_prestart_scan(cudaStream_t s, int nb, const int *count, int *prestart,
                                  unsigned *flags);
-// Skip pointers of the top nodes and their lists (TopArgs); max_level = the
-// largest block level.
+// Skip pointers of the top nodes and their lists (TopArgs).
 cudaError_t launch_top_nodes(cudaStream_t s, int nb, const unsigned long long *key,
                              const int4 *blk, const int *count, const int *prestart,
                              int64_t n_nodes, WalkRec *rec, float2 *aux, uint8_t *lvl,
                              unsigned *flags, const FieldArgs &fa, const int *orig,
-                             int max_level, const TopArgs &top);
+                             const TopArgs &top);
 // The launches from launch_sort_blocks to launch_top_nodes as one, for lists
 // of at most 512 blocks (small_geometry): keys and indices of caller blocks in,
 // in sorted order out.
@@ -320,7 +319,7 @@ cudaError_t launch_small_geometry(cudaStream_t s, int nb, unsigned long long *ke
                                   const int *level, const int *ijk, int *count, int *prestart,
                                   int4 *blk, int *orig, int *pos, int64_t n_nodes, WalkRec *rec,
                                   float2 *aux, uint8_t *lvl, unsigned *flags, const FieldArgs &fa,
-                                  int max_level, const TopArgs &top);
+                                  const TopArgs &top);
 // Largest cell mass of every field alone (a new density on the same tree).
 // Negative or non-finite densities set kErrDensity in flags.
 cudaError_t launch_mass_max(cudaStream_t s, int nb, const int *level, const void *density,

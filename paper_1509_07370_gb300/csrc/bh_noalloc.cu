@@ -192,7 +192,7 @@ extern "C" bh_status bh_solve_noalloc(int nblocks, const int32_t *level, const i
                            density_is_fp64));
   NA_CUDA(launch_small_geometry(s, nb, d_key[0], d_idx[0], d_level, d_ijk, d_count, d_prestart,
                                 d_blk, d_orig, nullptr, n_nodes, d_rec, d_aux, d_lvl, d_flags, fa,
-                                max_level, top));
+                                top));
   NA_CUDA(launch_moments(s, nb, d_blk, d_orig, d_count, d_prestart, density,
                          density_is_fp64, fa, n_nodes, d_mom, d_rec, d_aux, d_lvl, nullptr, nullptr,
                          d_flags, top, sib));

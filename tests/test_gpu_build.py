@@ -111,3 +111,32 @@ def test_both_sorts_restore_the_morton_order(split):
         trees.append(s.export_nodes())
     for k in ("level", "M", "R"):
         assert torch.equal(trees[0][k], trees[1][k]), k
+
+
+@pytest.mark.parametrize("extra", [1, 10, 11, 18])
+@pytest.mark.parametrize("shuffled", [False, True])
+def test_children_of_top_nodes_in_deep_trees(extra, shuffled):
+    """Top nodes of every level at one corner (8, 463 blocks: the geometry in
+    one launch; 519 and 911: in several), alone and as the last of a batch
+    behind single blocks and a shallow tree, whose slots come first: the
+    oracle's tree and masses, which the child lists carry upwards."""
+    m = corner(0, extra)
+    rng = np.random.Generator(np.random.PCG64(extra))
+    fs = [(corner(l, e), None) for l, e in ((0, 0), (1, 1), (0, 0))] + [(m, None)]
+    fs = [(x, rng.lognormal(size=(x.nblocks, 8, 8, 8)).astype(np.float32)) for x, _ in fs]
+    if shuffled:
+        fs = [mg.shuffled(x, r, i) for i, (x, r) in enumerate(fs)]
+    s = B.Solver()
+    for batch in ([fs[-1]], fs):
+        s.build_batch([x.nblocks for x, _ in batch], np.concatenate([x.level for x, _ in batch]),
+                      np.concatenate([x.ijk for x, _ in batch]),
+                      torch.as_tensor(np.concatenate([r.reshape(-1) for _, r in batch])).cuda())
+        e = {k: v.cpu().numpy() for k, v in s.export_nodes().items()}
+        at = 0
+        for x, rho in batch:
+            t = O.Tree(x.level, x.ijk, rho.astype(np.float64)).export()
+            n = t["M"].size
+            for k in ("level", "M", "R"):
+                assert np.array_equal(e[k][at:at + n], t[k]), k
+            at += n
+        assert at == e["M"].size
