@@ -80,7 +80,8 @@ typedef struct {
                      next term of the multipole expansion; the opening test is
                      unchanged).  Quadrupoles are reduced in binary32 for the
                      binary32 walk and in FP64 for the FP64 walk; they cost 32
-                     (binary32) or 80 (FP64) more bytes per internal node. */
+                     (binary32) or 80 (FP64) more bytes per node and 32 or 48
+                     per internal node. */
   int learned;    /* 0 (default).  1: every accepted node's term M/d is
                      multiplied by (1 + s^2 y), y = MLP(pair features), with the
                      network set by bh_set_mlp and evaluated on the tensor

@@ -101,7 +101,7 @@ void free_nodes(bhg::Tree &t) {
   release(t.d_smom);
   release(t.d_sq64);
   release(t.d_cmass64);
-  t.sib_cap = 0;
+  t.sib_cap = t.cell_cap = 0;
   release(t.d_q64);
   release(t.d_qrec);
   t.quad_cap = 0;
@@ -157,6 +157,7 @@ bh_status ensure_nodes(bh_ctx *ctx, int64_t n_nodes, int64_t nb) {
     BH_CUDA(bhg::dev_malloc(&t.d_cmass64, (size_t)nb * bhg::kCellsPerBlock * sizeof(double)));
   }
   t.sib_cap = entries;
+  t.cell_cap = nb;
   return BH_OK;
 }
 
@@ -1183,7 +1184,7 @@ bh_status bh_stats(const bh_ctx *ctx, bh_stats_t *out) {
   b += t.node_cap * (int64_t)(sizeof(double4_32a) + sizeof(bhg::WalkRec) + sizeof(float2) + 1);
   b += t.sib_cap * (int64_t)(sizeof(bhg::WalkSib) + (t.d_squad ? sizeof(bhg::WalkQuad) : 0) +
                             (t.d_smom ? sizeof(double4_32a) : 0) + (t.d_sq64 ? 48 : 0));
-  b += t.sib_cap / bhg::kSibsPerBlock * bhg::kCellsPerBlock *
+  b += t.cell_cap * bhg::kCellsPerBlock *
        (int64_t)(sizeof(float) + (t.d_cmass64 ? sizeof(double) : 0));
   b += t.quad_cap * (int64_t)sizeof(bhg::WalkQuad) + (t.d_q64 ? t.quad_cap * 48 : 0);
   b += t.nf_cap * (int64_t)(2 * sizeof(int) + 2 * sizeof(double)) + (t.nf_cap ? 4 : 0);

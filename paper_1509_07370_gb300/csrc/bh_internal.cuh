@@ -232,7 +232,7 @@ struct Tree {
   float *d_cmass = nullptr;
   double4_32a *d_smom = nullptr;  // binary64 walk
   double *d_sq64 = nullptr, *d_cmass64 = nullptr;
-  int64_t sib_cap = 0;
+  int64_t sib_cap = 0, cell_cap = 0;  // entries; blocks of d_cmass and d_cmass64
   double *d_q64 = nullptr;      // 6 per node, FP64 quadrupoles (quadrupole option)
   WalkQuad *d_qrec = nullptr;   // binary32 quadrupole walk records
   int64_t quad_cap = 0;

@@ -140,3 +140,17 @@ def test_children_of_top_nodes_in_deep_trees(extra, shuffled):
                 assert np.array_equal(e[k][at:at + n], t[k]), k
             at += n
         assert at == e["M"].size
+
+
+def test_device_bytes_of_the_binary64_arrays():
+    """What a binary64 context holds more than a binary32 one of the same tree:
+    a 32-byte moment for every place in sibling order (72 a block, 8 for each of
+    nb // 7 + 1 top nodes) and 8 bytes a cell."""
+    for m in (corner(0, 0), corner(2, 2), corner(4, 0)):
+        nb, held = m.nblocks, []
+        rho = torch.ones(512 * nb, device="cuda")
+        for prec in (B.BH_PREC_F32, B.BH_PREC_F64):
+            s = B.Solver(precision=prec)
+            s.build(m.level, m.ijk, rho)
+            held.append(s.stats()["device_bytes"])
+        assert held[1] - held[0] == 32 * (72 * nb + 8 * (nb // 7 + 1)) + 8 * 512 * nb
