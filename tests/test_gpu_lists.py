@@ -160,3 +160,82 @@ def test_deepest_meshes_match_the_oracle(depth, theta):
             ni, nt = (x.cpu().numpy()[tg] for x in s.walk_counts(theta))
             assert np.array_equal(ni, wi) and np.array_equal(nt, wt)
             assert np.max(np.abs(got / want - 1.0)) <= bar
+
+
+@pytest.mark.parametrize("level,extra,theta", CASES)
+@pytest.mark.parametrize("vote", [False, True])
+def test_binary64_walk_matches_oracle(level, extra, theta, vote):
+    """Terms within 2 2^-53 each and plain sums of runs of up to some 600 terms:
+    an rms error of about 2^-53 (2 + sqrt(600) / 2), 1.6e-15, and 1e-14 is six
+    times that (the oracle's own sums are compensated)."""
+    m, rho = field(level, extra, 10 * level + extra)
+    t = O.Tree(m.level, m.ijk, rho.astype(np.float64))
+    for quad in (False, True):
+        s = B.Solver(precision=B.BH_PREC_F64, quadrupole=quad,
+                     criterion=B.BH_CRIT_WARP_VOTE if vote else B.BH_CRIT_PER_CELL)
+        s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+        got = s.potential(theta).cpu().numpy()
+        if vote:
+            got = got.reshape(-1, 512)[:, O.local_morton_order()].reshape(-1)
+        want = (t.walk_vote if vote else t.walk)(theta, quad=quad)[0]
+        assert np.max(np.abs(got / want - 1.0)) <= 1e-14
+
+
+@pytest.mark.parametrize("quad", [False, True])
+def test_binary64_fields_keep_their_bits_in_a_batch(quad):
+    fs = [field(1, 14, 1), field(0, 0, 2), field(1, 1, 3), field(0, 5, 4)]
+    s = B.Solver(precision=B.BH_PREC_F64, quadrupole=quad)
+    s.build_batch([m.nblocks for m, _ in fs], np.concatenate([m.level for m, _ in fs]),
+                  np.concatenate([m.ijk for m, _ in fs]),
+                  torch.as_tensor(np.concatenate([r.reshape(-1) for _, r in fs])).cuda())
+    got = s.potential(0.6).cpu().numpy()
+    at = 0
+    for m, r in fs:
+        a = B.Solver(precision=B.BH_PREC_F64, quadrupole=quad)
+        a.build(m.level, m.ijk, torch.as_tensor(r.reshape(-1)).cuda())
+        want = a.potential(0.6).cpu().numpy()
+        assert np.array_equal(got[at:at + want.size], want)
+        at += want.size
+
+
+@pytest.mark.parametrize("heavy", [0, -1])
+def test_binary64_reciprocal_distance(heavy):
+    """All mass in one cell, a power of two at an exact centre: each potential is
+    one 1/sqrt of an exact d2 (180,000 cells of 9 levels).  The approximation's
+    relative error of 2^-20 makes e = 1 - d2 y y at most 2^-19, so the third-order
+    step leaves 5/16 e^3, 2^-58.7; rounding d2 y costs half of 2^-53, the last
+    operation 2^-53: 1.6 2^-53 in all."""
+    m, rho = field(0, 8, 0)
+    rho[:] = 0.0
+    rho[heavy, 3, 5, 2] = 1.0
+    s = B.Solver(precision=B.BH_PREC_F64)
+    s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+    got = s.potential(0.5).cpu().numpy().reshape(m.nblocks, 8, 8, 8)
+    h = 2.0 ** -(m.level.astype(np.float64) + 3)
+    c = [((8 * m.ijk[:, d, None] + np.arange(8)) + 0.5) * h[:, None] for d in range(3)]  # [b][i]
+    at = c[0][heavy, 2], c[1][heavy, 5], c[2][heavy, 3]
+    d2 = (((c[2] - at[2]) ** 2)[:, :, None, None] + ((c[1] - at[1]) ** 2)[:, None, :, None] +
+          ((c[0] - at[0]) ** 2)[:, None, None, :])  # exact: 23-bit differences
+    mine = d2 == 0.0
+    assert mine.sum() == 1 and got[mine][0] == 0.0
+    want = -np.longdouble(h[heavy] ** 3) / np.sqrt(np.longdouble(d2[~mine]))
+    assert np.abs(got[~mine] / want - 1).max() <= 1.6 * 2.0 ** -53
+
+
+@pytest.mark.parametrize("level,extra,theta", [(0, 0, 0.3), (0, 4, 0.25), (1, 2, 0.4), (2, 1, 1.0),
+                                               (1, 9, 0.6), (0, 18, 0.9)])
+def test_periodic_walk_matches_oracle(level, extra, theta):
+    """Counts exactly; potentials by the bar of the periodic tests (1e-5 of the
+    field's largest: they change sign).  Sampled cells of every block."""
+    m, rho = field(level, extra, 10 * level + extra)
+    t = O.Tree(m.level, m.ijk, rho.astype(np.float64))
+    tg = (512 * np.arange(m.nblocks)[:, None] +
+          np.random.default_rng(extra).integers(0, 512, (m.nblocks, 4))).reshape(-1)
+    want, wi, wt = t.walk_periodic(theta, targets=tg)
+    for kahan in (True, False):
+        s = B.Solver(periodic=True, kahan=kahan)
+        s.build(m.level, m.ijk, torch.as_tensor(rho.reshape(-1)).cuda())
+        got = s.potential(theta).cpu().numpy().astype(np.float64)
+        ni, nt = (x.cpu().numpy()[tg] for x in s.walk_counts(theta))
+        assert np.array_equal(ni, wi) and np.array_equal(nt, wt)
+        assert np.max(np.abs(got[tg] - want)) <= 1e-5 * np.abs(got).max()
