@@ -185,9 +185,13 @@ cudaError_t launch_mlp_tc(cudaStream_t s, int64_t n, const float *x, const MlpTc
                           unsigned *flags, int probe_limit) {
   const int smem = kTcSmem;
   const int64_t ntiles = (n + kTcRows - 1) / kTcRows;
-  const int64_t most = kTcCtasPerSm * 152;
+  if (ntiles <= 0) return cudaSuccess;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int64_t most = (int64_t)kTcCtasPerSm * sms;
   const int grid = (int)(ntiles < most ? ntiles : most);
-  if (grid <= 0) return cudaSuccess;
   k_mlp_tc<<<grid, kTcThreads, smem, s>>>(n, x, w, y, flags, probe_limit);
   return cudaGetLastError();
 }
