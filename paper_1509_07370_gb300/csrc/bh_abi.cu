@@ -536,7 +536,7 @@ static cudaError_t enqueue_walk(bh_ctx *ctx, cudaStream_t s, double G, void *out
                                 int32_t *n_int, int32_t *n_test, int32_t *n_leaf,
                                 bhg::WalkShape shape) {
   bhg::Tree &t = ctx->tree;
-  if (ctx->opt.periodic) {  // one pair per lane, a plain grid, optionally longest first
+  if (ctx->opt.periodic) {  // an octant a warp, a plain grid, optionally longest first
     const int64_t groups = (int64_t)t.nb * 8;
     const unsigned *order = shape.longest && t.order_n[0] == groups ? t.d_order[0] : nullptr;
     return bhg::launch_walk_periodic(s, ctx->opt, t.nb, t.d_rec, sib_args(t), t.d_blk, t.d_orig,
@@ -858,10 +858,10 @@ bh_status bh_export_quadrupoles(const bh_ctx *cctx, double *Q) {
   return BH_OK;
 }
 
-// The walk order of the groups for one and for two target pairs per lane,
+// The walk order of the groups of one and of two octants,
 // longest walk first: one walk of the tree at the prepared theta on the
 // persistent grid (4-warp CTAs, one group per take; the periodic walk: its
-// plain grid of 4-warp CTAs, one pair per lane) records the SM clock
+// plain grid of 4-warp CTAs, one octant) records the SM clock
 // cycles of each group's walk, under the load of a whole launch; the groups
 // are sorted by them on the host (stable, so equal times keep their Morton
 // order) and the order goes up.  The persistent walk then starts the long
@@ -929,7 +929,7 @@ bh_status bh_autotune(bh_ctx *ctx, double theta, int *shape) {
   bhg::Tree &t = ctx->tree;
   const bool tunable = ctx->opt.precision == BH_PREC_F32 &&
                        ctx->opt.criterion == BH_CRIT_PER_CELL && !ctx->opt.learned;
-  // the periodic walk has one target pair per lane and a plain grid: its CTA
+  // the periodic walk takes one octant a warp on a plain grid: its CTA
   // width and the octants' order are tuned
   const int npairs = ctx->opt.periodic ? 1 : 2;
   if (tunable) {
@@ -1017,7 +1017,7 @@ bh_status bh_set_walk_shape(bh_ctx *ctx, int warps_per_cta, int pairs_per_lane,
     return fail(ctx, BH_ERR_ARG,
                 "bh_set_walk_shape: warps 0..16, pairs 0..2, groups 0..64, longest_first 0/1");
   if (ctx->opt.periodic && (pairs_per_lane > 1 || groups_per_take > 0))
-    return fail(ctx, BH_ERR_ARG, "bh_set_walk_shape: the periodic walk has one pair per lane "
+    return fail(ctx, BH_ERR_ARG, "bh_set_walk_shape: the periodic walk has one octant per warp "
                                  "and a plain grid");
   const int np = pairs_per_lane > 0 ? pairs_per_lane : 1;
   if (longest_first && ctx->tree.order_n[np - 1] == 0)

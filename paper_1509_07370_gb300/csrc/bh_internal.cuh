@@ -215,7 +215,7 @@ struct Tree {
   double graph_theta = 0.0, graph_G = 0.0;
   WalkShape shape;              // launch shape of the walk (warps 0: not tuned)
   // walk order of the groups made by bh_autotune, longest walk first, for one
-  // (np = 1) or two (np = 2) target pairs per lane: d_order[np - 1] holds
+  // (np = 1) or two (np = 2) octants a group: d_order[np - 1] holds
   // order_n[np - 1] group indices (0 = none); used while the tree has that
   // many groups
   unsigned *d_order[2] = {nullptr, nullptr};
@@ -333,7 +333,7 @@ cudaError_t launch_moments(cudaStream_t s, int nb, const int4 *blk, const int *o
                            int64_t n_nodes, double4_32a *mom, WalkRec *rec, float2 *aux,
                            uint8_t *lvl, double *q64, WalkQuad *qrec, unsigned *flags,
                            const TopArgs &top, const SibArgs &sib,
-                        cudaEvent_t before_upper = nullptr);
+                           cudaEvent_t before_upper = nullptr);
 // Raises the dynamic shared-memory limit of the learned walk (more than 48 KB)
 // on the current device; called once per context, outside any graph capture.
 cudaError_t prepare_learned_kernels();
@@ -346,7 +346,7 @@ cudaError_t launch_prepare_sib_s2(cudaStream_t s, int64_t entries, WalkSib *sib,
 // out: float* (F32) or double* (F64); counts: optional per-cell n_int/n_test.
 // Potential scale of field f: -G * invL[f] (times the field's mass unit for
 // the binary32 walk).  shape = the launch shape of the per-cell binary32
-// walk (warps per CTA, target pairs per lane; 0 = defaults), tunable.
+// walk (WalkShape), tunable.
 cudaError_t launch_walk(cudaStream_t s, const bh_options &opt, int nb, const WalkRec *rec,
                         const SibArgs &sib, const int4 *blk, const int *orig, const FieldArgs &fa,
                         double G, void *out, int32_t *n_int, int32_t *n_test,
