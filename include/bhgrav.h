@@ -72,7 +72,10 @@ typedef struct {
   int precision;  /* BH_PREC_F32 (default): binary32 interaction arithmetic;
                      BH_PREC_F64: binary64 interaction arithmetic */
   int criterion;  /* BH_CRIT_PER_CELL (default) or BH_CRIT_WARP_VOTE */
-  int kahan;      /* F32 only: 1 (default) compensated (Kahan) summation, 0 plain */
+  int kahan;      /* F32 only: 1 (default) compensated (Kahan) summation, 0 plain.
+                     Compensated is every accepted node's term, its product
+                     unrounded; the cells of an opened bottom node join in plain
+                     sums of four (periodic: every term) */
   int quadrupole; /* 0 (default): monopole nodes, as in the paper.  1: every
                      accepted node also adds its quadrupole term,
                      -G (1/2) d^T Q d / |d|^5 with Q = sum m (3 x x^T - |x|^2 I)
@@ -129,6 +132,8 @@ bh_status bh_create(bh_ctx **out, const bh_options *opt, int device, void *cuda_
  *                    = 0) or double (1); every value finite and >= 0.  Cell
  *                    mass is density * cell volume.  Read on the stream until
  *                    the build's last kernel, which may run after the return.
+ * Device memory: 47 KB a block of 512 cells (binary32), 54 KB (BH_PREC_F64);
+ * with quadrupoles 68 and 104 KB; learned 66 KB.
  * Errors: BH_ERR_ARG, BH_ERR_GEOMETRY (nothing usable is kept: a later
  * bh_potential returns BH_ERR_STATE), BH_ERR_OOM, BH_ERR_CUDA. */
 bh_status bh_build(bh_ctx *ctx, int nblocks, const int32_t *level, const int32_t *ijk,

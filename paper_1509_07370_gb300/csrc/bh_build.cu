@@ -788,12 +788,14 @@ __device__ __forceinline__ void store_quad(int64_t id, const double Q[6], double
 
 constexpr int kBlockThreads = 128;
 
-// Bound by the FP64 pipe (2 operations a clock and SM) and the latency of its
-// chains: the exact forms take 3 of a cell's 7 operations off the sums
-// (accumulate_exact) and the conversions and the product off its mass
-// (exponent arithmetic), and five CTAs an SM instead of four hide more of the
-// chains.  A whole build of 3,984 blocks 209 -> 187 us (205 without the fifth
-// CTA), of 31,816 blocks 1034 -> 850 us.
+// Bound by latency: 20 warps an SM wait for the density and the block's records
+// (the largest stall, 12 cycles per issue; issue slots 17 % used) and for the
+// FP64 pipe's chains (2 operations a clock and SM; 55 % busy); the 163 MB that
+// it moves for 3,984 blocks, in 73 us, are a third of the copy rate.  The exact
+// forms take 3 of a cell's 7 FP64 operations off the sums (accumulate_exact) and
+// the conversions and the product off its mass (exponent arithmetic), and five
+// CTAs an SM instead of four hide more of the waiting.  A whole build of 3,984
+// blocks 209 -> 187 us (205 without the fifth CTA), of 31,816 blocks 1034 -> 850.
 template <typename T>
 __global__ void __launch_bounds__(kBlockThreads, 5)
     k_blocks(int nb, const int4 *__restrict__ blk, const int *__restrict__ orig,
