@@ -736,8 +736,8 @@ def batched_arm(args):
                              "speedup": value / (n / (u_ms * 1e-3))}},
             "roofline": roofline, "clocks": clocks, "e2e": e2e, "cpu_baseline": cpu,
             # per graph launch: largest-mass pass, k_blocks, k_upper_tree (the
-            # rest of the blocks and the top tree), opening radii, walk
-            "gpu_launches": 5 * args.steps}
+            # rest of the blocks and the top tree), walk
+            "gpu_launches": 4 * args.steps}
     print(json.dumps(line), flush=True)
     for ps in solvers:
         ps.close()
@@ -973,7 +973,7 @@ def build_roofline(ncells, nnodes, quad, build_ms):
     gbs = traffic / (build_ms * 1e-3) / 1e9
     return {"bound": "hbm", "kernel": "bh_build (keys, topology, FP64 moments)",
             "algorithmic_bytes": traffic, "achieved": gbs, "peak": peak, "unit": "GB/s",
-            "frac": gbs / peak, "note": "limited by FP64 arithmetic, not by HBM"}
+            "frac": gbs / peak, "note": "limited by latency and FP64 arithmetic, not by HBM"}
 
 
 def max_over_ranks(value, device=None):
@@ -1092,8 +1092,8 @@ def main():
     _, nn, maxlev = solver.tree_size()
     # keys with the largest mass, sort, tiling, scan, top nodes, top-node
     # child lists, k_blocks, k_upper_tree (the rest of the blocks and the top
-    # tree), walk
-    launches_per_step = 9
+    # tree), walk; the five from the sort to the child lists are one up to 512 blocks
+    launches_per_step = 9 if w.mesh.nblocks > 512 else 5
 
     # the plain walk (monopole, per-cell) at the theta of equal accuracy
     plain = None
@@ -1217,7 +1217,7 @@ def main():
                          "frac_monopole_count": (FLOP_PER_INTERACTION * n_int
                                                  + FLOP_PER_TEST * n_test) / walk_s / peak,
                          "kahan_ops": ("3 per node interaction (the compensation of the "
-                                       "compensated sum; a bottom node's 8 cell terms are "
+                                       "compensated sum; a bottom node's cell terms are "
                                        "summed plainly and folded once, not counted)"),
                          "mufu_bound_ms": n_int / (16 * props.multi_processor_count
                                                    * sm_mhz * 1e6) * 1e3,
